@@ -1,0 +1,17 @@
+// The four-column J^T kernels.
+#include "fft_apply_kernel.cuh"
+
+namespace fftgb {
+
+template <>
+fft_status launch_batch<MODE_JT4>(fft_geom g, const ApplyParams& P, cudaStream_t st) {
+    return launch_batch_impl<MODE_JT4>(g, P, st);
+}
+template <>
+fft_status set_attr_mode<MODE_JT4>(size_t smem) {
+    fft_status rc = set_attr_dt<MODE_JT4, FFT_DT_STABLE, PHI_TABLE>(smem);
+    if (rc != FFT_OK) return rc;
+    return set_attr_dt<MODE_JT4, FFT_DT_STABLE, PHI_TRIG>(smem);
+}
+
+}  // namespace fftgb
