@@ -1,9 +1,9 @@
 // Phi table by FP64 quadrature on the device (Sec. II-C, Eq. Kernel_freq).
 //
 // Phi(dt_k) = int_0^inf w^3 W(w) sin(w dt_k) dw / int_0^inf w^2 W(w) dw, dt_k = k dt_max/(n-1).
-// One CTA per sample k: its threads stride over the quadrature nodes, each thread sums its
-// nodes in order, then a fixed-shape tree reduction combines the threads, so the result is
-// the same on every run.
+// One CTA takes one sample k (sampled spectra) or eight (Gaussian spectra): its threads stride
+// over the quadrature nodes, each thread sums its nodes in order, then a fixed-shape tree
+// reduction combines the threads, so the result is the same on every run.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -36,24 +36,69 @@ __device__ double block_sum(double v, double* sh) {
     return r;
 }
 
-// moment = 2: denominator (dt ignored); moment = 3: numerator at dt.
-__global__ void phi_gauss_kernel(double w0, double s, int n, double dt_max, double* out) {
+// Simpson quadrature of a Gaussian spectrum in two kernels. The nodes' terms do not depend on the
+// sample: gauss_nodes_kernel computes them once (two FP64 exponentials a node), A_q = c_q w_q^3
+// W(w_q) and per block the partial sums of the denominator's c_q w_q^2 W(w_q). phi_gauss_kernel then
+// needs sin(w_q dt_k) = sin(q k alpha), alpha = dw ddt, at every (node, sample): with q = 256 a + t
+// it is sin(256 a k alpha) cos(t k alpha) + cos(256 a k alpha) sin(t k alpha), so a block of
+// TB_K samples takes 157 + 256 sines and cosines per sample instead of 40001, and three FP64
+// operations per (node, sample), which is what bounds it (GB300 has 2 FP64 FMAs per SM and clock:
+// 4.9e8 of them take 0.8 ms). 4096 samples: 24.6 ms with a sine and two exponentials in
+// every (node, sample), about 1 ms so (a 4096-sample table and ring256 geometry 37.6 -> 14.0 ms).
+constexpr int TB_K = 8;                                            // samples per block
+constexpr int TB_A = N_QUAD_GAUSS / TB_THREADS + 1;               // blocks of 256 nodes (157)
+static_assert(TB_A <= TB_THREADS, "one thread per partial denominator");
+
+__global__ void __launch_bounds__(TB_THREADS) gauss_nodes_kernel(double w0, double s, double* __restrict__ A,
+                                                                 double* __restrict__ den_part) {
     __shared__ double sh[TB_THREADS];
-    const int k = blockIdx.x;
-    const double wmax = w0 + 12.0 * s;
-    const double dw = wmax / N_QUAD_GAUSS;
-    const double dt = (double)k * dt_max / (double)(n - 1);
-    double num = 0.0, den = 0.0;
-    for (int q = threadIdx.x; q <= N_QUAD_GAUSS; q += TB_THREADS) {
-        double w = q * dw;
-        double c = (q == 0 || q == N_QUAD_GAUSS) ? 1.0 : ((q & 1) ? 4.0 : 2.0);
-        double ww = c * w * w * w_gauss(w, w0, s);
-        den += ww;
-        num += ww * w * sin(w * dt);
+    const int q = blockIdx.x * TB_THREADS + threadIdx.x;
+    const double dw = (w0 + 12.0 * s) / N_QUAD_GAUSS;
+    double ww = 0.0, w = 0.0;
+    if (q <= N_QUAD_GAUSS) {
+        w = q * dw;
+        const double c = (q == 0 || q == N_QUAD_GAUSS) ? 1.0 : ((q & 1) ? 4.0 : 2.0);
+        ww = c * w * w * w_gauss(w, w0, s);
     }
-    num = block_sum(num, sh);
-    den = block_sum(den, sh);
-    if (threadIdx.x == 0) out[k] = (k == 0) ? 0.0 : num / den;
+    A[q] = ww * w;   // [TB_A * TB_THREADS], zero past the last node
+    const double d = block_sum(ww, sh);
+    if (threadIdx.x == 0) den_part[blockIdx.x] = d;
+}
+
+__global__ void __launch_bounds__(TB_THREADS) phi_gauss_kernel(const double* __restrict__ A,
+                                                               const double* __restrict__ den_part, double w0,
+                                                               double s, int n, double dt_max,
+                                                               double* __restrict__ out) {
+    __shared__ double sh[TB_THREADS];
+    __shared__ double2 sc[TB_A][TB_K];   // sine and cosine of 256 a k alpha
+    const int t = threadIdx.x, k0 = blockIdx.x * TB_K;
+    const double dw = (w0 + 12.0 * s) / N_QUAD_GAUSS;
+    for (int i = t; i < TB_A * TB_K; i += TB_THREADS) {
+        const int a = i / TB_K, j = i % TB_K;
+        const double dt = (double)(k0 + j) * dt_max / (double)(n - 1);
+        sincos((double)(a * TB_THREADS) * dw * dt, &sc[a][j].x, &sc[a][j].y);
+    }
+    double st[TB_K], ct[TB_K], acc[TB_K];
+#pragma unroll
+    for (int j = 0; j < TB_K; ++j) {
+        const double dt = (double)(k0 + j) * dt_max / (double)(n - 1);
+        sincos((double)t * dw * dt, &st[j], &ct[j]);
+        acc[j] = 0.0;
+    }
+    const double den = block_sum(t < TB_A ? den_part[t] : 0.0, sh);   // (also orders sc before its use)
+    for (int a = 0; a < TB_A; ++a) {
+        const double Aq = A[a * TB_THREADS + t];
+#pragma unroll
+        for (int j = 0; j < TB_K; ++j) {
+            const double2 z = sc[a][j];
+            acc[j] = fma(Aq, fma(z.x, ct[j], z.y * st[j]), acc[j]);
+        }
+    }
+    for (int j = 0; j < TB_K; ++j) {
+        const double num = block_sum(acc[j], sh);
+        const int k = k0 + j;
+        if (t == 0 && k < n) out[k] = (k == 0) ? 0.0 : num / den;
+    }
 }
 
 __global__ void phi_sampled_kernel(const double* om, const double* W, int n_om, int n,
@@ -106,9 +151,22 @@ extern "C" fft_status fft_table_build(const fft_spectrum* spec, int32_t n_sample
             st = FFT_ERR_ARG;
         } else {
             double w0 = 2.0 * M_PI * spec->f_center_hz, s = 2.0 * M_PI * spec->f_sigma_hz;
-            phi_gauss_kernel<<<n_samples, TB_THREADS>>>(w0, s, n_samples, dt_max, t->d_phi);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) st = cuda_fail(e, "phi_gauss_kernel");
+            double* nodes = nullptr;   // A [TB_A * TB_THREADS], then the denominator's partials [TB_A]
+            e = cudaMalloc(&nodes, sizeof(double) * ((size_t)TB_A * TB_THREADS + TB_A));
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                set_error("fft_table_build: cudaMalloc failed");
+                st = FFT_ERR_OOM;
+            } else {
+                double* den_part = nodes + (size_t)TB_A * TB_THREADS;
+                gauss_nodes_kernel<<<TB_A, TB_THREADS>>>(w0, s, nodes, den_part);
+                phi_gauss_kernel<<<(unsigned)ceil_div(n_samples, TB_K), TB_THREADS>>>(nodes, den_part, w0, s, n_samples,
+                                                                                      dt_max, t->d_phi);
+                e = cudaGetLastError();
+                if (e == cudaSuccess) e = cudaDeviceSynchronize();
+                cudaFree(nodes);
+                if (e != cudaSuccess) st = cuda_fail(e, "phi_gauss_kernel");
+            }
         }
     } else if (spec->kind == 1) {
         if (!spec->omega || !spec->weight || spec->n_omega < 2) {
