@@ -109,9 +109,11 @@ void fft_table_destroy(fft_table t);
  *   dw_out       nullable, host: receives dw (rad/s).
  *   n_terms_out  nullable, host: receives n.
  *   out          receives the handle; release with fft_table_destroy.
- * Geometries built from series handles evaluate Phi on the fly by the Clenshaw recurrence
- * (one sine and one cosine per evaluation, two FP32 operations per term) instead of the
- * table lookup. Synchronous; host-only arithmetic.
+ * Geometries built from series handles evaluate Phi from piecewise quadratics of the series
+ * (formed at geometry creation in FP64, within 5e-8 of max |Phi|, held in shared memory) or,
+ * where those do not fit (many bands cut after many periods), by the Clenshaw recurrence (one
+ * sine and one cosine per evaluation, two FP32 operations per term). Synchronous; host-only
+ * arithmetic.
  */
 fft_status fft_trig_build(const fft_spectrum* spec, double dt_max, int32_t n_terms, double* coef_out,
                           double* dw_out, int32_t* n_terms_out, fft_table* out);

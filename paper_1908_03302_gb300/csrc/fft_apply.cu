@@ -154,6 +154,7 @@ static ApplyParams make_params(fft_geom g) {
     P.dsum = nullptr;
     P.icount = nullptr;
     P.trig_nq = g->trig_nq;
+    P.seg_n = g->seg_n;
     P.nvox = g->V;
     P.nrow = g->M;
     return P;

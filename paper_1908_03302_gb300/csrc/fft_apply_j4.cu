@@ -11,7 +11,8 @@ template <>
 fft_status set_attr_mode<MODE_J4>(size_t smem) {
     fft_status rc = set_attr_dt<MODE_J4, FFT_DT_STABLE, PHI_TABLE>(smem);
     if (rc != FFT_OK) return rc;
-    return set_attr_dt<MODE_J4, FFT_DT_STABLE, PHI_TRIG>(smem);
+    if ((rc = set_attr_dt<MODE_J4, FFT_DT_STABLE, PHI_TRIG>(smem)) != FFT_OK) return rc;
+    return set_attr_dt<MODE_J4, FFT_DT_STABLE, PHI_SEG>(smem);
 }
 
 }  // namespace fftgb

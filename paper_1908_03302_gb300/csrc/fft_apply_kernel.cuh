@@ -66,15 +66,18 @@ struct ApplyParams {
     float* gpart;            // J^T partials of multi-item tiles
     double* dsum;            // FROB: one per unit [n_items * 4]
     unsigned long long* icount;   // COUNT
-    int trig_nq;             // sine-series Phi: coefficient groups of 4 per band
+    int trig_nq;             // PHI_TRIG: coefficient groups of 4 per band
+    int seg_n;               // PHI_SEG: segments per band
     int64_t nvox, nrow;      // column lengths of the batch modes' blocks (V, M)
 };
 
-// Phi of the normalised detour v from the band data at shared address tb (table lookup or
-// sine series, see fft_device.cuh).
+// Phi of the normalised detour v (table lookup, sine series or its piecewise quadratics, see
+// fft_device.cuh): tb is the band data's shared address (PHI_SEG: the bits of the band's magic
+// number, `tab` the shared address of all bands' segments and `seg2` that of their c2).
 template <int PHI>
-__device__ __forceinline__ float phi_eval(float v, uint32_t tb, float nm1, int nq) {
+__device__ __forceinline__ float phi_eval(float v, uint32_t tb, float nm1, int nq, uint32_t tab, uint32_t seg2) {
     if (PHI == PHI_TRIG) return phi_trig(v, tb, nq);
+    if (PHI == PHI_SEG) return phi_seg(v, __uint_as_float(tb), nm1, tab, seg2);
     return phi_lookup(v, tb, nm1);
 }
 
@@ -122,7 +125,7 @@ __device__ __forceinline__ float detour_v64(const RowRec64& r, double ox, double
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr int apply_min_blocks() {
     return (SHARP || MODE == MODE_JT4 || MODE == MODE_J4) ? 2
-                                                          : ((DT == FFT_DT_STABLE && PHI == PHI_TABLE) ? 4 : 3);
+                                                          : ((DT == FFT_DT_STABLE && PHI != PHI_TRIG) ? 4 : 3);
 }
 
 // Sub-bricks per unit and units (regions) per item of each mode: see sub_dy below.
@@ -183,7 +186,8 @@ __device__ __forceinline__ void sub_step(int s, float hx, float hy, float hz, fl
 template <int MODE, int DT, bool GUARD, int PHI, int NSUB>
 __device__ __noinline__ void sharp_fix(const ApplyParams& P, float4 A, float4 B, float4 C, float Xl, float Yl,
                                        float Zl, bool planar, uint32_t inner_bits, float cutb, uint32_t tb,
-                                       float nm1, int nq, int ix0, int iy0, int iz0, float* d) {
+                                       float nm1, int nq, uint32_t tab, uint32_t seg2, int ix0, int iy0, int iz0,
+                                       float* d) {
     const float hx = B.x, hy = B.y, hz = B.z;
     const float hl = 0.5f * (A.x - A.y);
     const int b = __float_as_int(C.w) & 0xff;
@@ -233,8 +237,8 @@ __device__ __noinline__ void sharp_fix(const ApplyParams& P, float4 A, float4 B,
             continue;
         }
         const float w = is * ir;
-        const float val1 = phi_eval<PHI>(v, tb, nm1, nq) * w;
-        const float val2 = phi_eval<PHI>(v2, tb, nm1, nq) * w;
+        const float val1 = phi_eval<PHI>(v, tb, nm1, nq, tab, seg2) * w;
+        const float val2 = phi_eval<PHI>(v2, tb, nm1, nq, tab, seg2) * w;
         if (MODE == MODE_COV) d[k] = fabsf(val2) - fabsf(val1);
         else if (MODE == MODE_FROB) d[k] = val2 * val2 - val1 * val1;
         else d[k] = val2 - val1;
@@ -249,7 +253,7 @@ __device__ __noinline__ void sharp_fix(const ApplyParams& P, float4 A, float4 B,
 // second cost more.
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr bool apply_sharp_wide() {
-    return SHARP && DT == FFT_DT_STABLE && PHI == PHI_TABLE && MODE != MODE_JT4 && MODE != MODE_J4;
+    return SHARP && DT == FFT_DT_STABLE && PHI != PHI_TRIG && MODE != MODE_JT4 && MODE != MODE_J4;
 }
 constexpr int SHARP_MAX_WARPS = 20;
 
@@ -259,7 +263,7 @@ constexpr int SHARP_MAX_WARPS = 20;
 // 64 registers: slices3d J^T 408.0 -> 407.6 ms, J 412.6 -> 411.4 ms, ring256 J^T 3.75 -> 3.72 ms.
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr bool apply_plain_wide() {
-    return !SHARP && DT == FFT_DT_STABLE && PHI == PHI_TABLE && MODE != MODE_JT4 && MODE != MODE_J4;
+    return !SHARP && DT == FFT_DT_STABLE && PHI != PHI_TRIG && MODE != MODE_JT4 && MODE != MODE_J4;
 }
 constexpr int PLAIN_MAX_WARPS = 24;
 
@@ -286,7 +290,9 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
     __syncthreads();   // the only CTA-wide barrier: from here on every warp runs on its own
 
     const uint32_t tab_addr = smem_addr(s_tab);
-    const float nm1 = (float)(P.n_tab - 1);
+    // table lookups scale v by n_tab - 1, segment lookups by seg_n 2^-22
+    const float nm1 = PHI == PHI_SEG ? (float)P.seg_n * MAGIC2_ULP : (float)(P.n_tab - 1);
+    const uint32_t seg2_addr = tab_addr + (uint32_t)(P.n_bands * (P.seg_n + SEG_PAD)) * 8u;
     const int nq = P.trig_nq;
     const int lx = lane & 1, ly = (lane >> 1) & 3, lz = lane >> 3;
     constexpr bool BATCH = (MODE == MODE_JT4 || MODE == MODE_J4);
@@ -404,7 +410,9 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     // sub-bricks whose voxels all satisfy |p| <= hl (between the transducer planes)
                     if (fabsf(fmaf(cx, ex, fmaf(cy, ey, cz * ez))) + pext <= hl) inb |= 1u << s;
                 }
-                const uint32_t tb = tab_addr + (uint32_t)(b * P.n_tab) * 8u - (PHI == PHI_TABLE ? MAGIC_BITS_X8 : 0u);
+                const uint32_t tb =
+                    PHI == PHI_SEG ? __float_as_uint(fmaf((float)(b * (P.seg_n + SEG_PAD)), MAGIC2_ULP, MAGIC2))
+                                   : tab_addr + (uint32_t)(b * P.n_tab) * 8u - (PHI == PHI_TABLE ? MAGIC_BITS_X8 : 0u);
                 stg[lane * SR + 0] = base;
                 stg[lane * SR + 1] = make_float4(hb * ex, hb * ey, hb * ez, base3);
                 if (MODE == MODE_JT4) stg[lane * SR + 3] = W4;
@@ -518,7 +526,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
             ww[t] = is * ir;                                                                       \
             continue;                                                                              \
         }                                                                                          \
-        const float val = phi_lookup(v, tb, nm1) * (is * ir);                                      \
+        const float val = phi_eval<PHI>(v, tb, nm1, nq, tab_addr, seg2_addr) * (is * ir);          \
         if (MODE == MODE_JT) acc[s][t] = fmaf(val, W, acc[s][t]);                                  \
         if (MODE == MODE_COV) acc[s][t] = fmaf(fabsf(val), W, acc[s][t]);                          \
         if (MODE == MODE_JT4) {                                                                    \
@@ -583,7 +591,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     }
                     if (near)
                         sharp_fix<MODE, DT, GUARD, PHI, NSUB>(P, A, B, C, Xl, Yl, Zl, planar, inner_bits, cutb, tb, nm1,
-                                                              nq, TX + oxi, TY + oyi, TZ + ozi, d);
+                                                              nq, tab_addr, seg2_addr, TX + oxi, TY + oyi, TZ + ozi, d);
 #pragma unroll
                     for (int s = 0; s < NSUB; ++s) {
 #pragma unroll
@@ -720,6 +728,7 @@ inline fft_status set_attr_mode_impl(size_t smem) {
     if ((rc = set_attr_dt<MODE, FFT_DT_STABLE, PHI_TABLE>(smem)) != FFT_OK) return rc;
     if ((rc = set_attr_dt<MODE, FFT_DT_NAIVE, PHI_TABLE>(smem)) != FFT_OK) return rc;
     if (MODE != MODE_COUNT && (rc = set_attr_dt<MODE, FFT_DT_STABLE, PHI_TRIG>(smem)) != FFT_OK) return rc;
+    if (MODE != MODE_COUNT && (rc = set_attr_dt<MODE, FFT_DT_STABLE, PHI_SEG>(smem)) != FFT_OK) return rc;
     return set_attr_one<MODE, FFT_DT_FP64, false, false, PHI_TABLE>(smem);
 }
 
@@ -770,15 +779,17 @@ template <int MODE>
 inline fft_status launch_mode_impl(fft_geom g, const ApplyParams& P, cudaStream_t st) {
     FFT_CUDA(cudaMemsetAsync(g->counter, 0, 2 * sizeof(int32_t), st));
     if (g->n_items == 0) return FFT_OK;
-    // MODE_COUNT evaluates no Phi: the table variant serves both representations
-    constexpr int PHI_T = MODE == MODE_COUNT ? PHI_TABLE : PHI_TRIG;
+    // MODE_COUNT evaluates no Phi: the table variant serves every representation
+    constexpr int PHI_T = MODE == MODE_COUNT ? PHI_TABLE : PHI_TRIG, PHI_S = MODE == MODE_COUNT ? PHI_TABLE : PHI_SEG;
 #define FFT_LAUNCH_GS(DTV, PV)                                      \
     do {                                                            \
         if (g->guard) launch_split<MODE, DTV, true, PV>(g, P, st);  \
         else launch_split<MODE, DTV, false, PV>(g, P, st);          \
     } while (0)
-    if (g->phi_kind == PHI_TRIG) {   // geometry creation guarantees dt_mode STABLE
+    if (g->phi_eval == PHI_TRIG) {   // geometry creation guarantees dt_mode STABLE for series
         FFT_LAUNCH_GS(FFT_DT_STABLE, PHI_T);
+    } else if (g->phi_eval == PHI_SEG) {
+        FFT_LAUNCH_GS(FFT_DT_STABLE, PHI_S);
     } else if (g->dt_mode == FFT_DT_STABLE) {
         FFT_LAUNCH_GS(FFT_DT_STABLE, PHI_TABLE);
     } else if (g->dt_mode == FFT_DT_NAIVE) {
@@ -809,8 +820,10 @@ inline fft_status launch_batch_impl(fft_geom g, const ApplyParams& P, cudaStream
             else FFT_LAUNCH(false, false, PV);                      \
         }                                                           \
     } while (0)
-    if (g->phi_kind == PHI_TRIG)
+    if (g->phi_eval == PHI_TRIG)
         FFT_LAUNCH_GS(PHI_TRIG);
+    else if (g->phi_eval == PHI_SEG)
+        FFT_LAUNCH_GS(PHI_SEG);
     else
         FFT_LAUNCH_GS(PHI_TABLE);
 #undef FFT_LAUNCH_GS

@@ -85,8 +85,10 @@ constexpr float CUT_BAND = 2e-6f;
 
 // Representation of Phi inside the kernels.
 enum { PHI_TABLE = 0,   // sampled table, linear interpolation (fft_table_build)
-       PHI_TRIG = 1 };  // sine series, Clenshaw recurrence (fft_trig_build)
+       PHI_TRIG = 1,    // sine series (fft_trig_build), Clenshaw recurrence
+       PHI_SEG = 2 };   // sine series, piecewise quadratics in shared memory
 constexpr int TRIG_MAX_TERMS = 256;
+constexpr int SEG_PAD = 4;   // entries per band past the segments: the cut-off (zeros) and padding
 
 // Work item: rows [e0, e1) of tile `tile`'s entry list; J^T writes to slot `slot` of the
 // partial buffer when the tile has several items, else (slot < 0) straight to g.
@@ -120,7 +122,9 @@ struct fft_geom_s {
     int32_t n_tab;
     int32_t dt_mode;
     int32_t phi_kind = 0;                // fftgb::PHI_TABLE or fftgb::PHI_TRIG (all bands alike)
-    int32_t trig_nq = 0;                 // series: coefficient groups of 4 per band (padded)
+    int32_t phi_eval = 0;                // how the kernels evaluate Phi: PHI_TABLE, PHI_TRIG or PHI_SEG
+    int32_t seg_n = 0;                   // PHI_SEG: segments per band (entries: seg_n + SEG_PAD)
+    int32_t trig_nq = 0;                 // PHI_TRIG: coefficient groups of 4 per band (padded)
     int32_t trig_terms = 0;              // series: the largest term count over the bands
     double psf_tc_mma_flops = 0.0;       // MMA flops of the last tensor-core fft_psf_batch call
     double psf_tc_entries = 0.0;         // J entries it generated

@@ -212,6 +212,54 @@ __global__ void pack_table_kernel(const double* __restrict__ phi, int n, float2*
     }
 }
 
+// Phi of a sine series at x = theta v (0 at and outside [0, 1)): Clenshaw's recurrence in FP64.
+double series_phi(const fft_table t, double v) {
+    if (!(v > 0.0) || v >= 1.0) return 0.0;
+    const double x = t->dw * t->dt_max * v, c2 = 2.0 * cos(x);
+    double b1 = 0.0, b2 = 0.0;
+    for (int j = t->n; j >= 1; --j) {
+        const double b0 = t->coef[j - 1] + c2 * b1 - b2;
+        b2 = b1;
+        b1 = b0;
+    }
+    return b1 * sin(x);
+}
+
+// Piecewise quadratics of the bands' series (device layout of PHI_SEG, see phi_seg): (c0, c1) of all
+// bands' entries, then their c2. The fewest segments (a power of two) whose quadratics stay
+// within 5e-8 of each band's max |Phi| (a third of a segment off its ends and middle, where the
+// cubic remainder peaks), i.e. inside the FP32 rounding of the values: 2048 for spectra of the usual
+// width cut after three periods. Returns 0 if they do not fit `max_bytes` of shared memory: such series
+// (many bands, or cut after tens of periods) keep the recurrence.
+int build_segments(const fft_table* tables, int n_bands, size_t max_bytes, std::vector<float2>& packed) {
+    for (int n = 512; (size_t)n_bands * (n + SEG_PAD) * 12 <= max_bytes; n *= 2) {
+        const int ne = n + SEG_PAD;
+        packed.assign((size_t)n_bands * ne * 3 / 2, make_float2(0.0f, 0.0f));
+        float* c2 = reinterpret_cast<float*>(packed.data() + (size_t)n_bands * ne);
+        bool good = true;
+        for (int b = 0; b < n_bands && good; ++b) {
+            const fft_table t = tables[b];
+            // the series just below the cut-off, not the truncated 0 there, ends the last segment
+            const double end = 1.0 - 1e-12;
+            double mx = 0.0, err = 0.0, f2 = series_phi(t, 0.0);
+            for (int k = 0; k < n; ++k) {
+                const double f0 = f2, f1 = series_phi(t, (k + 0.5) / n);
+                f2 = series_phi(t, k + 1 < n ? (k + 1.0) / n : end);
+                const double a1 = -3.0 * f0 + 4.0 * f1 - f2, a2 = 2.0 * f0 - 4.0 * f1 + 2.0 * f2;
+                mx = fmax(mx, fmax(fabs(f0), fabs(f1)));
+                for (double u : {0.21, 0.79})
+                    err = fmax(err, fabs(f0 + u * (a1 + u * a2) - series_phi(t, (k + u) / n)));
+                const double s = 4194304.0;   // u is kept times 2^-22
+                packed[(size_t)b * ne + k] = make_float2((float)f0, (float)(a1 * s));
+                c2[(size_t)b * ne + k] = (float)(a2 * s * s);
+            }
+            good = err <= 5e-8 * mx;
+        }
+        if (good) return n;
+    }
+    return 0;
+}
+
 template <typename T>
 fft_status dmalloc(fft_geom g, T** p, size_t count) {
     *p = nullptr;
@@ -368,7 +416,7 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
     int32_t trig_terms = 0;
     for (int b = 0; b < n_tables; ++b) trig_terms = std::max(trig_terms, tables[b]->n);
     const int32_t trig_nq = (trig_terms + 3) / 4;
-    const int32_t n_tab = phi_kind == PHI_TABLE ? tables[0]->n : 2 + 2 * trig_nq;
+    int32_t n_tab = phi_kind == PHI_TABLE ? tables[0]->n : 2 + 2 * trig_nq;
     const int64_t V = (int64_t)grid->nx * grid->ny * grid->nz;
     FFT_ARG(V < ((int64_t)1 << 40), "fft_geom_create: grid too large");
     for (int64_t p = 0; p < n_rows; ++p) {
@@ -378,9 +426,19 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
         if (band_of_row)
             FFT_ARG(band_of_row[p] >= 0 && band_of_row[p] < n_tables, "fft_geom_create: band index out of range");
     }
+    int32_t phi_eval = phi_kind, seg_n = 0;
+    std::vector<float2> segments;
     {
         int optin = 0;
         FFT_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        if (phi_kind == PHI_TRIG) {   // piecewise quadratics where they leave room for 16 warps' staging
+            const size_t stage = (size_t)2 * APPLY_WARPS * 128 * sizeof(float4);
+            if ((size_t)optin > stage) seg_n = build_segments(tables, n_tables, (size_t)optin - stage, segments);
+            if (seg_n > 0) {
+                phi_eval = PHI_SEG;
+                n_tab = (seg_n + SEG_PAD) / 2 * 3;   // float2 words per band
+            }
+        }
         size_t need = (((size_t)n_tables * n_tab * sizeof(float2) + 15) & ~(size_t)15) +
                       (size_t)APPLY_WARPS * 128 * sizeof(float4);
         if (need > (size_t)optin) {
@@ -399,7 +457,9 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
     g->n_tab = n_tab;
     g->dt_mode = dt_mode;
     g->phi_kind = phi_kind;
-    g->trig_nq = phi_kind == PHI_TRIG ? trig_nq : 0;
+    g->phi_eval = phi_eval;
+    g->seg_n = seg_n;
+    g->trig_nq = phi_eval == PHI_TRIG ? trig_nq : 0;
     g->trig_terms = phi_kind == PHI_TRIG ? trig_terms : 0;
     g->guard = false;
     fft_status rc = FFT_OK;
@@ -441,12 +501,8 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
             }
         } else {   // the series on 4096 points of [0, dt_max]
             phi.resize(4096);
-            for (size_t k = 0; k < phi.size(); ++k) {
-                const double dt = tables[b]->dt_max * (double)k / (double)(phi.size() - 1);
-                double acc = 0.0;
-                for (int j = 1; j <= tables[b]->n; ++j) acc += tables[b]->coef[j - 1] * sin(j * tables[b]->dw * dt);
-                phi[k] = acc;
-            }
+            for (size_t k = 0; k + 1 < phi.size(); ++k) phi[k] = series_phi(tables[b], (double)k / (double)(phi.size() - 1));
+            phi.back() = series_phi(tables[b], 1.0 - 1e-12);
         }
         double mx = 0.0;
         for (double v : phi) mx = fmax(mx, fabs(v));
@@ -469,6 +525,8 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
                                                                             g->tab + (size_t)b * g->n_tab);
             GEOM_CUDA(cudaGetLastError());
         }
+    } else if (phi_eval == PHI_SEG) {
+        GEOM_CUDA(cudaMemcpy(g->tab, segments.data(), sizeof(float2) * segments.size(), cudaMemcpyHostToDevice));
     } else {
         // per band: (theta, 0), (0, 0), then a_1 .. a_{4 nq} as float pairs (zeros past n)
         std::vector<float2> packed((size_t)n_tables * n_tab, make_float2(0.0f, 0.0f));
