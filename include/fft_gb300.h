@@ -174,7 +174,7 @@ typedef struct {
 
 /*
  * fft_geom_autotune - pick the work decomposition of J and J^T for this geometry by timing
- * them on the device: a tile's candidate rows are cut into work items sized for 4, 8, 16, 32,
+ * them on the device (without it a rule on the number of entries sizes the items): a tile's candidate rows are cut into work items sized for 4, 8, 16, 32,
  * 64 or 128 items per persistent CTA (at least 64 rows each), with the most CTAs per SM that
  * fit or one fewer. The sizes are swept at the occupancy limit (stopping after two in a row
  * more than 2 % slower than the best), then the best size and its two neighbours with one CTA

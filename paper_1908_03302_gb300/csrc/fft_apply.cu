@@ -69,60 +69,66 @@ __global__ void __launch_bounds__(256) j_reduce4_kernel(const int64_t* __restric
     }
 }
 
-// g for voxels of tiles with several items (the slots summed in item order) or with none (0);
-// tiles with one item were written by the apply kernel. One thread takes 4 consecutive x
-// voxels of a tile (512 threads per tile); the slots are read 4 at a time so that several
-// loads are in flight, and added one by one from 0 in slot order (deterministic).
+// g for voxels of tiles with several items (the sum of their slots) or with none (0); tiles with
+// one item were written by the apply kernel. A CTA takes 32 runs of 4 x voxels of a tile, a lane
+// each; warp w adds slots w, w + 8, .. in that order (compensated, so that the sum does not lose
+// to the number of slots), the eight partial sums are added in FP64: a fixed order, and eight times
+// as many loads in flight as with one thread per run, which a tile cut into many small items
+// needs (32-element ring: about 45 slots per tile).
 // NCOL = 4: the four-column form, slot q of column r at gpart[((s0 + q) * 4 + r) * TILE_VOX],
 // g[r * V + v].
+constexpr int RED_WARPS = 8;
 template <int NCOL>
-__global__ void __launch_bounds__(256) jt_reduce_kernel(const int32_t* __restrict__ slot0,
-                                                        const int32_t* __restrict__ nslot,
-                                                        const float* __restrict__ gpart, int64_t n_tiles, int nx,
-                                                        int ny, int nz, int tiles_x, int tiles_y,
-                                                        float* __restrict__ g) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n_tiles * (TILE_VOX / 4)) return;
-    const int T = (int)(idx / (TILE_VOX / 4));
+__global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t* __restrict__ slot0,
+                                                                   const int32_t* __restrict__ nslot,
+                                                                   const float* __restrict__ gpart, int nx, int ny,
+                                                                   int nz, int tiles_x, int tiles_y,
+                                                                   float* __restrict__ g) {
+    __shared__ float4 sh[RED_WARPS][32];
+    constexpr int PER_TILE = TILE_VOX / (4 * 32);   // CTAs per tile
+    const int T = blockIdx.x / PER_TILE, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int s0 = slot0[T];
     if (s0 == -1) return;
-    const int loc = 4 * (int)(idx % (TILE_VOX / 4));
+    const int loc = 4 * (32 * (int)(blockIdx.x % PER_TILE) + lane);
     const int ix = TILE_X * (T % tiles_x) + loc % TILE_X;
     const int iy = TILE_Y * ((T / tiles_x) % tiles_y) + (loc / TILE_X) % TILE_Y;
     const int iz = TILE_Z * (T / (tiles_x * tiles_y)) + loc / (TILE_X * TILE_Y);
-    if (iy >= ny || iz >= nz || ix >= nx) return;
     const int64_t V = (int64_t)nx * ny * nz;
     const int64_t v = ((int64_t)iz * ny + iy) * nx + ix;
-    const int ns = (s0 == -2) ? 0 : nslot[T];
-#pragma unroll
+    const bool inside = iy < ny && iz < nz && ix < nx;
+    const int ns = (s0 == -2 || !inside) ? 0 : nslot[T];
     for (int r = 0; r < NCOL; ++r) {
-        float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, low[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         const float* base = ns > 0 ? gpart + ((int64_t)s0 * NCOL + r) * TILE_VOX + loc : nullptr;
-        int q = 0;
-        for (; q + 4 <= ns; q += 4) {
-            float4 w[4];
+        auto add = [&](const float4& x) {
+            const float xv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) w[k] = __ldcs(reinterpret_cast<const float4*>(base + (int64_t)(q + k) * NCOL * TILE_VOX));
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                acc.x += w[k].x;
-                acc.y += w[k].y;
-                acc.z += w[k].z;
-                acc.w += w[k].w;
+            for (int k = 0; k < 4; ++k) {   // Kahan's sum
+                const float y = xv[k] - low[k], t = acc[k] + y;
+                low[k] = (t - acc[k]) - y;
+                acc[k] = t;
             }
+        };
+        int q = w;
+        for (; q + 3 * RED_WARPS < ns; q += 4 * RED_WARPS) {   // four slots in flight
+            float4 x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                x[k] = __ldcs(reinterpret_cast<const float4*>(base + (int64_t)(q + k * RED_WARPS) * NCOL * TILE_VOX));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) add(x[k]);
         }
-        for (; q < ns; ++q) {
-            const float4 w = __ldcs(reinterpret_cast<const float4*>(base + (int64_t)q * NCOL * TILE_VOX));
-            acc.x += w.x;
-            acc.y += w.y;
-            acc.z += w.z;
-            acc.w += w.w;
+        for (; q < ns; q += RED_WARPS)
+            add(__ldcs(reinterpret_cast<const float4*>(base + (int64_t)q * NCOL * TILE_VOX)));
+        sh[w][lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        __syncthreads();
+        if (w < 4) {   // warp w: component w of the 32 runs
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < RED_WARPS; ++k) s += (double)reinterpret_cast<const float*>(&sh[k][lane])[w];
+            if (inside && ix + w < nx) g[(int64_t)r * V + v + w] = (float)s;
         }
-        float* out = g + (int64_t)r * V + v;
-        out[0] = acc.x;
-        if (ix + 1 < nx) out[1] = acc.y;
-        if (ix + 2 < nx) out[2] = acc.z;
-        if (ix + 3 < nx) out[3] = acc.w;
+        if (NCOL > 1) __syncthreads();
     }
 }
 
@@ -302,11 +308,9 @@ fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStrea
 
 template <int NCOL>
 static fft_status launch_jt_reduce(fft_geom g, const float* gpart, float* gout, cudaStream_t st) {
-    const int64_t threads = g->n_tiles * (TILE_VOX / 4);
-    if (threads == 0) return FFT_OK;
-    jt_reduce_kernel<NCOL><<<(unsigned)ceil_div(threads, 256), 256, 0, st>>>(
-        g->tile_slot0, g->tile_nslot, gpart, g->n_tiles, g->grid.nx, g->grid.ny, g->grid.nz, g->tiles[0],
-        g->tiles[1], gout);
+    if (g->n_tiles == 0) return FFT_OK;
+    jt_reduce_kernel<NCOL><<<(unsigned)(g->n_tiles * (TILE_VOX / 128)), 32 * RED_WARPS, 0, st>>>(
+        g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->tiles[0], g->tiles[1], gout);
     FFT_CUDA(cudaGetLastError());
     return FFT_OK;
 }

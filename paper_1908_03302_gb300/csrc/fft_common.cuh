@@ -54,7 +54,7 @@ constexpr int APPLY_THREADS = APPLY_WARPS * 32;
 constexpr int NX_LANE = 4;             // voxels per lane per sub-brick (along x)
 constexpr int SUBS_PER_WARP = 2;
 constexpr int MAX_BANDS = 8;
-constexpr int DEFAULT_ITEMS_PER_CTA = 8;   // work items per persistent CTA before tuning
+constexpr int DEFAULT_ITEMS_PER_CTA = 0;   // before tuning: items sized by default_item_rows
 constexpr float CULL_MARGIN = 2e-3f;   // in units of the band's maximum detour
 
 // Per-row record, lengths in units of the row's band maximum detour U_b = c0 * dt_max_b.

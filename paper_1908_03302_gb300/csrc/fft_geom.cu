@@ -293,17 +293,39 @@ void free_geom(fft_geom g) {
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
+// Rows per work item of a launch over E entries when no tuning has chosen it. Small items cost J^T
+// a partial slot each (8 KB written and read back, ~3 ns), large ones leave warps idle while the
+// last are finished (about 0.2 us per row: a unit's rows run one after another in one warp). The
+// sum of the two, 3 ns E / n + 0.2 us n, is least at n = sqrt(0.015 E): 230 rows on ring256 (3.5 M
+// entries; the autotuner picks 242 there), 11 on the 32-element ring (8 k entries), where it also
+// makes about one unit per resident warp. Against eight items per CTA of at least 64 rows: ring256 J
+// 3.79 -> 3.56 ms, its three-band J 14.05 -> 11.98 ms, a 20-iteration solve of four 32-element
+// slices 8.1 -> 5.2 ms.
+int64_t default_item_rows(int64_t E) {
+    const int64_t n = std::max<int64_t>(8, (int64_t)sqrt(0.015 * (double)E));
+    return n < 32 ? n : ceil_div(n, 32) * 32;
+}
+
 // Work items: a tile's candidate rows in ranges of at most ch rows, ch chosen so that each
-// persistent CTA sees about items_per_cta items (at least 64 rows, a multiple of 32); tiles
-// split over several items write J^T partial slots. Heaviest items first. Replaces the
-// geometry's previous items, slots and partial buffers (the J partials do not depend on them).
+// persistent CTA sees about items_per_cta items (at least 64 rows, a multiple of 32), or by
+// default_item_rows when items_per_cta is 0; tiles split over several items write J^T partial
+// slots. Heaviest items first. Replaces the geometry's previous items, slots and partial buffers
+// (the J partials do not depend on them).
 fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_per_cta) {
-    const int64_t target = (int64_t)items_per_cta * g->apply_ctas;
-    int64_t ch = std::max<int64_t>(64, ceil_div(std::max<int64_t>(g->E, 1), std::max<int64_t>(target, 1)));
-    ch = ceil_div(ch, 32) * 32;
     // plain rows [toff, toff + nplain) and sharp-band rows [toff + nplain, toff1) of a split
-    // geometry go to different items; the tile's slots number its plain items first
+    // geometry go to different items and launches; the tile's slots number its plain items first
     const bool split = !g->tile_nplain.empty();
+    int64_t chp, chs;   // rows per plain and per sharp item
+    if (items_per_cta > 0) {
+        const int64_t target = (int64_t)items_per_cta * g->apply_ctas;
+        chp = std::max<int64_t>(64, ceil_div(std::max<int64_t>(g->E, 1), std::max<int64_t>(target, 1)));
+        chp = chs = ceil_div(chp, 32) * 32;
+    } else {
+        int64_t Ep = g->E;
+        if (split) Ep = std::accumulate(g->tile_nplain.begin(), g->tile_nplain.end(), (int64_t)0);
+        chp = default_item_rows(Ep);
+        chs = default_item_rows(g->E - Ep);
+    }
     std::vector<Item> items, items_sharp;
     std::vector<int32_t> slot0(g->n_tiles, -2), nslot(g->n_tiles, 0);
     int32_t slots = 0;
@@ -311,7 +333,7 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
         const int64_t n = toff[T + 1] - toff[T];
         if (n == 0) continue;
         const int64_t np = split ? g->tile_nplain[T] : n;
-        const int64_t kp = ceil_div(np, ch), ks = ceil_div(n - np, ch), k = kp + ks;
+        const int64_t kp = ceil_div(np, chp), ks = ceil_div(n - np, chs), k = kp + ks;
         if (k == 1) {
             (kp == 1 ? items : items_sharp).push_back(Item{(int32_t)T, -1, toff[T], toff[T + 1]});
             slot0[T] = -1;
@@ -320,7 +342,7 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
             nslot[T] = (int32_t)k;
             for (int64_t q = 0; q < k; ++q) {
                 const int64_t lo = q < kp ? toff[T] : toff[T] + np, hi = q < kp ? toff[T] + np : toff[T + 1];
-                const int64_t a = lo + (q < kp ? q : q - kp) * ch, b = std::min(hi, a + ch);
+                const int64_t a = lo + (q < kp ? q * chp : (q - kp) * chs), b = std::min(hi, a + (q < kp ? chp : chs));
                 (q < kp ? items : items_sharp).push_back(Item{(int32_t)T, slots + (int32_t)q, a, b});
             }
             slots += (int32_t)k;
