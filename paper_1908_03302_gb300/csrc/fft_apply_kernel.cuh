@@ -17,7 +17,8 @@
 //     sub-bricks it reaches.
 //   * Per (row, voxel): pair-frame coordinates by FFMA from per-lane offsets, normalised
 //     detour (cancellation-free form), Phi from the band table in shared memory (one 64-bit
-//     load, linear interpolation), geometric factor 1 / (R_xs R_xr).
+//     load, linear interpolation), geometric factor 1 / (R_xs R_xr). A lane's voxels are
+//     evaluated as packed pairs (eval_deep, eval4).
 //   * J^T accumulates per voxel in registers over the item's rows (gather, no atomics).
 //     J folds each row's lane partials to 8 with two shuffles, parks them in the row's
 //     consumed staging record, and the row's own lane sums them after the chunk: one partial
@@ -71,14 +72,21 @@ struct ApplyParams {
     int64_t nvox, nrow;      // column lengths of the batch modes' blocks (V, M)
 };
 
-// Phi of the normalised detour v (table lookup, sine series or its piecewise quadratics, see
-// fft_device.cuh): tb is the band data's shared address (PHI_SEG: the bits of the band's magic
-// number, `tab` the shared address of all bands' segments and `seg2` that of their c2).
+// Where the kernels find Phi: `tab` the shared address of the bands' tables or segments, `seg2` that
+// of the segments' c2, scale and nq as in phi_lookup_at, phi_seg and phi_trig.
+struct PhiAt {
+    uint32_t tab, seg2;
+    float scale;
+    int nq;
+};
+
+// Phi of the normalised detour v (fft_device.cuh); row_m is the magic number of the row's band
+// (PHI_TRIG: the bits of the shared address of the band's block).
 template <int PHI>
-__device__ __forceinline__ float phi_eval(float v, uint32_t tb, float nm1, int nq, uint32_t tab, uint32_t seg2) {
-    if (PHI == PHI_TRIG) return phi_trig(v, tb, nq);
-    if (PHI == PHI_SEG) return phi_seg(v, __uint_as_float(tb), nm1, tab, seg2);
-    return phi_lookup(v, tb, nm1);
+__device__ __forceinline__ float phi_eval(float v, float row_m, const PhiAt& at) {
+    if (PHI == PHI_TRIG) return phi_trig(v, __float_as_uint(row_m), at.nq);
+    if (PHI == PHI_SEG) return phi_seg(v, row_m, at.scale, at.tab, at.seg2);
+    return phi_lookup_at(v, row_m, at.scale, at.tab);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -175,34 +183,201 @@ __device__ __forceinline__ void sub_step(int s, float hx, float hy, float hz, fl
     }
 }
 
+// Detour form of a sub-brick (staged per row): general, between the pair's transducer planes
+// (no absolute values), deep inside the pair's sphere (fft_device.cuh).
+enum { FORM_GENERAL = 0, FORM_INNER = 1, FORM_DEEP = 2 };
+
+// Staged flag word: band (bits 0-7), sharp band (8), planar pair (9), and per sub-brick s of the
+// unit: the row may reach it (12 + s), it is inner (16 + s), it is deep (20 + s); and per z layer h
+// of the unit (sub-bricks 2 h and 2 h + 1): both are reached and deep (24 + h).
+__device__ __forceinline__ int form_of(uint32_t cw, int s) {
+    return ((cw >> (20 + s)) & 1u) ? FORM_DEEP : (((cw >> (16 + s)) & 1u) ? FORM_INNER : FORM_GENERAL);
+}
+
+// Per-row values of the deep form at a lane: X = ps pr + q2 is a quadratic in the voxel index t
+// along the lane's run, X(t) = X(0) + t (b + t h^2) with b = 2 h (x - o)_x the same in every
+// sub-brick, so that the run needs no stepped axial offsets.
+struct DeepRow {
+    float b, hh;              // 2 h (x - o)_x and h^2
+    float lam, l2;            // L / U and its square
+    float k2, k3, k4, k5;     // lam DEEP_C2 .. lam DEEP_C5
+};
+
+__device__ __forceinline__ void deep_init(DeepRow& d, float lam) {
+    d.lam = lam;
+    d.l2 = __fmul_rn(lam, lam);
+    d.k2 = __fmul_rn(lam, DEEP_C2);
+    d.k3 = __fmul_rn(lam, DEEP_C3);
+    d.k4 = __fmul_rn(lam, DEEP_C4);
+    d.k5 = __fmul_rn(lam, DEEP_C5);
+}
+
+template <bool PL>
+__device__ __forceinline__ void deep_row(DeepRow& d, float ps, float pr, float c2, float c3, float hx, float hy,
+                                         float hz) {
+    float g = __fmul_rn(c3, hy);
+    d.hh = fmaf(hx, hx, __fmul_rn(hy, hy));
+    if (!PL) {
+        g = fmaf(-c2, hz, g);
+        d.hh = fmaf(hz, hz, d.hh);
+    }
+    d.b = fmaf(2.0f, g, __fmul_rn(hx, __fadd_rn(ps, pr)));
+}
+
+// Saturates the detour v = m0 m1 of each voxel pair to [0, 1]. SH: near becomes the smallest |v - 1|
+// seen before saturation.
+template <bool SH>
+__device__ __forceinline__ f2 settle(f2 m0, f2 m1, float& near) {
+    if (SH) {
+        const float2 d = up(add2(mul2(m0, m1), pk1(-1.0f)));
+        near = fminf(fminf(near, fabsf(d.x)), fabsf(d.y));
+    }
+    const float2 a = up(m0), b = up(m1);
+    return pk(__saturatef(a.x * b.x), __saturatef(a.y * b.y));
+}
+
+// q2 of a lane's four voxels t = 0 .. 3 of one sub-brick from the pair-frame values at t = 0, as
+// pairs (0, 1), (2, 3). c12 is c1^2 + c2^2 for a planar pair (constant along the run), c1^2
+// otherwise.
+template <bool PL>
+__device__ __forceinline__ void line_q2(float c2, float c3, float c12, float hy, float hz, f2 (&q2)[2]) {
+    const f2 T[2] = {pk(0.0f, 1.0f), pk(2.0f, 3.0f)};
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const f2 c3t = fma2(T[j], pk1(hy), pk1(c3));
+        q2[j] = fma2(c3t, c3t, pk1(c12));
+        if (!PL) {
+            const f2 c2t = fma2(T[j], pk1(-hz), pk1(c2));
+            q2[j] = fma2(c2t, c2t, q2[j]);
+        }
+    }
+}
+
+// Detours v (saturated) and w = 1 / (R_xs R_xr) of the lane's four voxels in each of NS deep
+// sub-bricks, stage by stage over all of them: 2 NS independent chains hide the latency of the
+// special-function unit better than one sub-brick's two.
+template <int NS, bool SH, bool PL>
+__device__ __forceinline__ void eval_deep(const float (&ps)[NS], const float (&pr)[NS], const float (&c2)[NS],
+                                          const float (&c3)[NS], const float (&c12)[NS], float hy, float hz,
+                                          const DeepRow& k, f2 (&v)[NS][2], f2 (&w)[NS][2], float& near) {
+    const f2 T[2] = {pk(0.0f, 1.0f), pk(2.0f, 3.0f)};
+    f2 q2[NS][2], X[NS][2], y[NS][2], Q[NS][2];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) line_q2<PL>(c2[s], c3[s], c12[s], hy, hz, q2[s]);
+#define FFT_EACH _Pragma("unroll") for (int s = 0; s < NS; ++s) _Pragma("unroll") for (int j = 0; j < 2; ++j)
+    FFT_EACH X[s][j] = fma2(T[j], fma2(T[j], pk1(k.hh), pk1(k.b)), pk1(fmaf(ps[s], pr[s], up(q2[s][0]).x)));
+    FFT_EACH Q[s][j] = fma2(X[s][j], X[s][j], mul2(pk1(k.l2), q2[s][j]));   // D
+    FFT_EACH w[s][j] = rsqrt2(Q[s][j]);
+    FFT_EACH y[s][j] = rcp2(fma2(Q[s][j], w[s][j], neg2(X[s][j])));
+    FFT_EACH y[s][j] = mul2(q2[s][j], y[s][j]);
+    FFT_EACH Q[s][j] = fma2(pk1(k.k5), y[s][j], pk1(k.k4));
+    FFT_EACH Q[s][j] = fma2(Q[s][j], y[s][j], pk1(k.k3));
+    FFT_EACH Q[s][j] = fma2(Q[s][j], y[s][j], pk1(k.k2));
+    FFT_EACH Q[s][j] = fma2(Q[s][j], y[s][j], pk1(k.lam));
+    FFT_EACH v[s][j] = settle<SH>(y[s][j], Q[s][j], near);
+#undef FFT_EACH
+}
+
+// The same for one sub-brick in the other forms (general, inner).
+template <int DT, bool GUARD, bool SH, int FORM, bool PL>
+__device__ __forceinline__ void eval4(float ps, float pr, float c2, float c3, float c12, float hx, float hy, float hz,
+                                      float hl, f2 (&v)[2], f2 (&w)[2], float& near) {
+    const f2 T[2] = {pk(0.0f, 1.0f), pk(2.0f, 3.0f)};
+    f2 q2[2];
+    line_q2<PL>(c2, c3, c12, hy, hz, q2);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const f2 pst = fma2(T[j], pk1(hx), pk1(ps)), prt = fma2(T[j], pk1(hx), pk1(pr));
+        f2 m0, m1;   // v is the product m0 m1
+        if (DT == FFT_DT_STABLE && !GUARD && FORM == FORM_INNER) {
+            const f2 ss = fma2(pst, pst, q2[j]), rr = fma2(prt, prt, q2[j]);
+            const f2 is = rsqrt2(ss), ir = rsqrt2(rr);
+            const f2 A = fma2(ss, is, pst), B = fma2(rr, ir, neg2(prt));
+            w[j] = mul2(is, ir);
+            m0 = mul2(q2[j], add2(A, B));
+            m1 = rcp2(mul2(A, B));
+        } else {
+            const float2 a = up(pst), b = up(prt), q = up(q2[j]);
+            float is0, ir0, is1, ir1;
+            const float v0 = detour_v<DT, GUARD, FORM == FORM_INNER, true>(a.x, b.x, q.x, hl, is0, ir0);
+            const float v1 = detour_v<DT, GUARD, FORM == FORM_INNER, true>(a.y, b.y, q.y, hl, is1, ir1);
+            w[j] = pk(is0 * ir0, is1 * ir1);
+            m0 = pk(v0, v1);
+            m1 = pk1(1.0f);
+        }
+        v[j] = settle<SH>(m0, m1, near);
+    }
+}
+
+// One voxel's detour before saturation, by the operations that eval_deep and eval4 pack (the same bits): t the
+// voxel of the run, the other arguments as there.
+template <int DT, bool GUARD>
+__device__ __forceinline__ float eval1_raw(int form, bool planar, int t, float ps, float pr, float c2, float c3,
+                                           float c12, float hx, float hy, float hz, float hl, const DeepRow& k,
+                                           float& w) {
+    const float ft = (float)t;
+    auto q2_at = [&](float f) {
+        const float c3t = fmaf(f, hy, c3);
+        float q = fmaf(c3t, c3t, c12);
+        if (!planar) {
+            const float c2t = fmaf(f, -hz, c2);
+            q = fmaf(c2t, c2t, q);
+        }
+        return q;
+    };
+    const float q2 = q2_at(ft);
+    if (form == FORM_DEEP) {
+        const float x0 = fmaf(ps, pr, q2_at(0.0f));
+        const float X = fmaf(ft, fmaf(ft, k.hh, k.b), x0);
+        const float D = fmaf(X, X, __fmul_rn(k.l2, q2));
+        w = rsqrt_approx(D);
+        const float y = __fmul_rn(q2, rcp_approx(fmaf(D, w, -X)));
+        float Q = fmaf(k.k5, y, k.k4);
+        Q = fmaf(Q, y, k.k3);
+        Q = fmaf(Q, y, k.k2);
+        return __fmul_rn(y, fmaf(Q, y, k.lam));
+    }
+    const float pst = fmaf(ft, hx, ps), prt = fmaf(ft, hx, pr);
+    float is, ir;
+    const float v = form == FORM_INNER ? detour_v<DT, GUARD, true, true>(pst, prt, q2, hl, is, ir)
+                                       : detour_v<DT, GUARD, false, true>(pst, prt, q2, hl, is, ir);
+    w = is * ir;
+    return v;
+}
+
 // The FP64 re-decision of the sharp-band kernels, out of line (called only for an entry where
 // some lane's FP32 detour lies within CUT_BAND of the cut), so that its FP64 temporaries do not
 // weigh on the register allocation of the main loop. For each of the lane's 4 NSUB voxels
 // (k = 4 s + t) it recomputes the FP32 detour by the operations of the main pass, and for the
 // voxels near the cut re-decides dt < dt_max in FP64. It returns in d[k] what the main pass's
 // term has to change by: val2 - val1 (J, J^T, four-column modes), |val2| - |val1| (coverage),
-// val2^2 - val1^2 (Frobenius), +1 / -1 (support count), 0 where nothing changes. `inner` holds
-// the sub-bricks lying between the transducer planes (bit s).
+// val2^2 - val1^2 (Frobenius), +1 / -1 (support count), 0 where nothing changes. p is the row.
 template <int MODE, int DT, bool GUARD, int PHI, int NSUB>
-__device__ __noinline__ void sharp_fix(const ApplyParams& P, float4 A, float4 B, float4 C, float Xl, float Yl,
-                                       float Zl, bool planar, uint32_t inner_bits, float cutb, uint32_t tb,
-                                       float nm1, int nq, uint32_t tab, uint32_t seg2, int ix0, int iy0, int iz0,
-                                       float* d) {
+__device__ __noinline__ void sharp_fix(const ApplyParams& P, float4 A, float4 B, float4 C, int p, float Xl, float Yl,
+                                       float Zl, const PhiAt& at, int ix0, int iy0, int iz0, float* d) {
     const float hx = B.x, hy = B.y, hz = B.z;
     const float hl = 0.5f * (A.x - A.y);
-    const int b = __float_as_int(C.w) & 0xff;
-    const double U = P.bc[b].U;
+    const uint32_t cw = (uint32_t)__float_as_int(C.w);
+    const bool planar = (cw >> 9) & 1u;
+    const double U = P.bc[cw & 0xffu].U;
+    DeepRow dr;
+    deep_init(dr, C.z);
     // one voxel per iteration, each recomputed from the lane base (few values live across
     // iterations, which keeps the caller's register saves around this call small)
 #pragma unroll 1
     for (int k = 0; k < 4 * NSUB; ++k) {
         const int s = k >> 2, t = k & 3;
         d[k] = 0.0f;
+        if (!((cw >> (12 + s)) & 1u)) continue;   // the main pass skipped the sub-brick
         const float offs = planar ? fmaf(Xl, hx, Yl * hy) : fmaf(Xl, hx, fmaf(Yl, hy, Zl * hz));
         float pss = A.x + offs, prs = A.y + offs;
         float c1s = planar ? fmaf(-Zl, hy, A.z) : fmaf(Yl, hz, fmaf(-Zl, hy, A.z));
         float c2s = planar ? fmaf(Zl, hx, A.w) : fmaf(Zl, hx, fmaf(-Xl, hz, A.w));
         float c3s = fmaf(Xl, hy, fmaf(-Yl, hx, B.w));
+        if (planar)
+            deep_row<true>(dr, pss, prs, c2s, c3s, hx, hy, hz);
+        else
+            deep_row<false>(dr, pss, prs, c2s, c3s, hx, hy, hz);
 #pragma unroll 1
         for (int q = 1; q <= s; ++q) {
             if (planar)
@@ -210,35 +385,23 @@ __device__ __noinline__ void sharp_fix(const ApplyParams& P, float4 A, float4 B,
             else
                 sub_step<NSUB, false>(q, hx, hy, hz, pss, prs, c1s, c2s, c3s);
         }
-        const float ft = (float)t;
-        const float c1sq = c1s * c1s;
-        const float pst = (t == 0 ? pss : fmaf(ft, hx, pss));
-        const float prt = (t == 0 ? prs : fmaf(ft, hx, prs));
-        const float c3t = (t == 0 ? c3s : fmaf(ft, hy, c3s));
-        float q2;
-        if (planar) {
-            q2 = fmaf(c3t, c3t, fmaf(c2s, c2s, c1sq));
-        } else {
-            const float c2t = (t == 0 ? c2s : fmaf(-ft, hz, c2s));
-            q2 = fmaf(c2t, c2t, fmaf(c3t, c3t, c1sq));
-        }
-        const bool inner = (DT == FFT_DT_STABLE) && ((inner_bits >> s) & 1u);
-        float is, ir;
-        const float vr = inner ? detour_v<DT, GUARD, true, true>(pst, prt, q2, hl, is, ir)
-                               : detour_v<DT, GUARD, false, true>(pst, prt, q2, hl, is, ir);
-        if (!(fabsf(vr - 1.0f) < cutb)) continue;
+        const float c1sq = __fmul_rn(c1s, c1s);
+        const float c12 = planar ? fmaf(c2s, c2s, c1sq) : c1sq;
+        float w;
+        const float vr = eval1_raw<DT, GUARD>(DT == FFT_DT_STABLE ? form_of(cw, s) : FORM_GENERAL, planar, t, pss, prs,
+                                              c2s, c3s, c12, hx, hy, hz, hl, dr, w);
+        if (!(fabsf(vr - 1.0f) < CUT_BAND)) continue;
         const float v = __saturatef(vr);
-        const bool in = in_support64(P.rec64[__float_as_int(C.z)], P.org[0], P.org[1], P.org[2], P.h, ix0 + t,
-                                     iy0 + sub_dy<NSUB>(s), iz0 + sub_dz<NSUB>(s), U);
+        const bool in = in_support64(P.rec64[p], P.org[0], P.org[1], P.org[2], P.h, ix0 + t, iy0 + sub_dy<NSUB>(s),
+                                     iz0 + sub_dz<NSUB>(s), U);
         const float v2 = settle_cut(v, in);
         if (v2 == v) continue;
         if (MODE == MODE_COUNT) {
             d[k] = (v2 < 1.0f) ? 1.0f : -1.0f;
             continue;
         }
-        const float w = is * ir;
-        const float val1 = phi_eval<PHI>(v, tb, nm1, nq, tab, seg2) * w;
-        const float val2 = phi_eval<PHI>(v2, tb, nm1, nq, tab, seg2) * w;
+        const float val1 = phi_eval<PHI>(v, C.y, at) * w;
+        const float val2 = phi_eval<PHI>(v2, C.y, at) * w;
         if (MODE == MODE_COV) d[k] = fabsf(val2) - fabsf(val1);
         else if (MODE == MODE_FROB) d[k] = val2 * val2 - val1 * val1;
         else d[k] = val2 - val1;
@@ -290,16 +453,16 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
     __syncthreads();   // the only CTA-wide barrier: from here on every warp runs on its own
 
     const uint32_t tab_addr = smem_addr(s_tab);
-    // table lookups scale v by n_tab - 1, segment lookups by seg_n 2^-22
-    const float nm1 = PHI == PHI_SEG ? (float)P.seg_n * MAGIC2_ULP : (float)(P.n_tab - 1);
-    const uint32_t seg2_addr = tab_addr + (uint32_t)(P.n_bands * (P.seg_n + SEG_PAD)) * 8u;
-    const int nq = P.trig_nq;
+    PhiAt at;
+    at.tab = tab_addr;
+    at.seg2 = tab_addr + (uint32_t)(P.n_bands * (P.seg_n + SEG_PAD)) * 8u;
+    at.scale = (float)(PHI == PHI_SEG ? P.seg_n : P.n_tab - 1) * MAGIC2_ULP;
+    at.nq = P.trig_nq;
     const int lx = lane & 1, ly = (lane >> 1) & 3, lz = lane >> 3;
     constexpr bool BATCH = (MODE == MODE_JT4 || MODE == MODE_J4);
-    constexpr int SR = BATCH ? 4 : 3;   // staged float4 per row
+    constexpr int SR = (MODE == MODE_JT4) ? 4 : 3;   // staged float4 per row
     constexpr int NSUB = apply_nsub<MODE>();
     constexpr int NREG = apply_regions<MODE>();
-    constexpr bool FLAGW = (NSUB == 4);
     float4* stg = s_stage + warp * STG_PER_WARP;
     const int n_units = P.n_items * NREG;
 
@@ -345,27 +508,29 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
         const uint32_t vmask = VM_LIVE ? lane_vmask() : 0u;
         const int64_t vbase = ((int64_t)(TZ + ozi) * P.ny + TY + oyi) * P.nx + TX + oxi;
 
-        float acc[NSUB][NX_LANE];
-        float mv[NSUB][NX_LANE];
-        float acc4[2][NX_LANE][4];   // four-column modes only (NSUB = 2)
-        float mv4[2][NX_LANE][4];
+        // accumulators (J^T) or model values (J) of the lane's voxels, as pairs (0, 1), (2, 3) of
+        // each run
+        f2 acc[NSUB][2], mv[NSUB][2];
+        f2 acc4[2][2][4], mv4[2][2][4];   // four-column modes only (NSUB = 2)
         double dacc = 0.0;
         unsigned long long cnt = 0, cnt_eval = 0;
 #pragma unroll
         for (int s = 0; s < NSUB; ++s)
 #pragma unroll
-            for (int t = 0; t < NX_LANE; ++t) {
-                const int64_t vo = vbase + ((int64_t)sub_dz<NSUB>(s) * P.ny + sub_dy<NSUB>(s)) * P.nx + t;
-                acc[s][t] = 0.0f;
-                mv[s][t] = 0.0f;
-                if (MODE == MODE_J && ((vmask >> (4 * s + t)) & 1u)) mv[s][t] = __ldg(P.vin + vo);
+            for (int j = 0; j < 2; ++j) {
+                const int64_t vo = vbase + ((int64_t)sub_dz<NSUB>(s) * P.ny + sub_dy<NSUB>(s)) * P.nx + 2 * j;
+                const bool ok0 = (vmask >> (4 * s + 2 * j)) & 1u, ok1 = (vmask >> (4 * s + 2 * j + 1)) & 1u;
+                acc[s][j] = mv[s][j] = 0ull;
+                if (MODE == MODE_J)
+                    mv[s][j] = pk(ok0 ? __ldg(P.vin + vo) : 0.0f, ok1 ? __ldg(P.vin + vo + 1) : 0.0f);
                 if (BATCH && s < 2) {
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
-                        acc4[s & 1][t][r] = 0.0f;
-                        mv4[s & 1][t][r] = 0.0f;
-                        if (MODE == MODE_J4 && ((vmask >> (4 * s + t)) & 1u))
-                            mv4[s & 1][t][r] = __ldg(P.vin + (int64_t)r * P.nvox + vo);
+                        acc4[s & 1][j][r] = mv4[s & 1][j][r] = 0ull;
+                        if (MODE == MODE_J4) {
+                            const float* mr = P.vin + (int64_t)r * P.nvox + vo;
+                            mv4[s & 1][j][r] = pk(ok0 ? __ldg(mr) : 0.0f, ok1 ? __ldg(mr + 1) : 0.0f);
+                        }
                     }
                 }
             }
@@ -374,7 +539,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
             // ---- stage: lane l prepares row e0 + l
             const int64_t e = e0 + lane;
             const bool have = e < item.e1;
-            uint32_t okb = 0, inb = 0;   // sub-bricks the row may reach / lying between its transducer planes
+            uint32_t okb = 0;   // sub-bricks the row may reach
             if (have) {
                 const int p = P.tile_rows[e];
                 const float4 base = P.ebase[e];
@@ -401,6 +566,12 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const bool live = (MODE == MODE_JT4) ? (W4.x != 0.0f || W4.y != 0.0f || W4.z != 0.0f || W4.w != 0.0f)
                                                      : ((MODE != MODE_JT && MODE != MODE_COV) || (W != 0.0f));
                 const float pext = hxx * fabsf(ex) + hyy * (fabsf(ey) + fabsf(ez)) + 1e-3f;
+                // deep sub-bricks: their voxel centres (half diagonal sqrt(3.5^2 + 2 1.5^2) = 4.1 steps)
+                // keep DEEP_MARGIN steps off the pair's sphere
+                const float lam = 2.0f * hl;
+                const float rim = hl - (4.1f + DEEP_MARGIN) * hb;
+                const float rim2 = (DT == FFT_DT_STABLE && lam >= DEEP_MIN_L && rim > 0.0f) ? rim * rim : -1.0f;
+                uint32_t inb = 0, dpb = 0;
 #pragma unroll
                 for (int s = 0; s < NSUB; ++s) {
                     const float cy = fmaf(8.0f * wy + (float)sub_dy<NSUB>(s) + 1.5f, hb, dy);
@@ -409,29 +580,22 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         okb |= 1u << s;
                     // sub-bricks whose voxels all satisfy |p| <= hl (between the transducer planes)
                     if (fabsf(fmaf(cx, ex, fmaf(cy, ey, cz * ez))) + pext <= hl) inb |= 1u << s;
+                    if (fmaf(cx, cx, fmaf(cy, cy, cz * cz)) <= rim2) dpb |= 1u << s;
                 }
-                const uint32_t tb =
-                    PHI == PHI_SEG ? __float_as_uint(fmaf((float)(b * (P.seg_n + SEG_PAD)), MAGIC2_ULP, MAGIC2))
-                                   : tab_addr + (uint32_t)(b * P.n_tab) * 8u - (PHI == PHI_TABLE ? MAGIC_BITS_X8 : 0u);
+                const uint32_t od = okb & dpb, both = ((od & 3u) == 3u ? 1u : 0u) | ((od & 12u) == 12u ? 2u : 0u);
                 stg[lane * SR + 0] = base;
                 stg[lane * SR + 1] = make_float4(hb * ex, hb * ey, hb * ez, base3);
-                if (MODE == MODE_JT4) stg[lane * SR + 3] = W4;
                 // planar pair (both transducers at one z): stepping along x changes only c3
                 const int planar = (ez == 0.0f) ? 1 : 0;
-                // flags word: band (bits 0-7), sharp band (8), planar pair (9); with four
-                // sub-bricks also the sub-bricks the row may reach (12 + s) and the inner ones
-                // (16 + s)
-                const uint32_t fl = FLAGW ? ((okb << 12) | (inb << 16)) : 0u;
-                stg[lane * SR + 2] = make_float4(W, __uint_as_float(tb), __int_as_float(p),
-                                                __int_as_float(b | (bc.sharp << 8) | (planar << 9) | (int)fl));
-            }
-            // With two sub-bricks the per-row tests read warp-uniform ballots (uniform branches);
-            // with four, the row's staged flag word (eight ballots per chunk cost more there).
-            uint32_t mk[NSUB], ik[NSUB];
-#pragma unroll
-            for (int s = 0; s < NSUB; ++s) {
-                mk[s] = FLAGW ? 0u : __ballot_sync(0xffffffffu, (okb >> s) & 1u);
-                ik[s] = FLAGW ? 0u : __ballot_sync(0xffffffffu, (inb >> s) & 1u);
+                // third word: the band's place (the magic number of its lookups; PHI_TRIG: the
+                // shared address of its block), the pair's length; fourth: see form_of
+                const float row_m =
+                    PHI == PHI_TRIG ? __uint_as_float(tab_addr + (uint32_t)(b * P.n_tab) * 8u)
+                                    : fmaf((float)(b * (PHI == PHI_SEG ? P.seg_n + SEG_PAD : P.n_tab)), MAGIC2_ULP, MAGIC2);
+                stg[lane * SR + 2] = make_float4(W, row_m, DT == FFT_DT_FP64 ? __int_as_float(p) : lam,
+                                                 __int_as_float(b | (bc.sharp << 8) | (planar << 9) |
+                                                                (int)((okb << 12) | (inb << 16) | (dpb << 20) | (both << 24))));
+                if (MODE == MODE_JT4) stg[lane * SR + 3] = W4;
             }
             uint32_t mm = __ballot_sync(0xffffffffu, okb != 0u);
             __syncwarp();
@@ -443,194 +607,219 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const float4 A = stg[bit * SR + 0];
                 const float4 B = stg[bit * SR + 1];
                 const float4 C = stg[bit * SR + 2];
-                const float4 W4 = (MODE == MODE_JT4) ? stg[bit * SR + 3] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                const float4 W4 = (MODE == MODE_JT4) ? stg[bit * SR + SR - 1] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 const float Wr[4] = {W4.x, W4.y, W4.z, W4.w};
-                const float hx = B.x, hy = B.y, hz = B.z, W = C.x;
+                const float hx = B.x, hy = B.y, hz = B.z, W = C.x, row_m = C.y;
                 const float hl = 0.5f * (A.x - A.y);   // used by the textbook (NAIVE) detour only
-                const uint32_t tb = __float_as_uint(C.y);
                 const uint32_t cw = (uint32_t)__float_as_int(C.w);
-                // voxels whose FP32 detour falls within CUT_BAND of a sharp band's cut-off
-                const float cutb = (SHARP && ((cw >> 8) & 1u)) ? CUT_BAND : -1.0f;
                 const bool planar = (DT != FFT_DT_FP64) && ((cw >> 9) & 1u);
-                bool near = false;   // a voxel of this lane has its FP32 detour within CUT_BAND of the cut
-                // lane base (sub-brick 0, t = 0) in the pair frame: small offsets added to the
-                // tile origin's FP64-derived values
-                float part = 0.0f;
-                float part4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                DeepRow dr;
+                deep_init(dr, C.z);
+                float near = 2.0f;   // smallest |v - 1| of this lane's voxels (sharp bands)
+                f2 part = 0ull;
+                f2 part4[4] = {0ull, 0ull, 0ull, 0ull};
+                uint32_t n_in = 0;
+                float fsum = 0.0f;
+                // Phi and the mode's sum over one sub-brick's four voxels.
+                auto accumulate = [&](int s, const f2 (&v)[2], const f2 (&w)[2]) {
+                    const float2 va = up(v[0]), vb = up(v[1]);
+                    if (MODE == MODE_COUNT) {
+                        const uint32_t vm = (vmask >> (4 * s)) & 15u;
+                        const uint32_t in = (va.x < 1.0f ? 1u : 0u) | (va.y < 1.0f ? 2u : 0u) | (vb.x < 1.0f ? 4u : 0u) |
+                                            (vb.y < 1.0f ? 8u : 0u);
+                        n_in += __popc(in & vm) | (__popc(vm) << 16);
+                        return;
+                    }
+                    float ph[NX_LANE];
+                    if (PHI == PHI_TRIG) {
+                        const float vv[NX_LANE] = {va.x, va.y, vb.x, vb.y};
+                        phi_trig_n<NX_LANE>(vv, __float_as_uint(row_m), at.nq, ph);
+                    } else if (PHI == PHI_SEG) {
+                        ph[0] = phi_eval<PHI>(va.x, row_m, at);
+                        ph[1] = phi_eval<PHI>(va.y, row_m, at);
+                        ph[2] = phi_eval<PHI>(vb.x, row_m, at);
+                        ph[3] = phi_eval<PHI>(vb.y, row_m, at);
+                    } else {
+                        const float2 ta = up(fma2_rd(v[0], pk1(at.scale), pk1(row_m)));
+                        const float2 tb = up(fma2_rd(v[1], pk1(at.scale), pk1(row_m)));
+                        const float2 T0 = lds_f2_table(tab_addr, ta.x), T1 = lds_f2_table(tab_addr, ta.y);
+                        const float2 T2 = lds_f2_table(tab_addr, tb.x), T3 = lds_f2_table(tab_addr, tb.y);
+                        ph[0] = fmaf(va.x, T0.y, T0.x);
+                        ph[1] = fmaf(va.y, T1.y, T1.x);
+                        ph[2] = fmaf(vb.x, T2.y, T2.x);
+                        ph[3] = fmaf(vb.y, T3.y, T3.x);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const f2 val = mul2(pk(ph[2 * j], ph[2 * j + 1]), w[j]);
+                        if (MODE == MODE_JT) acc[s][j] = fma2(val, pk1(W), acc[s][j]);
+                        if (MODE == MODE_COV) {
+                            const float2 x = up(val);
+                            acc[s][j] = fma2(pk(fabsf(x.x), fabsf(x.y)), pk1(W), acc[s][j]);
+                        }
+                        if (MODE == MODE_J) part = fma2(val, mv[s][j], part);
+                        if (MODE == MODE_JT4) {
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) acc4[s & 1][j][r] = fma2(val, pk1(Wr[r]), acc4[s & 1][j][r]);
+                        }
+                        if (MODE == MODE_J4) {
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) part4[r] = fma2(val, mv4[s & 1][j][r], part4[r]);
+                        }
+                        if (MODE == MODE_FROB) {
+                            const float2 x = up(val);
+                            if ((vmask >> (4 * s + 2 * j)) & 1u) fsum = fmaf(x.x, x.x, fsum);
+                            if ((vmask >> (4 * s + 2 * j + 1)) & 1u) fsum = fmaf(x.y, x.y, fsum);
+                        }
+                    }
+                };
                 // The entry's evaluation, specialised for planar pairs (both transducers at one
                 // z: the axis has no z component, so h_z = 0 exactly, c1 and c2 do not change
                 // along the lane's voxels or between sub-bricks at one z, and p does not change
-                // in z).
+                // in z). The lane base (sub-brick 0, t = 0) is a small offset added to the tile
+                // origin's FP64-derived values.
                 // SH: the near-cut checks, only for rows of a band whose Phi does not vanish at
-                // the cut (the other rows of a sharp geometry take the plain evaluation; both
-                // give the same values there).
+                // the cut (the four-column launches take a sharp geometry's other rows too).
                 auto entry_body = [&](auto planar_tag, auto sharp_tag) {
                     constexpr bool PL = decltype(planar_tag)::value;
                     constexpr bool SH = decltype(sharp_tag)::value;
-                const float off = PL ? fmaf(Xl, hx, Yl * hy) : fmaf(Xl, hx, fmaf(Yl, hy, Zl * hz));
-                float psb = A.x + off, prb = A.y + off;
-                float c1 = PL ? fmaf(-Zl, hy, A.z) : fmaf(Yl, hz, fmaf(-Zl, hy, A.z));
-                float c2 = PL ? fmaf(Zl, hx, A.w) : fmaf(Zl, hx, fmaf(-Xl, hz, A.w));
-                float c3 = fmaf(Xl, hy, fmaf(-Yl, hx, B.w));
-                float c12_planar = PL ? fmaf(c2, c2, c1 * c1) : 0.0f;
+                    const float off = PL ? fmaf(Xl, hx, Yl * hy) : fmaf(Xl, hx, fmaf(Yl, hy, Zl * hz));
+                    float psb = A.x + off, prb = A.y + off;
+                    float c1 = PL ? fmaf(-Zl, hy, A.z) : fmaf(Yl, hz, fmaf(-Zl, hy, A.z));
+                    float c2 = PL ? fmaf(Zl, hx, A.w) : fmaf(Zl, hx, fmaf(-Xl, hz, A.w));
+                    float c3 = fmaf(Xl, hy, fmaf(-Yl, hx, B.w));
+                    float c12_planar = PL ? fmaf(c2, c2, __fmul_rn(c1, c1)) : 0.0f;
+                    if (DT == FFT_DT_STABLE) deep_row<PL>(dr, psb, prb, c2, c3, hx, hy, hz);
+                    // two sub-bricks at a time (one z layer of the unit)
 #pragma unroll
-                for (int s = 0; s < NSUB; ++s) {
-                    if (s > 0) {
-                        sub_step<NSUB, PL>(s, hx, hy, hz, psb, prb, c1, c2, c3);
-                        if (PL && s == 2) c12_planar = fmaf(c2, c2, c1 * c1);
+                    for (int h = 0; h < NSUB / 2; ++h) {
+                        if (h > 0) {   // from sub-brick 1 to 2: +4 in z
+                            sub_step<NSUB, PL>(2, hx, hy, hz, psb, prb, c1, c2, c3);
+                            if (PL) c12_planar = fmaf(c2, c2, __fmul_rn(c1, c1));
+                        }
+                        float psv[2], prv[2], c2v[2], c3v[2], c12v[2];
+                        psv[0] = psb;
+                        prv[0] = prb;
+                        c2v[0] = c2;
+                        c3v[0] = c3;
+                        c12v[0] = PL ? c12_planar : __fmul_rn(c1, c1);
+                        sub_step<NSUB, PL>(2 * h + 1, hx, hy, hz, psb, prb, c1, c2, c3);
+                        psv[1] = psb;
+                        prv[1] = prb;
+                        c2v[1] = c2;
+                        c3v[1] = c3;
+                        c12v[1] = PL ? c12_planar : __fmul_rn(c1, c1);
+                        if (DT == FFT_DT_STABLE && ((cw >> (24 + h)) & 1u)) {
+                            f2 v[2][2], w[2][2];
+                            eval_deep<2, SH, PL>(psv, prv, c2v, c3v, c12v, hy, hz, dr, v, w, near);
+                            accumulate(2 * h, v[0], w[0]);
+                            accumulate(2 * h + 1, v[1], w[1]);
+                            continue;
+                        }
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const int s = 2 * h + q;
+                            if (!((cw >> (12 + s)) & 1u)) continue;
+                            f2 v[2], w[2];
+                            if (DT == FFT_DT_FP64) {
+                                const RowRec64 r64 = P.rec64[__float_as_int(C.z)];
+                                const double U = P.bc[cw & 0xffu].U;
+                                float vv[NX_LANE], ww[NX_LANE];
+#pragma unroll
+                                for (int t = 0; t < NX_LANE; ++t)
+                                    vv[t] = detour_v64(r64, P.org[0], P.org[1], P.org[2], P.h, TX + oxi + t,
+                                                       TY + oyi + sub_dy<NSUB>(s), TZ + ozi + sub_dz<NSUB>(s), U, ww[t]);
+                                v[0] = pk(vv[0], vv[1]);
+                                v[1] = pk(vv[2], vv[3]);
+                                w[0] = pk(ww[0], ww[1]);
+                                w[1] = pk(ww[2], ww[3]);
+                            } else if (DT == FFT_DT_STABLE && form_of(cw, s) == FORM_DEEP) {
+                                f2 v1[1][2], w1[1][2];
+                                const float a[1] = {psv[q]}, b[1] = {prv[q]}, c[1] = {c2v[q]}, d[1] = {c3v[q]}, f[1] = {c12v[q]};
+                                eval_deep<1, SH, PL>(a, b, c, d, f, hy, hz, dr, v1, w1, near);
+                                v[0] = v1[0][0];
+                                v[1] = v1[0][1];
+                                w[0] = w1[0][0];
+                                w[1] = w1[0][1];
+                            } else if (DT == FFT_DT_STABLE && form_of(cw, s) == FORM_INNER) {
+                                eval4<DT, GUARD, SH, FORM_INNER, PL>(psv[q], prv[q], c2v[q], c3v[q], c12v[q], hx, hy, hz, hl,
+                                                                     v, w, near);
+                            } else {
+                                eval4<DT, GUARD, SH, FORM_GENERAL, PL>(psv[q], prv[q], c2v[q], c3v[q], c12v[q], hx, hy, hz,
+                                                                       hl, v, w, near);
+                            }
+                            accumulate(s, v, w);
+                        }
                     }
-                    if (!(FLAGW ? ((cw >> (12 + s)) & 1u) : ((mk[s] >> bit) & 1u))) continue;
-                    const float c1sq = PL ? 0.0f : c1 * c1;
-                    const bool inner = (DT == FFT_DT_STABLE) &&
-                                       (FLAGW ? ((cw >> (16 + s)) & 1u) : ((ik[s] >> bit) & 1u));
-#define FFT_EVAL_SUB(INNER_V, PLANAR_V)                                                              \
-    float vv[NX_LANE], ww[NX_LANE];                                                                \
-    _Pragma("unroll") for (int t = 0; t < NX_LANE; ++t) {                                          \
-        const float ft = (float)t;                                                                 \
-        float is, ir, v, w;                                                                        \
-        if (DT == FFT_DT_FP64) {                                                                   \
-            const RowRec64 r64 = P.rec64[__float_as_int(C.z)];                                     \
-            const int b = (int)(cw & 0xffu);                                                       \
-            v = detour_v64(r64, P.org[0], P.org[1], P.org[2], P.h, TX + oxi + t,                   \
-                           TY + oyi + sub_dy<NSUB>(s), TZ + ozi + sub_dz<NSUB>(s), P.bc[b].U, w);  \
-            is = 1.0f;                                                                             \
-            ir = w;                                                                                \
-        } else {                                                                                   \
-            const float pst = (t == 0 ? psb : fmaf(ft, hx, psb));                                  \
-            const float prt = (t == 0 ? prb : fmaf(ft, hx, prb));                                  \
-            const float c3t = (t == 0 ? c3 : fmaf(ft, hy, c3));                                    \
-            float q2;                                                                              \
-            if (PLANAR_V) {                                                                        \
-                q2 = fmaf(c3t, c3t, c12sq);                                                        \
-            } else {                                                                               \
-                const float c2t = (t == 0 ? c2 : fmaf(-ft, hz, c2));                               \
-                q2 = fmaf(c2t, c2t, fmaf(c3t, c3t, c1sq));                                         \
-            }                                                                                      \
-            if (SH) {                                                                              \
-                v = detour_v<DT, GUARD, INNER_V, true>(pst, prt, q2, hl, is, ir);                  \
-                near |= (fabsf(v - 1.0f) < cutb);                                                  \
-                v = __saturatef(v);                                                                \
-            } else {                                                                               \
-                v = detour_v<DT, GUARD, INNER_V>(pst, prt, q2, hl, is, ir);                        \
-            }                                                                                      \
-        }                                                                                          \
-        if (MODE == MODE_COUNT) {                                                                  \
-            if ((vmask >> (4 * s + t)) & 1u) {                                                     \
-                ++cnt_eval;                                                                        \
-                if (v < 1.0f) ++cnt;                                                               \
-            }                                                                                      \
-            continue;                                                                              \
-        }                                                                                          \
-        if constexpr (PHI == PHI_TRIG) {                                                           \
-            vv[t] = v;                                                                             \
-            ww[t] = is * ir;                                                                       \
-            continue;                                                                              \
-        }                                                                                          \
-        const float val = phi_eval<PHI>(v, tb, nm1, nq, tab_addr, seg2_addr) * (is * ir);          \
-        if (MODE == MODE_JT) acc[s][t] = fmaf(val, W, acc[s][t]);                                  \
-        if (MODE == MODE_COV) acc[s][t] = fmaf(fabsf(val), W, acc[s][t]);                          \
-        if (MODE == MODE_JT4) {                                                                    \
-            _Pragma("unroll") for (int r = 0; r < 4; ++r) acc4[s & 1][t][r] = fmaf(val, Wr[r], acc4[s & 1][t][r]); \
-        }                                                                                          \
-        if (MODE == MODE_J4) {                                                                     \
-            _Pragma("unroll") for (int r = 0; r < 4; ++r) part4[r] = fmaf(val, mv4[s & 1][t][r], part4[r]); \
-        }                                                                                          \
-        if (MODE == MODE_J) part = fmaf(val, mv[s][t], part);                                      \
-        if (MODE == MODE_FROB) {                                                                   \
-            if ((vmask >> (4 * s + t)) & 1u) part = fmaf(val, val, part);                          \
-        }                                                                                          \
-    }                                                                                              \
-    if constexpr (PHI == PHI_TRIG && MODE != MODE_COUNT) {                                         \
-        float ph[NX_LANE];                                                                         \
-        phi_trig_n<NX_LANE>(vv, tb, nq, ph);                                                       \
-        _Pragma("unroll") for (int t = 0; t < NX_LANE; ++t) {                                      \
-            const float val = ph[t] * ww[t];                                                       \
-            if (MODE == MODE_JT) acc[s][t] = fmaf(val, W, acc[s][t]);                              \
-            if (MODE == MODE_COV) acc[s][t] = fmaf(fabsf(val), W, acc[s][t]);                      \
-            if (MODE == MODE_JT4) {                                                                \
-                _Pragma("unroll") for (int r = 0; r < 4; ++r) acc4[s & 1][t][r] = fmaf(val, Wr[r], acc4[s & 1][t][r]); \
-            }                                                                                      \
-            if (MODE == MODE_J4) {                                                                 \
-                _Pragma("unroll") for (int r = 0; r < 4; ++r) part4[r] = fmaf(val, mv4[s & 1][t][r], part4[r]); \
-            }                                                                                      \
-            if (MODE == MODE_J) part = fmaf(val, mv[s][t], part);                                  \
-            if (MODE == MODE_FROB) {                                                               \
-                if ((vmask >> (4 * s + t)) & 1u) part = fmaf(val, val, part);                      \
-            }                                                                                      \
-        }                                                                                          \
-    }
-                    const float c12sq = PL ? c12_planar : fmaf(c2, c2, c1sq);
-                    if (inner) {
-                        FFT_EVAL_SUB(true, PL)
-                    } else {
-                        FFT_EVAL_SUB(false, PL)
-                    }
-                }
                 };
-                if (SHARP && cutb > 0.0f) {
+                // single-column launches split a sharp geometry's rows by kind (launch_split)
+                const bool sharp_row = SHARP && (!BATCH || ((cw >> 8) & 1u));
+                if (SHARP && sharp_row) {
                     if (planar)
                         entry_body(std::true_type{}, std::integral_constant<bool, SHARP>{});
                     else
                         entry_body(std::false_type{}, std::integral_constant<bool, SHARP>{});
-                } else {
+                } else if (!SHARP || BATCH) {
                     if (planar)
                         entry_body(std::true_type{}, std::false_type{});
                     else
                         entry_body(std::false_type{}, std::false_type{});
                 }
-#undef FFT_EVAL_SUB
-                if (SHARP && DT != FFT_DT_FP64 && __any_sync(0xffffffffu, near)) {
+                if (SHARP && DT != FFT_DT_FP64 && __any_sync(0xffffffffu, near < CUT_BAND)) {
                     // FP64 re-decision of the voxels whose FP32 detour lies within CUT_BAND of
                     // the cut; d[k] is the change of this entry's term for voxel k = 4 s + t
                     float d[4 * NSUB];
-                    uint32_t inner_bits = (cw >> 16) & 15u;
-                    if (!FLAGW) {
-                        inner_bits = 0u;
-#pragma unroll
-                        for (int s = 0; s < NSUB; ++s) inner_bits |= ((ik[s] >> bit) & 1u) << s;
-                    }
-                    if (near)
-                        sharp_fix<MODE, DT, GUARD, PHI, NSUB>(P, A, B, C, Xl, Yl, Zl, planar, inner_bits, cutb, tb, nm1,
-                                                              nq, tab_addr, seg2_addr, TX + oxi, TY + oyi, TZ + ozi, d);
+                    if (near < CUT_BAND)
+                        sharp_fix<MODE, DT, GUARD, PHI, NSUB>(P, A, B, C, P.tile_rows[e0 + bit], Xl, Yl, Zl, at,
+                                                              TX + oxi, TY + oyi, TZ + ozi, d);
 #pragma unroll
                     for (int s = 0; s < NSUB; ++s) {
 #pragma unroll
-                        for (int t = 0; t < NX_LANE; ++t) {
-                            const float dk = near ? d[4 * s + t] : 0.0f;
-                            if (dk == 0.0f) continue;
-                            const bool valid = (vmask >> (4 * s + t)) & 1u;
-                            if (MODE == MODE_COUNT && valid) cnt += (dk > 0.0f) ? 1ull : ~0ull;
-                            if (MODE == MODE_JT || MODE == MODE_COV) acc[s][t] = fmaf(dk, W, acc[s][t]);
-                            if (MODE == MODE_J) part = fmaf(dk, mv[s][t], part);
+                        for (int j = 0; j < 2; ++j) {
+                            const float d0 = near < CUT_BAND ? d[4 * s + 2 * j] : 0.0f;
+                            const float d1 = near < CUT_BAND ? d[4 * s + 2 * j + 1] : 0.0f;
+                            if (d0 == 0.0f && d1 == 0.0f) continue;
+                            const f2 dk = pk(d0, d1);
+                            const bool ok0 = (vmask >> (4 * s + 2 * j)) & 1u, ok1 = (vmask >> (4 * s + 2 * j + 1)) & 1u;
+                            if (MODE == MODE_COUNT) n_in += (ok0 ? (int)d0 : 0) + (ok1 ? (int)d1 : 0);
+                            if (MODE == MODE_JT || MODE == MODE_COV) acc[s][j] = fma2(dk, pk1(W), acc[s][j]);
+                            if (MODE == MODE_J) part = fma2(dk, mv[s][j], part);
                             if (MODE == MODE_JT4) {
 #pragma unroll
-                                for (int r = 0; r < 4; ++r) acc4[s & 1][t][r] = fmaf(dk, Wr[r], acc4[s & 1][t][r]);
+                                for (int r = 0; r < 4; ++r) acc4[s & 1][j][r] = fma2(dk, pk1(Wr[r]), acc4[s & 1][j][r]);
                             }
                             if (MODE == MODE_J4) {
 #pragma unroll
-                                for (int r = 0; r < 4; ++r) part4[r] = fmaf(dk, mv4[s & 1][t][r], part4[r]);
+                                for (int r = 0; r < 4; ++r) part4[r] = fma2(dk, mv4[s & 1][j][r], part4[r]);
                             }
-                            if (MODE == MODE_FROB && valid) part += dk;
+                            if (MODE == MODE_FROB) fsum += (ok0 ? d0 : 0.0f) + (ok1 ? d1 : 0.0f);
                         }
                     }
+                }
+                if (MODE == MODE_COUNT) {
+                    cnt += n_in & 0xffffu;
+                    cnt_eval += n_in >> 16;
                 }
                 if (MODE == MODE_J) {
                     // Fold the row's 32 lane partials to 8 (lanes 0-7 then hold distinct sums)
                     // and park them in the row's own staged record, which every lane has read
                     // by now; the row's lane adds the 8 in a fixed order after the chunk.
-                    part += __shfl_xor_sync(0xffffffffu, part, 16);
-                    part += __shfl_xor_sync(0xffffffffu, part, 8);
+                    const float2 p2 = up(part);
+                    float ps = p2.x + p2.y;
+                    ps += __shfl_xor_sync(0xffffffffu, ps, 16);
+                    ps += __shfl_xor_sync(0xffffffffu, ps, 8);
                     __syncwarp();
-                    if (lane < 8) reinterpret_cast<float*>(stg + bit * SR)[lane] = part;
+                    if (lane < 8) reinterpret_cast<float*>(stg + bit * SR)[lane] = ps;
                 }
                 if (MODE == MODE_J4) {
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
-                        const float pr4 = warp_sum(part4[r]);
+                        const float2 p2 = up(part4[r]);
+                        const float pr4 = warp_sum(p2.x + p2.y);
                         if (lane == bit) mypart4[r] = pr4 * W;
                     }
                 }
-                if (MODE == MODE_FROB) dacc += (double)part * (double)W * (double)W;
+                if (MODE == MODE_FROB) dacc += (double)fsum * (double)W * (double)W;
             }
             if (MODE == MODE_J) {
                 __syncwarp();
@@ -655,16 +844,18 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
 #pragma unroll
             for (int s = 0; s < NSUB; ++s) {
                 const int dy = sub_dy<NSUB>(s), dz = sub_dz<NSUB>(s);
+                const float2 a0 = up(acc[s][0]), a1 = up(acc[s][1]);
+                const float av[NX_LANE] = {a0.x, a0.y, a1.x, a1.y};
                 if (item.slot < 0) {
 #pragma unroll
                     for (int t = 0; t < NX_LANE; ++t)
                         if ((vm >> (4 * s + t)) & 1u)
-                            P.vout[vbase + ((int64_t)dz * P.ny + dy) * P.nx + t] = acc[s][t];
+                            P.vout[vbase + ((int64_t)dz * P.ny + dy) * P.nx + t] = av[t];
                 } else {
                     // local index inside the tile: (z * 16 + y) * 16 + x
                     const int loc = (((ozi + dz) * TILE_Y) + oyi + dy) * TILE_X + oxi;
-                    float4 v4 = make_float4(acc[s][0], acc[s][1], acc[s][2], acc[s][3]);
-                    *reinterpret_cast<float4*>(P.gpart + (int64_t)item.slot * TILE_VOX + loc) = v4;
+                    *reinterpret_cast<float4*>(P.gpart + (int64_t)item.slot * TILE_VOX + loc) =
+                        make_float4(av[0], av[1], av[2], av[3]);
                 }
             }
         }
@@ -676,14 +867,16 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const int loc = ((ozi * TILE_Y) + oyi + 4 * s) * TILE_X + oxi;
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
+                    const float2 a0 = up(acc4[s][0][r]), a1 = up(acc4[s][1][r]);
+                    const float av[NX_LANE] = {a0.x, a0.y, a1.x, a1.y};
                     if (item.slot < 0) {
 #pragma unroll
                         for (int t = 0; t < NX_LANE; ++t)
                             if ((vm >> (4 * s + t)) & 1u)
-                                P.vout[(int64_t)r * P.nvox + vbase + (int64_t)(4 * s) * P.nx + t] = acc4[s][t][r];
+                                P.vout[(int64_t)r * P.nvox + vbase + (int64_t)(4 * s) * P.nx + t] = av[t];
                     } else {
-                        float4 v4 = make_float4(acc4[s][0][r], acc4[s][1][r], acc4[s][2][r], acc4[s][3][r]);
-                        *reinterpret_cast<float4*>(P.gpart + ((int64_t)item.slot * 4 + r) * TILE_VOX + loc) = v4;
+                        *reinterpret_cast<float4*>(P.gpart + ((int64_t)item.slot * 4 + r) * TILE_VOX + loc) =
+                            make_float4(av[0], av[1], av[2], av[3]);
                     }
                 }
             }

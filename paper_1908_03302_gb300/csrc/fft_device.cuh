@@ -46,6 +46,57 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// ---- packed pairs of floats (fma / mul / add .f32x2 of sm_100 and later). One packed
+// instruction does two FP32 operations in one issue slot, each rounded like its scalar form.
+// The FP32 pipe takes it at the scalar rate per operation (measured on GB300: 2.07 cycles a
+// packed FMA against 1.02 a scalar one), so packing frees issue slots, not FP32 lanes. Operands
+// that broadcast one float to both halves, or negate, cost nothing extra (instruction counts).
+typedef unsigned long long f2;
+
+__device__ __forceinline__ f2 pk(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ f2 pk1(float x) { return pk(x, x); }
+__device__ __forceinline__ float2 up(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 neg2(f2 v) {
+    const float2 a = up(v);
+    return pk(-a.x, -a.y);
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 fma2_rd(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rm.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 rsqrt2(f2 v) {
+    const float2 a = up(v);
+    return pk(rsqrt_approx(a.x), rsqrt_approx(a.y));
+}
+__device__ __forceinline__ f2 rcp2(f2 v) {
+    const float2 a = up(v);
+    return pk(rcp_approx(a.x), rcp_approx(a.y));
+}
+
 // Conservative test: may the row's support {R < 1} (band units) reach a box of voxel
 // centres with centre c and half extents hx, hy, hz? R(x) = |x - xs| + |x - xr| - 2 hl is
 // convex, so every tangent plane lies below it: R(x) >= R(x1) + grad R(x1) . (x - x1), whose
@@ -185,6 +236,40 @@ __device__ __forceinline__ float phi_lookup(float v, uint32_t tb, float nm1) {
     return fmaf(v, T.y, T.x);
 }
 
+// The same lookup for the J / J^T kernels, which add MAGIC2 = 2 instead: its ulp is 2^-22, so
+// t = v nm1 2^-22 + (2 + first 2^-22), rounded down, has the bit pattern 0x40000000 + first + k
+// (first: the band's first entry), and the pattern shifted left by 3 is the byte offset 8 (first
+// + k) without a subtraction. `scale` is nm1 2^-22, `base` the tables' shared address.
+constexpr float MAGIC2 = 2.0f;
+constexpr float MAGIC2_ULP = 2.384185791015625e-7f;   // 2^-22
+__device__ __forceinline__ float2 lds_f2_table(uint32_t base, float t) {
+    float2 v;
+    asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(base + (__float_as_uint(t) << 3)));
+    return v;
+}
+__device__ __forceinline__ float phi_lookup_at(float v, float magic, float scale, uint32_t base) {
+    const float2 T = lds_f2_table(base, __fmaf_rd(v, scale, magic));
+    return fmaf(v, T.y, T.x);
+}
+
+// ---- the detour deep inside a pair's sphere
+// Let X = (x - xs).(x - xr) = ps pr + q2 and G = R_xs R_xr = sqrt(X^2 + L^2 q2), in any unit.
+// Inside the sphere whose diameter is the pair X < 0, and with y = q2 / (G - X)
+//   (R_xs + R_xr)^2 = L^2 (1 + 2 y),  so  R = L (sqrt(1 + 2 y) - 1) = L y P(y),
+// every term positive (no cancellation near the ray). One reciprocal square root (which is also
+// the geometric factor 1 / (R_xs R_xr)) and one reciprocal take the place of the general form's
+// two and one: the special-function unit issues 1 lane in 8 cycles a warp, so that the
+// general form's three cap it at 24 cycles per evaluation.
+// P(y) = (sqrt(1 + 2 y) - 1) / y as 1 + DEEP_C2 y + .. + DEEP_C5 y^4: a relative minimax fit
+// (Lawson's weighted least squares) on 0 <= y <= (l + 1/2) / l^2 for l = L / U = DEEP_MIN_L, the
+// range of the support of rows at least that long; error 1.1e-8 there, and below 1e-9 for l >= 20. y P(y)
+// is increasing for all y >= 0, so voxels beyond the cut stay beyond it.
+constexpr float DEEP_MIN_L = 12.0f;
+constexpr float DEEP_C2 = -0.4999963045120239f, DEEP_C3 = 0.499575674533844f, DEEP_C4 = -0.6096726655960083f,
+                DEEP_C5 = 0.6489434838294983f;
+// Voxel steps by which a sub-brick keeps off the sphere (there X changes sign).
+constexpr float DEEP_MARGIN = 2.0f;
+
 // Phi(v) from the band's sine series (Sec. II-C stored form): Phi = sum_{k=1..n} a_k sin(k x),
 // x = theta v with theta = dw dt_max <= pi, and 0 for v <= 0 or v >= 1 (truncation).
 // Block at shared address tb: theta, 3 pad floats, then a_1 .. a_{4 nq} (zeros past n).
@@ -279,8 +364,6 @@ __device__ __forceinline__ void phi_trig_n(const float* v, uint32_t tb, int nq, 
 // of the 20-term recurrence (ring256 J^T 15.81 -> 4.54 ms, error against 64 bits 5.9e-7 -> 3.8e-7). t = v n 2^-22 + magic, magic = 2 + (first segment of the band)
 // 2^-22, rounded down has the bits 0x40000000 + segment, whose shifts by 3 and 2 are the byte
 // offsets; t - magic = k 2^-22 exactly. The entries past the segments are zeros: the cut-off.
-constexpr float MAGIC2 = 2.0f;
-constexpr float MAGIC2_ULP = 2.384185791015625e-7f;   // 2^-22
 __device__ __forceinline__ float phi_seg(float v, float magic, float scale, uint32_t base01, uint32_t base2) {
     const float t = __fmaf_rd(v, scale, magic);
     const float u = fmaf(v, scale, magic - t);
