@@ -82,8 +82,8 @@ template <int NCOL>
 __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t* __restrict__ slot0,
                                                                    const int32_t* __restrict__ nslot,
                                                                    const float* __restrict__ gpart, int nx, int ny,
-                                                                   int nz, int tiles_x, int tiles_y,
-                                                                   float* __restrict__ g) {
+                                                                   int nz, int z_lo, int z_end, int mirror,
+                                                                   int tiles_x, int tiles_y, float* __restrict__ g) {
     __shared__ float4 sh[RED_WARPS][32];
     constexpr int PER_TILE = TILE_VOX / (4 * 32);   // CTAs per tile
     const int T = blockIdx.x / PER_TILE, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
     const int iz = TILE_Z * (T / (tiles_x * tiles_y)) + loc / (TILE_X * TILE_Y);
     const int64_t V = (int64_t)nx * ny * nz;
     const int64_t v = ((int64_t)iz * ny + iy) * nx + ix;
-    const bool inside = iy < ny && iz < nz && ix < nx;
+    const bool inside = iy < ny && iz >= z_lo && iz < z_end && ix < nx;
+    const int64_t mo = (int64_t)mirror_step(mirror, iz, nz) * ny * nx;   // to the mirrored layer (0: none)
     const int ns = (s0 == -2 || !inside) ? 0 : nslot[T];
     for (int r = 0; r < NCOL; ++r) {
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, low[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -126,7 +127,10 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
             double s = 0.0;
 #pragma unroll
             for (int k = 0; k < RED_WARPS; ++k) s += (double)reinterpret_cast<const float*>(&sh[k][lane])[w];
-            if (inside && ix + w < nx) g[(int64_t)r * V + v + w] = (float)s;
+            if (inside && ix + w < nx) {
+                g[(int64_t)r * V + v + w] = (float)s;
+                if (mo != 0) g[(int64_t)r * V + v + mo + w] = (float)s;
+            }
         }
         if (NCOL > 1) __syncthreads();
     }
@@ -152,6 +156,9 @@ static ApplyParams make_params(fft_geom g) {
     P.nx = g->grid.nx;
     P.ny = g->grid.ny;
     P.nz = g->grid.nz;
+    P.z_lo = g->z_lo;
+    P.z_end = g->z_end;
+    P.mirror = g->mirror;
     for (int a = 0; a < 3; ++a) P.org[a] = g->grid.origin[a];
     P.h = g->grid.h;
     P.vin = nullptr;
@@ -310,7 +317,8 @@ template <int NCOL>
 static fft_status launch_jt_reduce(fft_geom g, const float* gpart, float* gout, cudaStream_t st) {
     if (g->n_tiles == 0) return FFT_OK;
     jt_reduce_kernel<NCOL><<<(unsigned)(g->n_tiles * (TILE_VOX / 128)), 32 * RED_WARPS, 0, st>>>(
-        g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->tiles[0], g->tiles[1], gout);
+        g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->z_lo, g->z_end, g->mirror, g->tiles[0],
+        g->tiles[1], gout);
     FFT_CUDA(cudaGetLastError());
     return FFT_OK;
 }

@@ -60,6 +60,7 @@ struct ApplyParams {
     int32_t* counter;
     int tiles_x, tiles_y;
     int nx, ny, nz;
+    int z_lo, z_end, mirror;   // layers to evaluate, mirror plane (fft_geom_s)
     double org[3];
     double h;
     const float* vin;        // J: m [V]; J^T: d [M]
@@ -490,7 +491,8 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
             uint32_t vm = 0;
 #pragma unroll
             for (int s = 0; s < NSUB; ++s) {
-                if (TZ + ozi + sub_dz<NSUB>(s) < P.nz && TY + oyi + sub_dy<NSUB>(s) < P.ny) {
+                const int z = TZ + ozi + sub_dz<NSUB>(s);
+                if (z >= P.z_lo && z < P.z_end && TY + oyi + sub_dy<NSUB>(s) < P.ny) {
 #pragma unroll
                     for (int t = 0; t < NX_LANE; ++t)
                         if (TX + oxi + t < P.nx) vm |= 1u << (4 * s + t);
@@ -501,12 +503,24 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
         uint32_t sub_ok = 0;
 #pragma unroll
         for (int s = 0; s < NSUB; ++s)
-            if (TX + 8 * wx < P.nx && TY + 8 * wy + sub_dy<NSUB>(s) < P.ny && TZ + 4 * wz + sub_dz<NSUB>(s) < P.nz)
+            if (TX + 8 * wx < P.nx && TY + 8 * wy + sub_dy<NSUB>(s) < P.ny && TZ + 4 * wz + sub_dz<NSUB>(s) < P.z_end &&
+                TZ + 4 * wz + sub_dz<NSUB>(s) + 3 >= P.z_lo)
                 sub_ok |= 1u << s;
         // the gather modes need the mask only for their stores: recomputed there
         constexpr bool VM_LIVE = !(MODE == MODE_JT || MODE == MODE_COV || MODE == MODE_JT4);
         const uint32_t vmask = VM_LIVE ? lane_vmask() : 0u;
         const int64_t vbase = ((int64_t)(TZ + ozi) * P.ny + TY + oyi) * P.nx + TX + oxi;
+        // voxels from this lane's run in sub-brick s to its mirror image (0: none)
+        auto mirror_off = [&](int s) {
+            return (int64_t)mirror_step(P.mirror, TZ + ozi + sub_dz<NSUB>(s), P.nz) * P.ny * P.nx;
+        };
+        // the count and the Frobenius norm take a mirrored run twice (bit s)
+        uint32_t twice = 0;
+        if (MODE == MODE_COUNT || MODE == MODE_FROB) {
+#pragma unroll
+            for (int s = 0; s < NSUB; ++s)
+                if (mirror_off(s) != 0) twice |= 1u << s;
+        }
 
         // accumulators (J^T) or model values (J) of the lane's voxels, as pairs (0, 1), (2, 3) of
         // each run
@@ -521,8 +535,12 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const int64_t vo = vbase + ((int64_t)sub_dz<NSUB>(s) * P.ny + sub_dy<NSUB>(s)) * P.nx + 2 * j;
                 const bool ok0 = (vmask >> (4 * s + 2 * j)) & 1u, ok1 = (vmask >> (4 * s + 2 * j + 1)) & 1u;
                 acc[s][j] = mv[s][j] = 0ull;
-                if (MODE == MODE_J)
+                if (MODE == MODE_J) {
                     mv[s][j] = pk(ok0 ? __ldg(P.vin + vo) : 0.0f, ok1 ? __ldg(P.vin + vo + 1) : 0.0f);
+                    if (const int64_t mo = mirror_off(s))
+                        mv[s][j] = add2(mv[s][j], pk(ok0 ? __ldg(P.vin + vo + mo) : 0.0f,
+                                                     ok1 ? __ldg(P.vin + vo + mo + 1) : 0.0f));
+                }
                 if (BATCH && s < 2) {
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
@@ -530,6 +548,9 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         if (MODE == MODE_J4) {
                             const float* mr = P.vin + (int64_t)r * P.nvox + vo;
                             mv4[s & 1][j][r] = pk(ok0 ? __ldg(mr) : 0.0f, ok1 ? __ldg(mr + 1) : 0.0f);
+                            if (const int64_t mo = mirror_off(s))
+                                mv4[s & 1][j][r] = add2(mv4[s & 1][j][r], pk(ok0 ? __ldg(mr + mo) : 0.0f,
+                                                                             ok1 ? __ldg(mr + mo + 1) : 0.0f));
                         }
                     }
                 }
@@ -584,7 +605,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 }
                 const uint32_t od = okb & dpb, both = ((od & 3u) == 3u ? 1u : 0u) | ((od & 12u) == 12u ? 2u : 0u);
                 stg[lane * SR + 0] = base;
-                stg[lane * SR + 1] = make_float4(hb * ex, hb * ey, hb * ez, base3);
+                stg[lane * SR + 1] = make_float4(r.c.x, r.c.y, r.c.z, base3);
                 // planar pair (both transducers at one z): stepping along x changes only c3
                 const int planar = (ez == 0.0f) ? 1 : 0;
                 // third word: the band's place (the magic number of its lookups; PHI_TRIG: the
@@ -627,7 +648,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         const uint32_t vm = (vmask >> (4 * s)) & 15u;
                         const uint32_t in = (va.x < 1.0f ? 1u : 0u) | (va.y < 1.0f ? 2u : 0u) | (vb.x < 1.0f ? 4u : 0u) |
                                             (vb.y < 1.0f ? 8u : 0u);
-                        n_in += __popc(in & vm) | (__popc(vm) << 16);
+                        n_in += (__popc(in & vm) | (__popc(vm) << 16)) << ((twice >> s) & 1u);
                         return;
                     }
                     float ph[NX_LANE];
@@ -668,8 +689,9 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         }
                         if (MODE == MODE_FROB) {
                             const float2 x = up(val);
-                            if ((vmask >> (4 * s + 2 * j)) & 1u) fsum = fmaf(x.x, x.x, fsum);
-                            if ((vmask >> (4 * s + 2 * j + 1)) & 1u) fsum = fmaf(x.y, x.y, fsum);
+                            const float f = ((twice >> s) & 1u) ? 2.0f : 1.0f;
+                            if ((vmask >> (4 * s + 2 * j)) & 1u) fsum = fmaf(f * x.x, x.x, fsum);
+                            if ((vmask >> (4 * s + 2 * j + 1)) & 1u) fsum = fmaf(f * x.y, x.y, fsum);
                         }
                     }
                 };
@@ -781,7 +803,8 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                             if (d0 == 0.0f && d1 == 0.0f) continue;
                             const f2 dk = pk(d0, d1);
                             const bool ok0 = (vmask >> (4 * s + 2 * j)) & 1u, ok1 = (vmask >> (4 * s + 2 * j + 1)) & 1u;
-                            if (MODE == MODE_COUNT) n_in += (ok0 ? (int)d0 : 0) + (ok1 ? (int)d1 : 0);
+                            const int f = 1 + (int)((twice >> s) & 1u);   // count, Frobenius
+                            if (MODE == MODE_COUNT) n_in += f * ((ok0 ? (int)d0 : 0) + (ok1 ? (int)d1 : 0));
                             if (MODE == MODE_JT || MODE == MODE_COV) acc[s][j] = fma2(dk, pk1(W), acc[s][j]);
                             if (MODE == MODE_J) part = fma2(dk, mv[s][j], part);
                             if (MODE == MODE_JT4) {
@@ -792,7 +815,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
 #pragma unroll
                                 for (int r = 0; r < 4; ++r) part4[r] = fma2(dk, mv4[s & 1][j][r], part4[r]);
                             }
-                            if (MODE == MODE_FROB) fsum += (ok0 ? d0 : 0.0f) + (ok1 ? d1 : 0.0f);
+                            if (MODE == MODE_FROB) fsum += (float)f * ((ok0 ? d0 : 0.0f) + (ok1 ? d1 : 0.0f));
                         }
                     }
                 }
@@ -847,10 +870,14 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const float2 a0 = up(acc[s][0]), a1 = up(acc[s][1]);
                 const float av[NX_LANE] = {a0.x, a0.y, a1.x, a1.y};
                 if (item.slot < 0) {
+                    const int64_t mo = mirror_off(s);
 #pragma unroll
                     for (int t = 0; t < NX_LANE; ++t)
-                        if ((vm >> (4 * s + t)) & 1u)
-                            P.vout[vbase + ((int64_t)dz * P.ny + dy) * P.nx + t] = av[t];
+                        if ((vm >> (4 * s + t)) & 1u) {
+                            float* o = P.vout + vbase + ((int64_t)dz * P.ny + dy) * P.nx + t;
+                            o[0] = av[t];
+                            if (mo != 0) o[mo] = av[t];
+                        }
                 } else {
                     // local index inside the tile: (z * 16 + y) * 16 + x
                     const int loc = (((ozi + dz) * TILE_Y) + oyi + dy) * TILE_X + oxi;
@@ -870,10 +897,14 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     const float2 a0 = up(acc4[s][0][r]), a1 = up(acc4[s][1][r]);
                     const float av[NX_LANE] = {a0.x, a0.y, a1.x, a1.y};
                     if (item.slot < 0) {
+                        const int64_t mo = mirror_off(s);
 #pragma unroll
                         for (int t = 0; t < NX_LANE; ++t)
-                            if ((vm >> (4 * s + t)) & 1u)
-                                P.vout[(int64_t)r * P.nvox + vbase + (int64_t)(4 * s) * P.nx + t] = av[t];
+                            if ((vm >> (4 * s + t)) & 1u) {
+                                float* o = P.vout + (int64_t)r * P.nvox + vbase + (int64_t)(4 * s) * P.nx + t;
+                                o[0] = av[t];
+                                if (mo != 0) o[mo] = av[t];
+                            }
                     } else {
                         *reinterpret_cast<float4*>(P.gpart + ((int64_t)item.slot * 4 + r) * TILE_VOX + loc) =
                             make_float4(av[0], av[1], av[2], av[3]);

@@ -62,6 +62,7 @@ struct RowRec {
     float4 a;   // (o_x, o_y, o_z, hl): pair midpoint, half pair length
     float4 b;   // (e_x, e_y, e_z, C): unit axis, C = -L h^3 / (2 pi c0^3 U_b^2) (SI seconds per m/s per
                 // unit Phi / (R_xs R_xr) in band units)
+    float4 c;   // (h e_x, h e_y, h e_z, 0): voxel step along the axis in band units, rounded once
 };
 
 // Per-row FP64 record used by the FP64 detour mode (SI metres).
@@ -138,6 +139,11 @@ struct fft_geom_s {
     fftgb::RowRec64* rec64 = nullptr;    // [M] (FP64 mode only)
     int32_t* row_band = nullptr;         // [M]
     float2* tab = nullptr;               // [n_bands * n_tab] (Phi_k, Phi_{k+1} - Phi_k)
+    // Mirror plane (find_mirror): with every transducer in one plane z = z0 that is a mirror plane of
+    // the voxel lattice, layers k and mirror - k see the same entries of J; items then cover only
+    // the layers [z_lo, z_end) and the products serve the mirrored layer of each from the same
+    // evaluation. Without one: all layers, mirror = -1. (The tile lists always cover the grid.)
+    int32_t z_lo = 0, z_end = 0, mirror = -1;
     int32_t tiles[3];
     int64_t n_tiles = 0;
     int64_t E = 0;                       // entries
@@ -217,6 +223,12 @@ int psf_tc_max_spikes(fft_geom g, int n_groups);
 fft_status launch_psf_tc(fft_geom g, const int64_t* d_off, const uint32_t* d_ent, const uint8_t* grp, int n_groups,
                          const uint32_t* gmask, int n_sub, int n_spike, int k0, int nk, float* out, cudaStream_t st);
 int64_t ceil_div(int64_t a, int64_t b);
+
+// Layers from layer z to its mirror image, 0 if it has none inside the grid (or is its own).
+__host__ __device__ __forceinline__ int mirror_step(int mirror, int z, int nz) {
+    const int zm = mirror - z;
+    return (mirror < 0 || zm < 0 || zm >= nz) ? 0 : zm - z;
+}
 // Resolve (and so load) the no-allocation PSF's static scratch on device `dev` (current).
 fft_status noalloc_prepare(int dev);
 }  // namespace fftgb
