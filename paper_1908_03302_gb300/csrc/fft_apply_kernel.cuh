@@ -621,7 +621,6 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
             uint32_t mm = __ballot_sync(0xffffffffu, okb != 0u);
             __syncwarp();
             float mypart = 0.0f;
-            float mypart4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
             while (mm) {
                 const int bit = __ffs(mm) - 1;
                 mm &= mm - 1;
@@ -700,8 +699,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 // along the lane's voxels or between sub-bricks at one z, and p does not change
                 // in z). The lane base (sub-brick 0, t = 0) is a small offset added to the tile
                 // origin's FP64-derived values.
-                // SH: the near-cut checks, only for rows of a band whose Phi does not vanish at
-                // the cut (the four-column launches take a sharp geometry's other rows too).
+                // SH: the near-cut checks, for rows of a band whose Phi does not vanish at the cut.
                 auto entry_body = [&](auto planar_tag, auto sharp_tag) {
                     constexpr bool PL = decltype(planar_tag)::value;
                     constexpr bool SH = decltype(sharp_tag)::value;
@@ -774,19 +772,11 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         }
                     }
                 };
-                // single-column launches split a sharp geometry's rows by kind (launch_split)
-                const bool sharp_row = SHARP && (!BATCH || ((cw >> 8) & 1u));
-                if (SHARP && sharp_row) {
-                    if (planar)
-                        entry_body(std::true_type{}, std::integral_constant<bool, SHARP>{});
-                    else
-                        entry_body(std::false_type{}, std::integral_constant<bool, SHARP>{});
-                } else if (!SHARP || BATCH) {
-                    if (planar)
-                        entry_body(std::true_type{}, std::false_type{});
-                    else
-                        entry_body(std::false_type{}, std::false_type{});
-                }
+                // (a launch's rows are all of one kind: launch_split)
+                if (planar)
+                    entry_body(std::true_type{}, std::integral_constant<bool, SHARP>{});
+                else
+                    entry_body(std::false_type{}, std::integral_constant<bool, SHARP>{});
                 if (SHARP && DT != FFT_DT_FP64 && __any_sync(0xffffffffu, near < CUT_BAND)) {
                     // FP64 re-decision of the voxels whose FP32 detour lies within CUT_BAND of
                     // the cut; d[k] is the change of this entry's term for voxel k = 4 s + t
@@ -835,12 +825,24 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     if (lane < 8) reinterpret_cast<float*>(stg + bit * SR)[lane] = ps;
                 }
                 if (MODE == MODE_J4) {
+                    // Transposing fold: each exchange halves the columns a lane carries (2 + 1
+                    // shuffles), three more add the eight lanes that hold one column; lane 8 r then
+                    // parks column r in the row's consumed record: 6 shuffles instead of the 20 of four
+                    // butterflies (ring256, a block of 8 columns: J and J^T 10.93 -> 10.54 ms).
+                    float q[4];
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
                         const float2 p2 = up(part4[r]);
-                        const float pr4 = warp_sum(p2.x + p2.y);
-                        if (lane == bit) mypart4[r] = pr4 * W;
+                        q[r] = p2.x + p2.y;
                     }
+                    const bool hi = lane & 16, odd = lane & 8;
+                    const float a0 = (hi ? q[2] : q[0]) + __shfl_xor_sync(0xffffffffu, hi ? q[0] : q[2], 16);
+                    const float a1 = (hi ? q[3] : q[1]) + __shfl_xor_sync(0xffffffffu, hi ? q[1] : q[3], 16);
+                    float ps = (odd ? a1 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+                    __syncwarp();
+                    if ((lane & 7) == 0) reinterpret_cast<float*>(stg + bit * SR)[lane >> 3] = ps;
                 }
                 if (MODE == MODE_FROB) dacc += (double)fsum * (double)W * (double)W;
             }
@@ -856,9 +858,18 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     P.vout[e * NREG + region] = mypart;
                 }
             }
-            if (MODE == MODE_J4 && have)
-                *reinterpret_cast<float4*>(P.vout + (e * NREG + region) * 4) =
-                    make_float4(mypart4[0], mypart4[1], mypart4[2], mypart4[3]);
+            if (MODE == MODE_J4) {
+                __syncwarp();
+                if (have) {
+                    float4 r0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if (okb) {
+                        r0 = stg[lane * SR + 0];
+                        const float Wl = stg[lane * SR + 2].x;
+                        r0 = make_float4(r0.x * Wl, r0.y * Wl, r0.z * Wl, r0.w * Wl);
+                    }
+                    *reinterpret_cast<float4*>(P.vout + (e * NREG + region) * 4) = r0;
+                }
+            }
             __syncwarp();
         }
 
@@ -1029,29 +1040,20 @@ inline fft_status launch_mode_impl(fft_geom g, const ApplyParams& P, cudaStream_
 // The four-column modes (stable detour only).
 template <int MODE>
 inline fft_status launch_batch_impl(fft_geom g, const ApplyParams& P, cudaStream_t st) {
-    const size_t smem = apply_smem(g);
-    const int ctas = g->apply_ctas;
-    FFT_CUDA(cudaMemsetAsync(g->counter, 0, sizeof(int32_t), st));
+    FFT_CUDA(cudaMemsetAsync(g->counter, 0, 2 * sizeof(int32_t), st));
     if (g->n_items == 0) return FFT_OK;
-#define FFT_LAUNCH(GV, SV, PV) apply_kernel<MODE, FFT_DT_STABLE, GV, SV, PV><<<ctas, APPLY_THREADS, smem, st>>>(P)
-#define FFT_LAUNCH_GS(PV)                                           \
-    do {                                                            \
-        if (g->guard) {                                             \
-            if (g->sharp) FFT_LAUNCH(true, true, PV);               \
-            else FFT_LAUNCH(true, false, PV);                       \
-        } else {                                                    \
-            if (g->sharp) FFT_LAUNCH(false, true, PV);              \
-            else FFT_LAUNCH(false, false, PV);                      \
-        }                                                           \
+#define FFT_LAUNCH_G(PV)                                                          \
+    do {                                                                          \
+        if (g->guard) launch_split<MODE, FFT_DT_STABLE, true, PV>(g, P, st);      \
+        else launch_split<MODE, FFT_DT_STABLE, false, PV>(g, P, st);              \
     } while (0)
     if (g->phi_eval == PHI_TRIG)
-        FFT_LAUNCH_GS(PHI_TRIG);
+        FFT_LAUNCH_G(PHI_TRIG);
     else if (g->phi_eval == PHI_SEG)
-        FFT_LAUNCH_GS(PHI_SEG);
+        FFT_LAUNCH_G(PHI_SEG);
     else
-        FFT_LAUNCH_GS(PHI_TABLE);
-#undef FFT_LAUNCH_GS
-#undef FFT_LAUNCH
+        FFT_LAUNCH_G(PHI_TABLE);
+#undef FFT_LAUNCH_G
     FFT_CUDA(cudaGetLastError());
     return FFT_OK;
 }
