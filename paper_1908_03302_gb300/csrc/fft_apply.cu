@@ -159,6 +159,7 @@ static ApplyParams make_params(fft_geom g) {
     P.z_lo = g->z_lo;
     P.z_end = g->z_end;
     P.mirror = g->mirror;
+    P.zw = g->zw;
     for (int a = 0; a < 3; ++a) P.org[a] = g->grid.origin[a];
     P.h = g->grid.h;
     P.vin = nullptr;
@@ -290,6 +291,7 @@ static fft_status batch_scratch(fft_geom g) {
 // d[:, c] = J m[:, c] for n columns: groups of four with the batch kernel on stable-detour
 // geometries, single columns otherwise.
 fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st) {
+    if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_J(g, m, n, d, st);
     int c = 0;
     if (g->dt_mode == FFT_DT_STABLE && n >= 4) {
         fft_status rc = batch_scratch(g);
@@ -325,6 +327,7 @@ static fft_status launch_jt_reduce(fft_geom g, const float* gpart, float* gout, 
 
 // g[:, c] = J^T d[:, c] for n columns (groups of four as above).
 fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st) {
+    if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_JT(g, din, n, gout, st);
     int c = 0;
     if (g->dt_mode == FFT_DT_STABLE && n >= 4) {
         fft_status rc = batch_scratch(g);
@@ -346,6 +349,7 @@ fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cud
 }
 
 fft_status launch_J(fft_geom g, const float* m, float* d, cudaStream_t st) {
+    if (!g->stk.empty()) return stack_J(g, m, 1, d, st);
     ApplyParams P = make_params(g);
     P.vin = m;
     P.vout = g->jpart;
@@ -360,6 +364,7 @@ fft_status launch_J(fft_geom g, const float* m, float* d, cudaStream_t st) {
 }
 
 fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st) {
+    if (!g->stk.empty()) return stack_JT(g, din, 1, gout, st);
     ApplyParams P = make_params(g);
     P.vin = din;
     P.vout = gout;
@@ -380,6 +385,17 @@ fft_status launch_cov(fft_geom g, const float* w, float* cov, cudaStream_t st) {
 
 // In-support evaluations (dt < dt_max) of one apply and evaluations actually performed.
 fft_status count_support(fft_geom g, int64_t* support, int64_t* evaluated) {
+    if (!g->stk.empty()) {   // each class's operator counts its slices through zw
+        *support = *evaluated = 0;
+        for (StackClass& c : g->stk) {
+            int64_t s = 0, e = 0;
+            const fft_status rc = count_support(c.sub, &s, &e);
+            if (rc != FFT_OK) return rc;
+            *support += s;
+            *evaluated += e;
+        }
+        return FFT_OK;
+    }
     ApplyParams P = make_params(g);
     unsigned long long* d_cnt = nullptr;
     FFT_CUDA(cudaMalloc(&d_cnt, 2 * sizeof(unsigned long long)));
@@ -402,6 +418,16 @@ fft_status count_support(fft_geom g, int64_t* support, int64_t* evaluated) {
 }
 
 fft_status compute_frob2(fft_geom g, double* out) {
+    if (!g->stk.empty()) {
+        *out = 0.0;
+        for (StackClass& c : g->stk) {
+            double s = 0.0;
+            const fft_status rc = compute_frob2(c.sub, &s);
+            if (rc != FFT_OK) return rc;
+            *out += s;
+        }
+        return FFT_OK;
+    }
     ApplyParams P = make_params(g);
     double* d_sum = nullptr;
     size_t n = (size_t)(g->n_items > 0 ? g->n_items : 1) * APPLY_WARPS;   // one per unit

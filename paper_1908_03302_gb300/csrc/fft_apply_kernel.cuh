@@ -61,6 +61,7 @@ struct ApplyParams {
     int tiles_x, tiles_y;
     int nx, ny, nz;
     int z_lo, z_end, mirror;   // layers to evaluate, mirror plane (fft_geom_s)
+    const uint8_t* zw;         // COUNT, FROB: weight of each layer (null: 1)
     double org[3];
     double h;
     const float* vin;        // J: m [V]; J^T: d [M]
@@ -514,12 +515,19 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
         auto mirror_off = [&](int s) {
             return (int64_t)mirror_step(P.mirror, TZ + ozi + sub_dz<NSUB>(s), P.nz) * P.ny * P.nx;
         };
-        // the count and the Frobenius norm take a mirrored run twice (bit s)
-        uint32_t twice = 0;
+        // the count and the Frobenius norm weigh a run with its layer and its image (8 bits per
+        // sub-brick; at most 2 STACK_MAX_SLICES)
+        uint32_t mult = 0;
         if (MODE == MODE_COUNT || MODE == MODE_FROB) {
 #pragma unroll
-            for (int s = 0; s < NSUB; ++s)
-                if (mirror_off(s) != 0) twice |= 1u << s;
+            for (int s = 0; s < NSUB; ++s) {
+                const int z = TZ + ozi + sub_dz<NSUB>(s);
+                if (z >= P.nz) continue;
+                const int zs = mirror_step(P.mirror, z, P.nz);
+                uint32_t w = P.zw ? P.zw[z] : 1u;
+                if (zs != 0) w += P.zw ? P.zw[z + zs] : 1u;
+                mult |= w << (8 * s);
+            }
         }
 
         // accumulators (J^T) or model values (J) of the lane's voxels, as pairs (0, 1), (2, 3) of
@@ -647,7 +655,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         const uint32_t vm = (vmask >> (4 * s)) & 15u;
                         const uint32_t in = (va.x < 1.0f ? 1u : 0u) | (va.y < 1.0f ? 2u : 0u) | (vb.x < 1.0f ? 4u : 0u) |
                                             (vb.y < 1.0f ? 8u : 0u);
-                        n_in += (__popc(in & vm) | (__popc(vm) << 16)) << ((twice >> s) & 1u);
+                        n_in += (__popc(in & vm) | (__popc(vm) << 16)) * ((mult >> (8 * s)) & 255u);
                         return;
                     }
                     float ph[NX_LANE];
@@ -688,7 +696,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         }
                         if (MODE == MODE_FROB) {
                             const float2 x = up(val);
-                            const float f = ((twice >> s) & 1u) ? 2.0f : 1.0f;
+                            const float f = (float)((mult >> (8 * s)) & 255u);
                             if ((vmask >> (4 * s + 2 * j)) & 1u) fsum = fmaf(f * x.x, x.x, fsum);
                             if ((vmask >> (4 * s + 2 * j + 1)) & 1u) fsum = fmaf(f * x.y, x.y, fsum);
                         }
@@ -793,7 +801,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                             if (d0 == 0.0f && d1 == 0.0f) continue;
                             const f2 dk = pk(d0, d1);
                             const bool ok0 = (vmask >> (4 * s + 2 * j)) & 1u, ok1 = (vmask >> (4 * s + 2 * j + 1)) & 1u;
-                            const int f = 1 + (int)((twice >> s) & 1u);   // count, Frobenius
+                            const int f = (int)((mult >> (8 * s)) & 255u);   // count, Frobenius
                             if (MODE == MODE_COUNT) n_in += f * ((ok0 ? (int)d0 : 0) + (ok1 ? (int)d1 : 0));
                             if (MODE == MODE_JT || MODE == MODE_COV) acc[s][j] = fma2(dk, pk1(W), acc[s][j]);
                             if (MODE == MODE_J) part = fma2(dk, mv[s][j], part);

@@ -112,6 +112,22 @@ struct fft_table_s {
     std::vector<double> coef;  // series: a_1 .. a_n (host, FP64)
 };
 
+namespace fftgb {
+// Elevation stacks (fft_stack.cu): slices of equal rows whole numbers of layers apart.
+constexpr size_t STACK_MAX_SLICES = 64, STACK_MAX_CLASSES = 8;
+constexpr int64_t STACK_MIN_ENTRIES = 1 << 18;   // see build_stack
+struct StackPlan {                               // host: a class as find_stack sees it
+    double z;                                    // plane of its lowest slice
+    std::vector<int32_t> shift;                  // each slice's layers above that
+    std::vector<std::vector<int32_t>> rows;      // each slice's rows, in one order
+};
+struct StackClass {
+    fft_geom sub = nullptr;                      // operator of the lowest slice on the extended grid
+    std::vector<int32_t> off;                    // per slice: grid layer z is extended layer z + off
+    int64_t row0 = 0;                            // first of the slices' rows in stk_rows
+};
+}  // namespace fftgb
+
 struct fft_geom_s {
     int dev;
     int64_t M;
@@ -144,6 +160,20 @@ struct fft_geom_s {
     // the layers [z_lo, z_end) and the products serve the mirrored layer of each from the same
     // evaluation. Without one: all layers, mirror = -1. (The tile lists always cover the grid.)
     int32_t z_lo = 0, z_end = 0, mirror = -1;
+    // Elevation stack (fft_stack.cu): J and J^T go through these classes' operators when there are any
+    // (several columns at once only if stk_batch says that it evaluates less). The operators use the
+    // parent's partial buffers; theirs (`nested`) are never allocated or freed on their own.
+    std::vector<fftgb::StackClass> stk;
+    bool stk_batch = false;
+    int32_t* stk_rows = nullptr;         // [M] the slices' rows, class by class
+    float* stk_x = nullptr;              // [4 x extended voxels] columns of a pass
+    float* stk_d = nullptr;              // [4 x rows of a slice]
+    float* stk_jpart = nullptr;          // J partials of the operators
+    float* stk_gpart = nullptr;          // their J^T partials
+    int64_t stk_gpart_cap = 0;           // (floats)
+    bool nested = false;
+    uint8_t* zw = nullptr;               // nested: [nz] slices that hold the layer (support count, Frobenius norm)
+    int64_t E_used = 0;                  // entries of the tiles that the products evaluate
     int32_t tiles[3];
     int64_t n_tiles = 0;
     int64_t E = 0;                       // entries
@@ -207,7 +237,14 @@ fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st)
 fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st);
 fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_per_cta);
 fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st);
-fft_status launch_JT_rows(fft_geom g, const float* din, float* gout, cudaStream_t st);
+bool find_stack(const double* tx, const int32_t* rows, int64_t M, const int32_t* band, const fft_grid& gr,
+                std::vector<StackPlan>& plan);
+double stack_cost(const std::vector<StackPlan>& plan, int64_t M, const fft_grid& gr);
+double stack_entries(fft_geom g, int64_t n);
+fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st);
+fft_status stack_JT(fft_geom g, const float* d, int n, float* gout, cudaStream_t st);
+fft_status stack_scratch(fft_geom g);
+fft_status stack_build_items(fft_geom g, int items_per_cta);
 fft_status check_device(int dev);
 fft_status count_support(fft_geom g, int64_t* support, int64_t* evaluated);
 fft_status compute_frob2(fft_geom g, double* out);

@@ -307,11 +307,13 @@ fft_status dmalloc(fft_geom g, T** p, size_t count) {
 
 void free_geom(fft_geom g) {
     if (!g) return;
+    for (StackClass& c : g->stk) free_geom(c.sub);
+    if (g->nested) g->jpart = g->jpart4 = g->gpart = g->gpart4 = nullptr;   // the parent's
     void* ptrs[] = {g->d_band, g->rec, g->rec64, g->row_band, g->tab, g->tile_off, g->tile_rows, g->ebase, g->ebase3,
                     g->row_off, g->row_ent, g->items, g->tile_slot0, g->tile_nslot, g->jpart,
                     g->gpart, g->counter, g->cg_r, g->cg_q, g->cg_s, g->cg_p, g->cg_d, g->cg_m,
                     g->cg_scal, g->cg_dots, g->cg_status, g->cg_hist, g->vol, g->jpart4, g->gpart4,
-                    g->psf_crec};
+                    g->psf_crec, g->stk_rows, g->stk_x, g->stk_d, g->stk_jpart, g->stk_gpart, g->zw};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (g->cg_graph) cudaGraphExecDestroy((cudaGraphExec_t)g->cg_graph);
@@ -395,9 +397,10 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
     std::stable_sort(items_sharp.begin(), items_sharp.end(), heavier);
     g->n_items_plain = (int32_t)items.size();
     items.insert(items.end(), items_sharp.begin(), items_sharp.end());
+    if (g->nested) g->jpart4 = g->gpart = g->gpart4 = nullptr;   // the parent's (stack_scratch sets them again)
     if (g->items) {   // the buffers below are replaced: take them out of the scratch count
-        g->scratch_bytes -= (int64_t)(sizeof(Item) * g->n_items + 2 * sizeof(int32_t) * g->n_tiles +
-                                      sizeof(float) * (size_t)g->n_slots * TILE_VOX);
+        g->scratch_bytes -= (int64_t)(sizeof(Item) * g->n_items + 2 * sizeof(int32_t) * g->n_tiles);
+        if (!g->nested) g->scratch_bytes -= (int64_t)(sizeof(float) * (size_t)g->n_slots * TILE_VOX);
         if (g->jpart4)
             g->scratch_bytes -= (int64_t)(sizeof(float) * ((size_t)g->E * 32 + (size_t)g->n_slots * 4 * TILE_VOX));
     }
@@ -418,7 +421,7 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
     if ((rc = dmalloc(g, &g->items, items.size())) != FFT_OK) return rc;
     if ((rc = dmalloc(g, &g->tile_slot0, g->n_tiles)) != FFT_OK) return rc;
     if ((rc = dmalloc(g, &g->tile_nslot, g->n_tiles)) != FFT_OK) return rc;
-    if ((rc = dmalloc(g, &g->gpart, (size_t)slots * TILE_VOX)) != FFT_OK) return rc;
+    if (!g->nested && (rc = dmalloc(g, &g->gpart, (size_t)slots * TILE_VOX)) != FFT_OK) return rc;
     cudaError_t e = cudaSuccess;
     if (!items.empty()) e = cudaMemcpy(g->items, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
@@ -440,15 +443,152 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
     return FFT_OK;
 }
 
+// The partial buffers that a stack's operators share: their passes follow each other on one stream.
+// (J^T partials grow with the items; the J partials do not.)
+fft_status stack_scratch(fft_geom g) {
+    int64_t need = 0;
+    for (StackClass& c : g->stk) need = std::max(need, (int64_t)c.sub->n_slots * 4 * TILE_VOX);
+    if (need > g->stk_gpart_cap || !g->stk_gpart) {
+        cudaFree(g->stk_gpart);
+        g->scratch_bytes -= (int64_t)sizeof(float) * g->stk_gpart_cap;
+        g->stk_gpart = nullptr;
+        g->stk_gpart_cap = 0;
+        const fft_status rc = dmalloc(g, &g->stk_gpart, (size_t)std::max<int64_t>(need, 1));
+        if (rc != FFT_OK) return rc;
+        g->stk_gpart_cap = std::max<int64_t>(need, 1);
+    }
+    for (StackClass& c : g->stk) {
+        c.sub->jpart = c.sub->jpart4 = g->stk_jpart;
+        c.sub->gpart = c.sub->gpart4 = g->stk_gpart;
+    }
+    return FFT_OK;
+}
+
+// Work items of the operators of a stack (the autotuner's candidates).
+fft_status stack_build_items(fft_geom g, int items_per_cta) {
+    for (StackClass& c : g->stk) {
+        std::vector<int64_t> toff(c.sub->n_tiles + 1);
+        FFT_CUDA(cudaMemcpy(toff.data(), c.sub->tile_off, sizeof(int64_t) * toff.size(), cudaMemcpyDeviceToHost));
+        c.sub->apply_ctas = g->apply_ctas;
+        const fft_status rc = build_items(c.sub, toff, items_per_cta);
+        if (rc != FFT_OK) return rc;
+    }
+    return stack_scratch(g);
+}
+
+namespace {
+
+fft_status create_geom(const double* tx_xyz, int32_t n_tx, const int32_t* rows, int64_t n_rows,
+                       const int32_t* band_of_row, const fft_grid* grid, double c0, const fft_table* tables,
+                       int32_t n_tables, int32_t dt_mode, bool nested, fft_geom* out);
+
+void drop_stack(fft_geom g) {
+    for (StackClass& c : g->stk) free_geom(c.sub);
+    g->stk.clear();
+    void* ptrs[] = {g->stk_rows, g->stk_x, g->stk_d, g->stk_jpart, g->stk_gpart};
+    for (void* q : ptrs)
+        if (q) cudaFree(q);
+    g->stk_rows = nullptr;
+    g->stk_x = g->stk_d = g->stk_jpart = g->stk_gpart = nullptr;
+    g->stk_gpart_cap = 0;
+}
+
+// Operators of an elevation stack's classes where they pay: from STACK_MIN_ENTRIES entries (below, a
+// product is bound by launches and the classes add more of them), with at most 0.8 of the entries of a
+// pass over all rows left to evaluate, and with memory to spare. g stays as it is otherwise.
+void build_stack(fft_geom g, const double* tx, const int32_t* rows, const int32_t* band, const fft_table* tables) {
+    std::vector<StackPlan> plan;
+    if (g->nested || g->dt_mode != FFT_DT_STABLE || g->E_used < STACK_MIN_ENTRIES) return;
+    if (!find_stack(tx, rows, g->M, band, g->grid, plan) || stack_cost(plan, g->M, g->grid) > 0.8) return;
+    size_t mem_free = 0, mem_total = 0;
+    if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    const int64_t plane = (int64_t)g->grid.nx * g->grid.ny;
+    // (an operator's entries: 32 bytes of lists and 128 of partials each, about its slices' share of E)
+    double need = 0.0;
+    for (const StackPlan& c : plan)
+        need = std::max(need, 160.0 * (double)g->E * (double)c.rows[0].size() / (double)g->M +
+                                  16.0 * (double)plane * (g->grid.nz + c.shift.back()));
+    if (2.0 * need > 0.5 * (double)mem_free) return;
+    const int64_t before = g->scratch_bytes;
+    std::vector<int32_t> ids;
+    ids.reserve((size_t)g->M);
+    int64_t v_max = 0, m_max = 0, e_max = 0;
+    bool ok = true;
+    for (const StackPlan& c : plan) {
+        const int32_t top = c.shift.back();
+        fft_grid eg = g->grid;
+        eg.nz += top;
+        eg.origin[2] -= top * eg.h;
+        // the transducers of the lowest slice alone, in the order of its rows
+        std::vector<double> stx;
+        std::vector<int32_t> srows, sband, at;
+        const std::vector<int32_t>& base = c.rows[0];
+        at.assign((size_t)g->n_tx, -1);
+        for (int32_t p : base) {
+            for (int e = 0; e < 2; ++e) {
+                const int32_t t = rows[2 * (int64_t)p + e];
+                if (at[t] < 0) {
+                    at[t] = (int32_t)(stx.size() / 3);
+                    stx.insert(stx.end(), tx + 3 * (int64_t)t, tx + 3 * (int64_t)t + 3);
+                }
+                srows.push_back(at[t]);
+            }
+            sband.push_back(band ? band[p] : 0);
+        }
+        StackClass k;
+        if (create_geom(stx.data(), (int32_t)(stx.size() / 3), srows.data(), (int64_t)base.size(), sband.data(), &eg, g->c0,
+                        tables, g->n_bands, g->dt_mode, true, &k.sub) != FFT_OK) {
+            ok = false;
+            break;
+        }
+        k.row0 = (int64_t)ids.size();
+        std::vector<uint8_t> zw((size_t)eg.nz, 0);
+        for (size_t s = 0; s < c.rows.size(); ++s) {
+            k.off.push_back(top - c.shift[s]);
+            ids.insert(ids.end(), c.rows[s].begin(), c.rows[s].end());
+            for (int z = 0; z < g->grid.nz; ++z) ++zw[z + k.off[s]];
+        }
+        g->stk.push_back(k);
+        ok = dmalloc(k.sub, &k.sub->zw, zw.size()) == FFT_OK &&
+             cudaMemcpy(k.sub->zw, zw.data(), zw.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+        if (!ok) break;
+        g->scratch_bytes += k.sub->scratch_bytes;
+        v_max = std::max(v_max, k.sub->V);
+        m_max = std::max(m_max, k.sub->M);
+        e_max = std::max(e_max, k.sub->E);
+    }
+    ok = ok && stack_entries(g, 1) <= 0.8 * (double)g->E_used;
+    ok = ok && dmalloc(g, &g->stk_rows, ids.size()) == FFT_OK &&
+         cudaMemcpy(g->stk_rows, ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+         dmalloc(g, &g->stk_x, 4 * (size_t)v_max) == FFT_OK && dmalloc(g, &g->stk_d, 4 * (size_t)m_max) == FFT_OK &&
+         dmalloc(g, &g->stk_jpart, 32 * (size_t)e_max) == FFT_OK && stack_scratch(g) == FFT_OK;
+    if (!ok) {
+        cudaGetLastError();
+        drop_stack(g);
+        g->scratch_bytes = before;
+        return;
+    }
+    // n columns at once: the four-column pass over all rows costs 1.45 passes
+    g->stk_batch = stack_entries(g, 4) <= 1.45 * (double)g->E_used;
+}
+
+}  // namespace
+
 }  // namespace fftgb
 
 using namespace fftgb;
 
-extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const int32_t* rows,
-                                      int64_t n_rows, const int32_t* band_of_row, const fft_grid* grid,
-                                      double c0, const fft_table* tables, int32_t n_tables,
-                                      int32_t dt_mode, fft_geom* out) {
-    FFT_API_RANGE("fft_geom_create");
+namespace fftgb {
+
+namespace {
+
+// nested: an operator of a stack's class (fft_geom_s): no partial buffers of its own, no support count.
+fft_status create_geom(const double* tx_xyz, int32_t n_tx, const int32_t* rows, int64_t n_rows,
+                       const int32_t* band_of_row, const fft_grid* grid, double c0, const fft_table* tables,
+                       int32_t n_tables, int32_t dt_mode, bool nested, fft_geom* out) {
     FFT_ARG(out, "fft_geom_create: null out");
     *out = nullptr;
     FFT_ARG(tx_xyz && n_tx >= 2, "fft_geom_create: need at least two transducers");
@@ -511,6 +651,7 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
         }
     }
     fft_geom g = new fft_geom_s();
+    g->nested = nested;
     g->dev = dev;
     g->M = n_rows;
     g->V = V;
@@ -749,6 +890,7 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
         const int64_t per_z = (int64_t)g->tiles[0] * g->tiles[1];
         const int64_t e_lo = toff[per_z * (g->z_lo / TILE_Z)], e_hi = toff[per_z * ceil_div(g->z_end, TILE_Z)];
         const int64_t Ek = e_hi - e_lo;
+        g->E_used = Ek;
         int32_t* d_rc = nullptr;
         int32_t* d_cur = nullptr;
         cudaError_t ea = cudaMalloc(&d_rc, sizeof(int32_t) * n_rows);
@@ -790,16 +932,30 @@ extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const 
     g->apply_ctas = apply_occupancy(g);
     sharp_launch_shape(g);
     plain_launch_shape(g);
-    GEOM_TRY(dmalloc(g, &g->jpart, (size_t)g->E * 4));   // one J partial per (entry, 8 x 8 x 8 region)
+    build_stack(g, tx_xyz, rows, band_of_row, tables);
+    // one J partial per (entry, 8 x 8 x 8 region); a stack's products use its classes' buffer
+    if (!nested && g->stk.empty()) GEOM_TRY(dmalloc(g, &g->jpart, (size_t)g->E * 4));
     GEOM_TRY(dmalloc(g, &g->counter, 4));
     GEOM_TRY(build_items(g, toff, DEFAULT_ITEMS_PER_CTA));
     GEOM_CUDA(cudaDeviceSynchronize());
-    GEOM_TRY(count_support(g, &g->support, &g->evaluated));
+    if (!nested) GEOM_TRY(count_support(g, &g->support, &g->evaluated));
     GEOM_CUDA(cudaDeviceSynchronize());
 #undef GEOM_TRY
 #undef GEOM_CUDA
     *out = g;
     return FFT_OK;
+}
+
+}  // namespace
+
+}  // namespace fftgb
+
+extern "C" fft_status fft_geom_create(const double* tx_xyz, int32_t n_tx, const int32_t* rows,
+                                      int64_t n_rows, const int32_t* band_of_row, const fft_grid* grid,
+                                      double c0, const fft_table* tables, int32_t n_tables,
+                                      int32_t dt_mode, fft_geom* out) {
+    FFT_API_RANGE("fft_geom_create");
+    return create_geom(tx_xyz, n_tx, rows, n_rows, band_of_row, grid, c0, tables, n_tables, dt_mode, false, out);
 }
 
 extern "C" void fft_geom_destroy(fft_geom g) {

@@ -65,6 +65,7 @@ extern "C" fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_
     auto try_one = [&](int ctas, int ii) -> bool {
         g->apply_ctas = ctas * sms;
         if ((rc = build_items(g, toff, cand_items[ii])) != FFT_OK) return false;
+        if (!g->stk.empty() && (rc = stack_build_items(g, cand_items[ii])) != FFT_OK) return false;
         if (tried == 0 || last < 20.0) {
             if ((rc = launch_JT(g, d, out_v, st)) != FFT_OK) return false;
             if ((rc = launch_J(g, m, out_m, st)) != FFT_OK) return false;
@@ -107,6 +108,7 @@ extern "C" fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_
     if (e == cudaSuccess && rc == FFT_OK) {
         g->apply_ctas = best_ctas * sms;
         rc = build_items(g, toff, best_items);
+        if (rc == FFT_OK && !g->stk.empty()) rc = stack_build_items(g, best_items);
     }
     if (e == cudaSuccess && rc == FFT_OK) e = cudaStreamSynchronize(st);
     cudaFree(m);
