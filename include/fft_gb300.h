@@ -213,7 +213,8 @@ fft_status fft_JT_apply(fft_geom g, const float* d_dev, float* g_dev, void* stre
  * Columns are processed in groups of four; a remainder (and every column of geometries with
  * a non-stable detour mode) goes through the single-vector kernels. Each column matches the
  * single-vector call to rounding (same entries, same summation order). The first call
- * allocates the handle's four-column scratch (E * 32 + slots * 4 * 2048 floats).
+ * allocates the handle's batch scratch (E * 32 + slots * 4 * 2048 floats; twice that
+ * from five columns on, where it takes at most half of the free memory).
  */
 fft_status fft_J_apply_batch(fft_geom g, const float* m_dev, int32_t n, float* d_dev, void* stream);
 fft_status fft_JT_apply_batch(fft_geom g, const float* d_dev, int32_t n, float* g_dev, void* stream);

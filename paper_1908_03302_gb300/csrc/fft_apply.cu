@@ -39,33 +39,39 @@ __global__ void __launch_bounds__(256) j_reduce_kernel(const int64_t* __restrict
     if (lane == 0) d[p] = (float)s;
 }
 
-// The four-column form of j_reduce_kernel: jpart4[(entry * 8 + region) * 4 + r]; the same lane
-// order, pairing and butterfly per column, d[r * M + p].
-__global__ void __launch_bounds__(256) j_reduce4_kernel(const int64_t* __restrict__ row_off,
-                                                        const int64_t* __restrict__ row_ent,
-                                                        const float* __restrict__ jpart4, int64_t M,
-                                                        float* __restrict__ d) {
+// The batch form of j_reduce_kernel: jpart[(entry * 8 + region) * NC + r]; the same lane order,
+// pairing and butterfly per column, d[r * M + p], columns r < ncol.
+template <int NC>
+__global__ void __launch_bounds__(256) j_reduce_n_kernel(const int64_t* __restrict__ row_off,
+                                                         const int64_t* __restrict__ row_ent,
+                                                         const float* __restrict__ jpart, int64_t M, int ncol,
+                                                         float* __restrict__ d) {
     const int lane = threadIdx.x & 31;
     const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (p >= M) return;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    double s[NC];
+#pragma unroll
+    for (int r = 0; r < NC; ++r) s[r] = 0.0;
     const int64_t j1 = row_off[p + 1];
     for (int64_t j = row_off[p] + lane; j < j1; j += 32) {
-        const float4* q = reinterpret_cast<const float4*>(jpart4 + row_ent[j] * 32);
-        float4 g[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) g[k] = __ldg(q + k);
-        s[0] += (double)(((g[0].x + g[1].x) + (g[2].x + g[3].x)) + ((g[4].x + g[5].x) + (g[6].x + g[7].x)));
-        s[1] += (double)(((g[0].y + g[1].y) + (g[2].y + g[3].y)) + ((g[4].y + g[5].y) + (g[6].y + g[7].y)));
-        s[2] += (double)(((g[0].z + g[1].z) + (g[2].z + g[3].z)) + ((g[4].z + g[5].z) + (g[6].z + g[7].z)));
-        s[3] += (double)(((g[0].w + g[1].w) + (g[2].w + g[3].w)) + ((g[4].w + g[5].w) + (g[6].w + g[7].w)));
+        for (int h = 0; h < NC / 4; ++h) {
+            const float4* q = reinterpret_cast<const float4*>(jpart + row_ent[j] * (8 * NC)) + h;
+            float4 g[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) g[k] = __ldg(q + k * (NC / 4));
+            s[4 * h] += (double)(((g[0].x + g[1].x) + (g[2].x + g[3].x)) + ((g[4].x + g[5].x) + (g[6].x + g[7].x)));
+            s[4 * h + 1] += (double)(((g[0].y + g[1].y) + (g[2].y + g[3].y)) + ((g[4].y + g[5].y) + (g[6].y + g[7].y)));
+            s[4 * h + 2] += (double)(((g[0].z + g[1].z) + (g[2].z + g[3].z)) + ((g[4].z + g[5].z) + (g[6].z + g[7].z)));
+            s[4 * h + 3] += (double)(((g[0].w + g[1].w) + (g[2].w + g[3].w)) + ((g[4].w + g[5].w) + (g[6].w + g[7].w)));
+        }
     }
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < NC; ++r) {
         double v = s[r];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) d[(int64_t)r * M + p] = (float)v;
+        if (lane == 0 && r < ncol) d[(int64_t)r * M + p] = (float)v;
     }
 }
 
@@ -75,15 +81,16 @@ __global__ void __launch_bounds__(256) j_reduce4_kernel(const int64_t* __restric
 // to the number of slots), the eight partial sums are added in FP64: a fixed order, and eight times
 // as many loads in flight as with one thread per run, which a tile cut into many small items
 // needs (32-element ring: about 45 slots per tile).
-// NCOL = 4: the four-column form, slot q of column r at gpart[((s0 + q) * 4 + r) * TILE_VOX],
-// g[r * V + v].
+// NCOL = 4, 8: the batch forms, slot q of column r at gpart[((s0 + q) * NCOL + r) * TILE_VOX],
+// g[r * V + v], columns r < ncol.
 constexpr int RED_WARPS = 8;
 template <int NCOL>
 __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t* __restrict__ slot0,
                                                                    const int32_t* __restrict__ nslot,
                                                                    const float* __restrict__ gpart, int nx, int ny,
                                                                    int nz, int z_lo, int z_end, int mirror,
-                                                                   int tiles_x, int tiles_y, float* __restrict__ g) {
+                                                                   int tiles_x, int tiles_y, int ncol,
+                                                                   float* __restrict__ g) {
     __shared__ float4 sh[RED_WARPS][32];
     constexpr int PER_TILE = TILE_VOX / (4 * 32);   // CTAs per tile
     const int T = blockIdx.x / PER_TILE, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -98,7 +105,7 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
     const bool inside = iy < ny && iz >= z_lo && iz < z_end && ix < nx;
     const int64_t mo = (int64_t)mirror_step(mirror, iz, nz) * ny * nx;   // to the mirrored layer (0: none)
     const int ns = (s0 == -2 || !inside) ? 0 : nslot[T];
-    for (int r = 0; r < NCOL; ++r) {
+    for (int r = 0; r < ncol; ++r) {
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, low[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         const float* base = ns > 0 ? gpart + ((int64_t)s0 * NCOL + r) * TILE_VOX + loc : nullptr;
         auto add = [&](const float4& x) {
@@ -171,6 +178,7 @@ static ApplyParams make_params(fft_geom g) {
     P.seg_n = g->seg_n;
     P.nvox = g->V;
     P.nrow = g->M;
+    P.ncol = 1;
     return P;
 }
 
@@ -180,6 +188,8 @@ size_t apply_smem(fft_geom g, int warps) {
 }
 
 size_t apply_smem(fft_geom g) { return apply_smem(g, APPLY_WARPS); }
+
+size_t apply_smem8(fft_geom g) { return apply_smem(g, 0) + (size_t)COL8_WARPS * STG_PER_WARP8 * sizeof(float4); }
 
 // Most warps (a multiple of 8, at most 24) one sharp-variant CTA can stage for.
 static int sharp_max_warps(fft_geom g) {
@@ -213,6 +223,16 @@ fft_status set_apply_attributes(fft_geom g) {
     // batch modes: stable detour only (other geometries apply the columns one by one)
     if ((rc = set_attr_mode<MODE_JT4>(smem)) != FFT_OK) return rc;
     if ((rc = set_attr_mode<MODE_J4>(smem)) != FFT_OK) return rc;
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, dev);
+    g->sms = std::max(g->sms, 1);
+    g->col8 = g->dt_mode == FFT_DT_STABLE && apply_smem8(g) <= (size_t)optin;
+    if (g->col8) {
+        if ((rc = set_attr_mode<MODE_JT8>(apply_smem8(g))) != FFT_OK) return rc;
+        if ((rc = set_attr_mode<MODE_J8>(apply_smem8(g))) != FFT_OK) return rc;
+    }
     return set_attr_mode<MODE_FROB>(smem);
 }
 
@@ -271,81 +291,125 @@ void plain_launch_shape(fft_geom g) {
     g->plain_ctas = std::max(best_b, 1) * sms;
 }
 
-static fft_status batch_scratch(fft_geom g) {
-    if (!g->jpart4) {
-        cudaError_t e = cudaMalloc(&g->jpart4, sizeof(float) * (size_t)(g->E > 0 ? g->E : 1) * 32);
+// Partials of a batch of n columns: for eight columns at once where n is more than four, the kernels
+// fit and memory allows it, else for four. Kept with the geometry, and grown unless the stream is capturing.
+static fft_status batch_scratch(fft_geom g, int n, cudaStream_t st) {
+    if (g->nested) return FFT_OK;   // the parent's (stack_scratch)
+    int cols = (n > 4 && g->col8) ? 8 : 4;
+    if (g->batch_cols >= cols) return FFT_OK;
+    if (cols == 8) {   // taken, or grown to, only with memory to spare
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        size_t mem_free = 0, mem_total = 0;
+        FFT_CUDA(cudaStreamIsCapturing(st, &cap));
+        FFT_CUDA(cudaMemGetInfo(&mem_free, &mem_total));
+        const double need = 8.0 * sizeof(float) * ((double)g->E * 8 + (double)g->n_slots * TILE_VOX);
+        if (cap != cudaStreamCaptureStatusNone || 2.0 * need > (double)mem_free) cols = 4;
+        if (g->batch_cols >= cols) return FFT_OK;
+        free_batch_scratch(g);
+    }
+    for (; cols >= 4; cols -= 4) {
+        cudaError_t e = cudaMalloc(&g->jpart4, sizeof(float) * (size_t)(g->E > 0 ? g->E : 1) * 8 * cols);
         if (e == cudaSuccess && g->n_slots > 0)
-            e = cudaMalloc(&g->gpart4, sizeof(float) * (size_t)g->n_slots * 4 * TILE_VOX);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(g->jpart4);
-            g->jpart4 = nullptr;
-            set_error("batch apply: cudaMalloc of the four-column scratch failed");
-            return FFT_ERR_OOM;
+            e = cudaMalloc(&g->gpart4, sizeof(float) * (size_t)g->n_slots * cols * TILE_VOX);
+        if (e == cudaSuccess) {
+            g->batch_cols = cols;
+            g->scratch_bytes += batch_scratch_bytes(g);
+            return FFT_OK;
         }
-        g->scratch_bytes += (int64_t)(sizeof(float) * ((size_t)g->E * 32 + (size_t)g->n_slots * 4 * TILE_VOX));
+        cudaGetLastError();
+        cudaFree(g->jpart4);
+        g->jpart4 = nullptr;
     }
-    return FFT_OK;
+    set_error("batch apply: cudaMalloc of the partial buffers failed");
+    return FFT_ERR_OOM;
 }
 
-// d[:, c] = J m[:, c] for n columns: groups of four with the batch kernel on stable-detour
-// geometries, single columns otherwise.
-fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st) {
-    if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_J(g, m, n, d, st);
-    int c = 0;
-    if (g->dt_mode == FFT_DT_STABLE && n >= 4) {
-        fft_status rc = batch_scratch(g);
-        if (rc != FFT_OK) return rc;
-        for (; c + 4 <= n; c += 4) {
-            ApplyParams P = make_params(g);
-            P.vin = m + (int64_t)c * g->V;
-            P.vout = g->jpart4;
-            if ((rc = launch_batch<MODE_J4>(g, P, st)) != FFT_OK) return rc;
-            if (g->M > 0) {
-                j_reduce4_kernel<<<(unsigned)ceil_div(g->M, 8), 256, 0, st>>>(g->row_off, g->row_ent, g->jpart4, g->M,
-                                                                              d + (int64_t)c * g->M);
-                FFT_CUDA(cudaGetLastError());
-            }
-        }
-    }
-    for (; c < n; ++c) {
-        fft_status rc = launch_J(g, m + (int64_t)c * g->V, d + (int64_t)c * g->M, st);
-        if (rc != FFT_OK) return rc;
-    }
-    return FFT_OK;
+int64_t batch_scratch_bytes(fft_geom g) {
+    return (int64_t)sizeof(float) * g->batch_cols * (g->E * 8 + (int64_t)g->n_slots * TILE_VOX);
 }
 
-template <int NCOL>
-static fft_status launch_jt_reduce(fft_geom g, const float* gpart, float* gout, cudaStream_t st) {
-    if (g->n_tiles == 0) return FFT_OK;
-    jt_reduce_kernel<NCOL><<<(unsigned)(g->n_tiles * (TILE_VOX / 128)), 32 * RED_WARPS, 0, st>>>(
-        g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->z_lo, g->z_end, g->mirror, g->tiles[0],
-        g->tiles[1], gout);
+void free_batch_scratch(fft_geom g) {
+    if (g->nested || g->batch_cols == 0) return;
+    g->scratch_bytes -= batch_scratch_bytes(g);
+    cudaFree(g->jpart4);
+    cudaFree(g->gpart4);
+    g->jpart4 = g->gpart4 = nullptr;
+    g->batch_cols = 0;
+}
+
+// Columns of the next pass of rem columns: one alone, two to four in a four-column pass, five to eight
+// in an eight-column one. Over the same rows of slices3d J^T the three take 25.6, 32.5 and 38.9 ms, so
+// that two columns already pay for the wider kernel (ring256, block of 8, J and J^T: 10.54 ms in two
+// four-column passes, 6.91 ms in one).
+int pass_columns(fft_geom g, int64_t rem) {
+    if (rem > 4 && g->batch_cols == 8) return (int)std::min<int64_t>(rem, 8);
+    return (int)std::min<int64_t>(rem, 4);
+}
+
+template <int NC, int MODE>
+static fft_status j_pass(fft_geom g, const float* m, int nc, float* d, cudaStream_t st) {
+    ApplyParams P = make_params(g);
+    P.vin = m;
+    P.vout = g->jpart4;
+    P.ncol = nc;
+    fft_status rc = launch_batch<MODE>(g, P, st);
+    if (rc != FFT_OK || g->M == 0) return rc;
+    j_reduce_n_kernel<NC><<<(unsigned)ceil_div(g->M, 8), 256, 0, st>>>(g->row_off, g->row_ent, g->jpart4, g->M, nc, d);
     FFT_CUDA(cudaGetLastError());
     return FFT_OK;
 }
 
-// g[:, c] = J^T d[:, c] for n columns (groups of four as above).
+template <int NCOL>
+static fft_status launch_jt_reduce(fft_geom g, const float* gpart, int ncol, float* gout, cudaStream_t st) {
+    if (g->n_tiles == 0) return FFT_OK;
+    jt_reduce_kernel<NCOL><<<(unsigned)(g->n_tiles * (TILE_VOX / 128)), 32 * RED_WARPS, 0, st>>>(
+        g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->z_lo, g->z_end, g->mirror, g->tiles[0],
+        g->tiles[1], ncol, gout);
+    FFT_CUDA(cudaGetLastError());
+    return FFT_OK;
+}
+
+template <int NC, int MODE>
+static fft_status jt_pass(fft_geom g, const float* d, int nc, float* gout, cudaStream_t st) {
+    ApplyParams P = make_params(g);
+    P.vin = d;
+    P.vout = gout;
+    P.gpart = g->gpart4;
+    P.ncol = nc;
+    fft_status rc = launch_batch<MODE>(g, P, st);
+    if (rc != FFT_OK) return rc;
+    return launch_jt_reduce<NC>(g, g->gpart4, nc, gout, st);
+}
+
+// d[:, c] = J m[:, c] for n columns: on stable-detour geometries passes of up to eight or four columns
+// (from four columns on: fewer need no batch scratch; a stack's operator has it), single columns otherwise.
+fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st) {
+    if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_J(g, m, n, d, st);
+    const bool batch = g->dt_mode == FFT_DT_STABLE && (n >= 4 || g->nested);
+    fft_status rc = batch ? batch_scratch(g, n, st) : FFT_OK;
+    for (int c = 0; c < n && rc == FFT_OK;) {
+        const int nc = batch ? pass_columns(g, n - c) : 1;
+        const float* mc = m + (int64_t)c * g->V;
+        float* dc = d + (int64_t)c * g->M;
+        rc = nc == 1 ? launch_J(g, mc, dc, st) : (nc > 4 ? j_pass<8, MODE_J8>(g, mc, nc, dc, st) : j_pass<4, MODE_J4>(g, mc, nc, dc, st));
+        c += nc;
+    }
+    return rc;
+}
+
+// g[:, c] = J^T d[:, c] for n columns (passes as above).
 fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st) {
     if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_JT(g, din, n, gout, st);
-    int c = 0;
-    if (g->dt_mode == FFT_DT_STABLE && n >= 4) {
-        fft_status rc = batch_scratch(g);
-        if (rc != FFT_OK) return rc;
-        for (; c + 4 <= n; c += 4) {
-            ApplyParams P = make_params(g);
-            P.vin = din + (int64_t)c * g->M;
-            P.vout = gout + (int64_t)c * g->V;
-            P.gpart = g->gpart4;
-            if ((rc = launch_batch<MODE_JT4>(g, P, st)) != FFT_OK) return rc;
-            if ((rc = launch_jt_reduce<4>(g, g->gpart4, gout + (int64_t)c * g->V, st)) != FFT_OK) return rc;
-        }
+    const bool batch = g->dt_mode == FFT_DT_STABLE && (n >= 4 || g->nested);
+    fft_status rc = batch ? batch_scratch(g, n, st) : FFT_OK;
+    for (int c = 0; c < n && rc == FFT_OK;) {
+        const int nc = batch ? pass_columns(g, n - c) : 1;
+        const float* dc = din + (int64_t)c * g->M;
+        float* gc = gout + (int64_t)c * g->V;
+        rc = nc == 1 ? launch_JT(g, dc, gc, st) : (nc > 4 ? jt_pass<8, MODE_JT8>(g, dc, nc, gc, st) : jt_pass<4, MODE_JT4>(g, dc, nc, gc, st));
+        c += nc;
     }
-    for (; c < n; ++c) {
-        fft_status rc = launch_JT(g, din + (int64_t)c * g->M, gout + (int64_t)c * g->V, st);
-        if (rc != FFT_OK) return rc;
-    }
-    return FFT_OK;
+    return rc;
 }
 
 fft_status launch_J(fft_geom g, const float* m, float* d, cudaStream_t st) {
@@ -370,7 +434,7 @@ fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st)
     P.vout = gout;
     fft_status rc = launch_mode<MODE_JT>(g, P, st);
     if (rc != FFT_OK) return rc;
-    return launch_jt_reduce<1>(g, g->gpart, gout, st);
+    return launch_jt_reduce<1>(g, g->gpart, 1, gout, st);
 }
 
 // cov_v = sum_p |J[p, v] w_p| (w null: all ones), gathered like J^T.
@@ -380,7 +444,7 @@ fft_status launch_cov(fft_geom g, const float* w, float* cov, cudaStream_t st) {
     P.vout = cov;
     fft_status rc = launch_mode<MODE_COV>(g, P, st);
     if (rc != FFT_OK) return rc;
-    return launch_jt_reduce<1>(g, g->gpart, cov, st);
+    return launch_jt_reduce<1>(g, g->gpart, 1, cov, st);
 }
 
 // In-support evaluations (dt < dt_max) of one apply and evaluations actually performed.

@@ -1,0 +1,18 @@
+// The eight-column J^T kernels.
+#include "fft_apply_kernel.cuh"
+
+namespace fftgb {
+
+template <>
+fft_status launch_batch<MODE_JT8>(fft_geom g, const ApplyParams& P, cudaStream_t st) {
+    return launch_batch_impl<MODE_JT8>(g, P, st);
+}
+template <>
+fft_status set_attr_mode<MODE_JT8>(size_t smem) {
+    fft_status rc = set_attr_dt<MODE_JT8, FFT_DT_STABLE, PHI_TABLE>(smem);
+    if (rc != FFT_OK) return rc;
+    if ((rc = set_attr_dt<MODE_JT8, FFT_DT_STABLE, PHI_TRIG>(smem)) != FFT_OK) return rc;
+    return set_attr_dt<MODE_JT8, FFT_DT_STABLE, PHI_SEG>(smem);
+}
+
+}  // namespace fftgb

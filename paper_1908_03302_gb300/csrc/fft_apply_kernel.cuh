@@ -6,7 +6,7 @@
 //     (built once per geometry by a conservative cull). A work item is a tile and a range of
 //     its rows; a unit is one region of one item: an 8 x 8 x 8 region (four 8 x 4 x 4
 //     sub-bricks, four regions per tile) for the single-column modes, an 8 x 8 x 4 region
-//     (two sub-bricks, eight per tile) for the four-column ones. Every warp of the persistent
+//     (two sub-bricks, eight per tile) for the four- and eight-column ones. Every warp of the persistent
 //     grid pulls units from a counter, heaviest items first, on its own (the only CTA barrier
 //     follows the table load). The launch shape (warps per CTA, CTAs per SM) is picked per
 //     variant from its register budget and the shared memory the band tables take.
@@ -39,10 +39,25 @@
 namespace fftgb {
 
 // MODE_COV: sensitivity coverage sum_p |J[p, v] w_p| (J^T of |J|, same gather as MODE_JT).
-// MODE_JT4 / MODE_J4: J^T and J for four right-hand sides at once (every evaluated entry is
-// applied to all four; blocks are column-major: column r at r * V or r * M).
-enum { MODE_JT = 0, MODE_J = 1, MODE_COUNT = 2, MODE_FROB = 3, MODE_COV = 4, MODE_JT4 = 5, MODE_J4 = 6 };
-constexpr int STG_PER_WARP = 128;   // staged float4 per warp: 32 rows x (3 or 4)
+// MODE_JT4 / MODE_J4, MODE_JT8 / MODE_J8: J^T and J for up to four or eight right-hand sides at once
+// (every evaluated entry is applied to all; blocks are column-major: column r at r * V or r * M).
+enum { MODE_JT = 0, MODE_J = 1, MODE_COUNT = 2, MODE_FROB = 3, MODE_COV = 4, MODE_JT4 = 5, MODE_J4 = 6, MODE_JT8 = 7,
+       MODE_J8 = 8 };
+constexpr int STG_PER_WARP = 128;    // staged float4 per warp: 32 rows x (3 or 4)
+constexpr int STG_PER_WARP8 = 160;   // the eight-column J^T: 32 rows x 5
+// CTA of the eight-column kernels: one of 12 warps per SM, up to 168 registers (64 of them hold a lane's
+// accumulators or model values: 8 voxels x 8 columns). Fewer warps than the four-column kernels' 16
+// hide less latency, yet an entry's evaluation serves twice the columns: 1.2 times the time a pass.
+constexpr int COL8_WARPS = 12;
+
+template <int MODE>
+constexpr int apply_ncol() {
+    return (MODE == MODE_JT8 || MODE == MODE_J8) ? 8 : ((MODE == MODE_JT4 || MODE == MODE_J4) ? 4 : 1);
+}
+template <int MODE>
+constexpr int apply_stage() {
+    return MODE == MODE_JT8 ? STG_PER_WARP8 : STG_PER_WARP;
+}
 
 struct ApplyParams {
     const RowRec* rec;
@@ -72,6 +87,7 @@ struct ApplyParams {
     int trig_nq;             // PHI_TRIG: coefficient groups of 4 per band
     int seg_n;               // PHI_SEG: segments per band
     int64_t nvox, nrow;      // column lengths of the batch modes' blocks (V, M)
+    int ncol;                // columns of the block (at most the mode's; the others count as zero)
 };
 
 // Where the kernels find Phi: `tab` the shared address of the bands' tables or segments, `seg2` that
@@ -134,14 +150,14 @@ __device__ __forceinline__ float detour_v64(const RowRec64& r, double ox, double
 // (apply_sharp_wide and apply_plain_wide below).
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr int apply_min_blocks() {
-    return (SHARP || MODE == MODE_JT4 || MODE == MODE_J4) ? 2
+    return (SHARP || apply_ncol<MODE>() == 4) ? 2
                                                           : ((DT == FFT_DT_STABLE && PHI != PHI_TRIG) ? 4 : 3);
 }
 
 // Sub-bricks per unit and units (regions) per item of each mode: see sub_dy below.
 template <int MODE>
 constexpr int apply_nsub() {
-    return (MODE == MODE_JT4 || MODE == MODE_J4) ? 2 : 4;
+    return apply_ncol<MODE>() > 1 ? 2 : 4;
 }
 template <int MODE>
 constexpr int apply_regions() {
@@ -149,7 +165,7 @@ constexpr int apply_regions() {
 }
 
 // Sub-bricks of a unit. The single-column modes take an 8 x 8 x 8 region (NSUB = 4) and the
-// four-column modes, whose per-voxel state is four times larger, an 8 x 8 x 4 region (NSUB =
+// batch modes, whose per-voxel state is four or eight times larger, an 8 x 8 x 4 region (NSUB =
 // 2). Sub-brick s of a lane sits at y offset sub_dy(s) and z offset sub_dz(s) from sub-brick 0;
 // for NSUB = 4 the order (0,0), (4,0), (4,4), (0,4) lets every step between consecutive
 // sub-bricks move along one axis only.
@@ -418,7 +434,7 @@ __device__ __noinline__ void sharp_fix(const ApplyParams& P, float4 A, float4 B,
 // second cost more.
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr bool apply_sharp_wide() {
-    return SHARP && DT == FFT_DT_STABLE && PHI != PHI_TRIG && MODE != MODE_JT4 && MODE != MODE_J4;
+    return SHARP && DT == FFT_DT_STABLE && PHI != PHI_TRIG && apply_ncol<MODE>() == 1;
 }
 constexpr int SHARP_MAX_WARPS = 20;
 
@@ -428,13 +444,14 @@ constexpr int SHARP_MAX_WARPS = 20;
 // 64 registers: slices3d J^T 408.0 -> 407.6 ms, J 412.6 -> 411.4 ms, ring256 J^T 3.75 -> 3.72 ms.
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr bool apply_plain_wide() {
-    return !SHARP && DT == FFT_DT_STABLE && PHI != PHI_TRIG && MODE != MODE_JT4 && MODE != MODE_J4;
+    return !SHARP && DT == FFT_DT_STABLE && PHI != PHI_TRIG && apply_ncol<MODE>() == 1;
 }
 constexpr int PLAIN_MAX_WARPS = 24;
 
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr int apply_block_bound() {
-    return apply_sharp_wide<MODE, DT, SHARP, PHI>()   ? 32 * SHARP_MAX_WARPS
+    return apply_ncol<MODE>() == 8                    ? 32 * COL8_WARPS
+           : apply_sharp_wide<MODE, DT, SHARP, PHI>() ? 32 * SHARP_MAX_WARPS
            : apply_plain_wide<MODE, DT, SHARP, PHI>() ? 32 * PLAIN_MAX_WARPS
                                                       : APPLY_THREADS;
 }
@@ -461,11 +478,13 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
     at.scale = (float)(PHI == PHI_SEG ? P.seg_n : P.n_tab - 1) * MAGIC2_ULP;
     at.nq = P.trig_nq;
     const int lx = lane & 1, ly = (lane >> 1) & 3, lz = lane >> 3;
-    constexpr bool BATCH = (MODE == MODE_JT4 || MODE == MODE_J4);
-    constexpr int SR = (MODE == MODE_JT4) ? 4 : 3;   // staged float4 per row
+    constexpr int NC = apply_ncol<MODE>();
+    constexpr bool JTN = (MODE == MODE_JT4 || MODE == MODE_JT8), JN = (MODE == MODE_J4 || MODE == MODE_J8);
+    constexpr bool BATCH = NC > 1;
+    constexpr int SR = JTN ? 3 + NC / 4 : 3;   // staged float4 per row
     constexpr int NSUB = apply_nsub<MODE>();
     constexpr int NREG = apply_regions<MODE>();
-    float4* stg = s_stage + warp * STG_PER_WARP;
+    float4* stg = s_stage + warp * apply_stage<MODE>();
     const int n_units = P.n_items * NREG;
 
     for (;;) {
@@ -508,7 +527,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 TZ + 4 * wz + sub_dz<NSUB>(s) + 3 >= P.z_lo)
                 sub_ok |= 1u << s;
         // the gather modes need the mask only for their stores: recomputed there
-        constexpr bool VM_LIVE = !(MODE == MODE_JT || MODE == MODE_COV || MODE == MODE_JT4);
+        constexpr bool VM_LIVE = !(MODE == MODE_JT || MODE == MODE_COV || JTN);
         const uint32_t vmask = VM_LIVE ? lane_vmask() : 0u;
         const int64_t vbase = ((int64_t)(TZ + ozi) * P.ny + TY + oyi) * P.nx + TX + oxi;
         // voxels from this lane's run in sub-brick s to its mirror image (0: none)
@@ -533,7 +552,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
         // accumulators (J^T) or model values (J) of the lane's voxels, as pairs (0, 1), (2, 3) of
         // each run
         f2 acc[NSUB][2], mv[NSUB][2];
-        f2 acc4[2][2][4], mv4[2][2][4];   // four-column modes only (NSUB = 2)
+        f2 accn[2][2][NC], mvn[2][2][NC];   // batch modes only (NSUB = 2)
         double dacc = 0.0;
         unsigned long long cnt = 0, cnt_eval = 0;
 #pragma unroll
@@ -551,13 +570,13 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 }
                 if (BATCH && s < 2) {
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        acc4[s & 1][j][r] = mv4[s & 1][j][r] = 0ull;
-                        if (MODE == MODE_J4) {
+                    for (int r = 0; r < NC; ++r) {
+                        accn[s & 1][j][r] = mvn[s & 1][j][r] = 0ull;
+                        if (JN && r < P.ncol) {
                             const float* mr = P.vin + (int64_t)r * P.nvox + vo;
-                            mv4[s & 1][j][r] = pk(ok0 ? __ldg(mr) : 0.0f, ok1 ? __ldg(mr + 1) : 0.0f);
+                            mvn[s & 1][j][r] = pk(ok0 ? __ldg(mr) : 0.0f, ok1 ? __ldg(mr + 1) : 0.0f);
                             if (const int64_t mo = mirror_off(s))
-                                mv4[s & 1][j][r] = add2(mv4[s & 1][j][r], pk(ok0 ? __ldg(mr + mo) : 0.0f,
+                                mvn[s & 1][j][r] = add2(mvn[s & 1][j][r], pk(ok0 ? __ldg(mr + mo) : 0.0f,
                                                                              ok1 ? __ldg(mr + mo + 1) : 0.0f));
                         }
                     }
@@ -580,10 +599,15 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 float W = r.b.w;
                 if (MODE == MODE_JT) W *= __ldg(P.vin + p);
                 if (MODE == MODE_COV) W = fabsf(W) * (P.vin ? fabsf(__ldg(P.vin + p)) : 1.0f);
-                float4 W4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (MODE == MODE_JT4)
-                    W4 = make_float4(W * __ldg(P.vin + p), W * __ldg(P.vin + P.nrow + p),
-                                     W * __ldg(P.vin + 2 * P.nrow + p), W * __ldg(P.vin + 3 * P.nrow + p));
+                float Wn[NC];
+                bool any_w = false;
+                if (JTN) {
+#pragma unroll
+                    for (int r = 0; r < NC; ++r) {
+                        Wn[r] = r < P.ncol ? W * __ldg(P.vin + (int64_t)r * P.nrow + p) : 0.0f;
+                        any_w = any_w || Wn[r] != 0.0f;
+                    }
+                }
                 const float ex = r.b.x, ey = r.b.y, ez = r.b.z, hl = r.a.w;
                 // sub-brick centres relative to the pair midpoint (FP32; used by the bound only)
                 const float dx = fmaf((float)TX, hb, bc.org[0]) - r.a.x;
@@ -592,8 +616,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const float cx = fmaf(8.0f * wx + 3.5f, hb, dx);
                 const float hxx = 3.5f * hb, hyy = 1.5f * hb;
                 // rows with zero weight add exactly nothing to J^T: skip them
-                const bool live = (MODE == MODE_JT4) ? (W4.x != 0.0f || W4.y != 0.0f || W4.z != 0.0f || W4.w != 0.0f)
-                                                     : ((MODE != MODE_JT && MODE != MODE_COV) || (W != 0.0f));
+                const bool live = JTN ? any_w : ((MODE != MODE_JT && MODE != MODE_COV) || (W != 0.0f));
                 const float pext = hxx * fabsf(ex) + hyy * (fabsf(ey) + fabsf(ez)) + 1e-3f;
                 // deep sub-bricks: their voxel centres (half diagonal sqrt(3.5^2 + 2 1.5^2) = 4.1 steps)
                 // keep DEEP_MARGIN steps off the pair's sphere
@@ -624,7 +647,11 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 stg[lane * SR + 2] = make_float4(W, row_m, DT == FFT_DT_FP64 ? __int_as_float(p) : lam,
                                                  __int_as_float(b | (bc.sharp << 8) | (planar << 9) |
                                                                 (int)((okb << 12) | (inb << 16) | (dpb << 20) | (both << 24))));
-                if (MODE == MODE_JT4) stg[lane * SR + 3] = W4;
+                if (JTN) {
+#pragma unroll
+                    for (int k = 0; k < NC / 4; ++k)
+                        stg[lane * SR + 3 + k] = make_float4(Wn[4 * k], Wn[4 * k + 1], Wn[4 * k + 2], Wn[4 * k + 3]);
+                }
             }
             uint32_t mm = __ballot_sync(0xffffffffu, okb != 0u);
             __syncwarp();
@@ -635,8 +662,17 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const float4 A = stg[bit * SR + 0];
                 const float4 B = stg[bit * SR + 1];
                 const float4 C = stg[bit * SR + 2];
-                const float4 W4 = (MODE == MODE_JT4) ? stg[bit * SR + SR - 1] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                const float Wr[4] = {W4.x, W4.y, W4.z, W4.w};
+                float Wr[NC];
+                if (JTN) {
+#pragma unroll
+                    for (int k = 0; k < NC / 4; ++k) {
+                        const float4 x = stg[bit * SR + 3 + k];
+                        Wr[4 * k] = x.x;
+                        Wr[4 * k + 1] = x.y;
+                        Wr[4 * k + 2] = x.z;
+                        Wr[4 * k + 3] = x.w;
+                    }
+                }
                 const float hx = B.x, hy = B.y, hz = B.z, W = C.x, row_m = C.y;
                 const float hl = 0.5f * (A.x - A.y);   // used by the textbook (NAIVE) detour only
                 const uint32_t cw = (uint32_t)__float_as_int(C.w);
@@ -645,7 +681,9 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 deep_init(dr, C.z);
                 float near = 2.0f;   // smallest |v - 1| of this lane's voxels (sharp bands)
                 f2 part = 0ull;
-                f2 part4[4] = {0ull, 0ull, 0ull, 0ull};
+                f2 partn[NC];
+#pragma unroll
+                for (int r = 0; r < NC; ++r) partn[r] = 0ull;
                 uint32_t n_in = 0;
                 float fsum = 0.0f;
                 // Phi and the mode's sum over one sub-brick's four voxels.
@@ -686,13 +724,13 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                             acc[s][j] = fma2(pk(fabsf(x.x), fabsf(x.y)), pk1(W), acc[s][j]);
                         }
                         if (MODE == MODE_J) part = fma2(val, mv[s][j], part);
-                        if (MODE == MODE_JT4) {
+                        if (JTN) {
 #pragma unroll
-                            for (int r = 0; r < 4; ++r) acc4[s & 1][j][r] = fma2(val, pk1(Wr[r]), acc4[s & 1][j][r]);
+                            for (int r = 0; r < NC; ++r) accn[s & 1][j][r] = fma2(val, pk1(Wr[r]), accn[s & 1][j][r]);
                         }
-                        if (MODE == MODE_J4) {
+                        if (JN) {
 #pragma unroll
-                            for (int r = 0; r < 4; ++r) part4[r] = fma2(val, mv4[s & 1][j][r], part4[r]);
+                            for (int r = 0; r < NC; ++r) partn[r] = fma2(val, mvn[s & 1][j][r], partn[r]);
                         }
                         if (MODE == MODE_FROB) {
                             const float2 x = up(val);
@@ -805,13 +843,13 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                             if (MODE == MODE_COUNT) n_in += f * ((ok0 ? (int)d0 : 0) + (ok1 ? (int)d1 : 0));
                             if (MODE == MODE_JT || MODE == MODE_COV) acc[s][j] = fma2(dk, pk1(W), acc[s][j]);
                             if (MODE == MODE_J) part = fma2(dk, mv[s][j], part);
-                            if (MODE == MODE_JT4) {
+                            if (JTN) {
 #pragma unroll
-                                for (int r = 0; r < 4; ++r) acc4[s & 1][j][r] = fma2(dk, pk1(Wr[r]), acc4[s & 1][j][r]);
+                                for (int r = 0; r < NC; ++r) accn[s & 1][j][r] = fma2(dk, pk1(Wr[r]), accn[s & 1][j][r]);
                             }
-                            if (MODE == MODE_J4) {
+                            if (JN) {
 #pragma unroll
-                                for (int r = 0; r < 4; ++r) part4[r] = fma2(dk, mv4[s & 1][j][r], part4[r]);
+                                for (int r = 0; r < NC; ++r) partn[r] = fma2(dk, mvn[s & 1][j][r], partn[r]);
                             }
                             if (MODE == MODE_FROB) fsum += (float)f * ((ok0 ? d0 : 0.0f) + (ok1 ? d1 : 0.0f));
                         }
@@ -832,25 +870,29 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     __syncwarp();
                     if (lane < 8) reinterpret_cast<float*>(stg + bit * SR)[lane] = ps;
                 }
-                if (MODE == MODE_J4) {
-                    // Transposing fold: each exchange halves the columns a lane carries (2 + 1
-                    // shuffles), three more add the eight lanes that hold one column; lane 8 r then
-                    // parks column r in the row's consumed record: 6 shuffles instead of the 20 of four
-                    // butterflies (ring256, a block of 8 columns: J and J^T 10.93 -> 10.54 ms).
-                    float q[4];
+                if (JN) {
+                    // Transposing fold: each exchange halves the columns a lane carries (NC / 2 + .. + 1
+                    // shuffles), the others add the lanes that hold one column; the first of them
+                    // parks the column in the row's consumed record: 6 shuffles (four columns) instead of
+                    // the 20 of four butterflies (ring256, a block of 8 columns: J and J^T 10.93 -> 10.54 ms).
+                    float q[NC];
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const float2 p2 = up(part4[r]);
+                    for (int r = 0; r < NC; ++r) {
+                        const float2 p2 = up(partn[r]);
                         q[r] = p2.x + p2.y;
                     }
-                    const bool hi = lane & 16, odd = lane & 8;
-                    const float a0 = (hi ? q[2] : q[0]) + __shfl_xor_sync(0xffffffffu, hi ? q[0] : q[2], 16);
-                    const float a1 = (hi ? q[3] : q[1]) + __shfl_xor_sync(0xffffffffu, hi ? q[1] : q[3], 16);
-                    float ps = (odd ? a1 : a0) + __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
+                    constexpr int LANES = 32 / NC;   // lanes of a column
 #pragma unroll
-                    for (int o = 4; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
+                    for (int o = 16, n = NC / 2; o >= LANES; o >>= 1, n >>= 1) {
+                        const bool hi = lane & o;
+#pragma unroll
+                        for (int r = 0; r < n; ++r)
+                            q[r] = (hi ? q[r + n] : q[r]) + __shfl_xor_sync(0xffffffffu, hi ? q[r] : q[r + n], o);
+                    }
+#pragma unroll
+                    for (int o = LANES / 2; o > 0; o >>= 1) q[0] += __shfl_xor_sync(0xffffffffu, q[0], o);
                     __syncwarp();
-                    if ((lane & 7) == 0) reinterpret_cast<float*>(stg + bit * SR)[lane >> 3] = ps;
+                    if (lane % LANES == 0) reinterpret_cast<float*>(stg + bit * SR)[lane / LANES] = q[0];
                 }
                 if (MODE == MODE_FROB) dacc += (double)fsum * (double)W * (double)W;
             }
@@ -866,16 +908,19 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     P.vout[e * NREG + region] = mypart;
                 }
             }
-            if (MODE == MODE_J4) {
+            if (JN) {
                 __syncwarp();
                 if (have) {
-                    float4 r0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    if (okb) {
-                        r0 = stg[lane * SR + 0];
-                        const float Wl = stg[lane * SR + 2].x;
-                        r0 = make_float4(r0.x * Wl, r0.y * Wl, r0.z * Wl, r0.w * Wl);
+#pragma unroll
+                    for (int k = 0; k < NC / 4; ++k) {
+                        float4 r0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                        if (okb) {
+                            r0 = stg[lane * SR + k];
+                            const float Wl = stg[lane * SR + 2].x;
+                            r0 = make_float4(r0.x * Wl, r0.y * Wl, r0.z * Wl, r0.w * Wl);
+                        }
+                        *reinterpret_cast<float4*>(P.vout + (e * NREG + region) * NC + 4 * k) = r0;
                     }
-                    *reinterpret_cast<float4*>(P.vout + (e * NREG + region) * 4) = r0;
                 }
             }
             __syncwarp();
@@ -905,16 +950,17 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 }
             }
         }
-        if (MODE == MODE_JT4) {
-            static_assert(!BATCH || NSUB == 2, "the four-column modes take 8 x 8 x 4 regions");
+        if (JTN) {
+            static_assert(!BATCH || NSUB == 2, "the batch modes take 8 x 8 x 4 regions");
             const uint32_t vm = lane_vmask();
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
                 const int loc = ((ozi * TILE_Y) + oyi + 4 * s) * TILE_X + oxi;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const float2 a0 = up(acc4[s][0][r]), a1 = up(acc4[s][1][r]);
+                for (int r = 0; r < NC; ++r) {
+                    const float2 a0 = up(accn[s][0][r]), a1 = up(accn[s][1][r]);
                     const float av[NX_LANE] = {a0.x, a0.y, a1.x, a1.y};
+                    if (r >= P.ncol) continue;
                     if (item.slot < 0) {
                         const int64_t mo = mirror_off(s);
 #pragma unroll
@@ -925,7 +971,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                                 if (mo != 0) o[mo] = av[t];
                             }
                     } else {
-                        *reinterpret_cast<float4*>(P.gpart + ((int64_t)item.slot * 4 + r) * TILE_VOX + loc) =
+                        *reinterpret_cast<float4*>(P.gpart + ((int64_t)item.slot * NC + r) * TILE_VOX + loc) =
                             make_float4(av[0], av[1], av[2], av[3]);
                     }
                 }
@@ -976,6 +1022,7 @@ inline fft_status set_attr_mode_impl(size_t smem) {
 }
 
 size_t apply_smem(fft_geom g, int warps);
+size_t apply_smem8(fft_geom g);
 // Resident CTAs per SM of the J^T kernel (stable detour, tables; plain or sharp).
 int apply_blocks_per_sm(bool sharp, int threads, size_t smem);
 
@@ -984,7 +1031,9 @@ int apply_blocks_per_sm(bool sharp, int threads, size_t smem);
 // the persistent grid.
 template <int MODE, int DT, bool G, bool S, int PHI>
 inline void launch_apply(fft_geom g, const ApplyParams& P, cudaStream_t st) {
-    if (apply_sharp_wide<MODE, DT, S, PHI>()) {
+    if (apply_ncol<MODE>() == 8) {
+        apply_kernel<MODE, DT, G, S, PHI><<<g->sms, 32 * COL8_WARPS, apply_smem8(g), st>>>(P);
+    } else if (apply_sharp_wide<MODE, DT, S, PHI>()) {
         apply_kernel<MODE, DT, G, S, PHI><<<g->sharp_ctas, 32 * g->sharp_warps, apply_smem(g, g->sharp_warps), st>>>(P);
     } else if (apply_plain_wide<MODE, DT, S, PHI>() && g->plain_warps > APPLY_WARPS) {
         apply_kernel<MODE, DT, G, S, PHI><<<g->plain_ctas, 32 * g->plain_warps, apply_smem(g, g->plain_warps), st>>>(P);
@@ -1045,7 +1094,7 @@ inline fft_status launch_mode_impl(fft_geom g, const ApplyParams& P, cudaStream_
     return FFT_OK;
 }
 
-// The four-column modes (stable detour only).
+// The batch modes (stable detour only).
 template <int MODE>
 inline fft_status launch_batch_impl(fft_geom g, const ApplyParams& P, cudaStream_t st) {
     FFT_CUDA(cudaMemsetAsync(g->counter, 0, 2 * sizeof(int32_t), st));
@@ -1080,13 +1129,17 @@ template <> fft_status launch_mode<MODE_COUNT>(fft_geom g, const ApplyParams& P,
 template <> fft_status launch_mode<MODE_FROB>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status launch_mode<MODE_COV>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status launch_batch<MODE_JT4>(fft_geom g, const ApplyParams& P, cudaStream_t st);
+template <> fft_status launch_batch<MODE_JT8>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status launch_batch<MODE_J4>(fft_geom g, const ApplyParams& P, cudaStream_t st);
+template <> fft_status launch_batch<MODE_J8>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status set_attr_mode<MODE_JT>(size_t smem);
 template <> fft_status set_attr_mode<MODE_J>(size_t smem);
 template <> fft_status set_attr_mode<MODE_COUNT>(size_t smem);
 template <> fft_status set_attr_mode<MODE_FROB>(size_t smem);
 template <> fft_status set_attr_mode<MODE_COV>(size_t smem);
 template <> fft_status set_attr_mode<MODE_JT4>(size_t smem);
+template <> fft_status set_attr_mode<MODE_JT8>(size_t smem);
 template <> fft_status set_attr_mode<MODE_J4>(size_t smem);
+template <> fft_status set_attr_mode<MODE_J8>(size_t smem);
 
 }  // namespace fftgb

@@ -166,8 +166,8 @@ struct fft_geom_s {
     std::vector<fftgb::StackClass> stk;
     bool stk_batch = false;
     int32_t* stk_rows = nullptr;         // [M] the slices' rows, class by class
-    float* stk_x = nullptr;              // [4 x extended voxels] columns of a pass
-    float* stk_d = nullptr;              // [4 x rows of a slice]
+    float* stk_x = nullptr;              // [columns of a pass x extended voxels]
+    float* stk_d = nullptr;              // [columns of a pass x rows of a slice]
     float* stk_jpart = nullptr;          // J partials of the operators
     float* stk_gpart = nullptr;          // their J^T partials
     int64_t stk_gpart_cap = 0;           // (floats)
@@ -195,6 +195,8 @@ struct fft_geom_s {
     int64_t evaluated = 0;
     double frob2 = -1.0;
     int64_t scratch_bytes = 0;
+    int sms = 1;                         // multiprocessors of the device
+    bool col8 = false;                   // the eight-column kernels fit beside the tables
     int apply_ctas = 0;                  // persistent grid of the apply kernels (8-warp CTAs)
     int sharp_warps = 8;                 // warps per CTA of the sharp-band single-column kernels
     int sharp_ctas = 0;                  // their persistent grid
@@ -218,8 +220,9 @@ struct fft_geom_s {
     float* vol = nullptr;                // [V] volume scratch of the 2-D apply (allocated on first use)
     float4* psf_crec = nullptr;          // candidate records of the tensor-core PSF path (grow-only)
     int64_t psf_crec_cap = 0;            // its capacity in candidates (3 float4 each)
-    float* jpart4 = nullptr;             // [E * 8 * 4] J partials of the four-column apply (first use)
-    float* gpart4 = nullptr;             // [n_slots * 4 * TILE_VOX] J^T partials of the four-column apply
+    int batch_cols = 0;                  // columns that the batch partials hold: 0 (none yet), 4 or 8
+    float* jpart4 = nullptr;             // [E * 8 * batch_cols] J partials of the batch applies
+    float* gpart4 = nullptr;             // [n_slots * batch_cols * TILE_VOX] their J^T partials
     double* cg_hist = nullptr;           // [cg_hist_cap]
     int32_t cg_hist_cap = 0;
     void* cg_graph = nullptr;            // cudaGraphExec_t of the iteration loop
@@ -241,9 +244,13 @@ bool find_stack(const double* tx, const int32_t* rows, int64_t M, const int32_t*
                 std::vector<StackPlan>& plan);
 double stack_cost(const std::vector<StackPlan>& plan, int64_t M, const fft_grid& gr);
 double stack_entries(fft_geom g, int64_t n);
+double pass_cost(int64_t cols, bool col8);
 fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st);
 fft_status stack_JT(fft_geom g, const float* d, int n, float* gout, cudaStream_t st);
 fft_status stack_scratch(fft_geom g);
+int pass_columns(fft_geom g, int64_t rem);
+int64_t batch_scratch_bytes(fft_geom g);
+void free_batch_scratch(fft_geom g);
 fft_status stack_build_items(fft_geom g, int items_per_cta);
 fft_status check_device(int dev);
 fft_status count_support(fft_geom g, int64_t* support, int64_t* evaluated);

@@ -398,22 +398,17 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
     g->n_items_plain = (int32_t)items.size();
     items.insert(items.end(), items_sharp.begin(), items_sharp.end());
     if (g->nested) g->jpart4 = g->gpart = g->gpart4 = nullptr;   // the parent's (stack_scratch sets them again)
-    if (g->items) {   // the buffers below are replaced: take them out of the scratch count
+    free_batch_scratch(g);   // rebuilt with the new slot count on first use
+    if (g->items) {          // the buffers below are replaced: take them out of the scratch count
         g->scratch_bytes -= (int64_t)(sizeof(Item) * g->n_items + 2 * sizeof(int32_t) * g->n_tiles);
         if (!g->nested) g->scratch_bytes -= (int64_t)(sizeof(float) * (size_t)g->n_slots * TILE_VOX);
-        if (g->jpart4)
-            g->scratch_bytes -= (int64_t)(sizeof(float) * ((size_t)g->E * 32 + (size_t)g->n_slots * 4 * TILE_VOX));
     }
-    void* old[] = {g->items, g->tile_slot0, g->tile_nslot, g->gpart, g->gpart4};
+    void* old[] = {g->items, g->tile_slot0, g->tile_nslot, g->gpart};
     for (void* q : old)
         if (q) cudaFree(q);
     g->items = nullptr;
     g->tile_slot0 = g->tile_nslot = nullptr;
-    g->gpart = g->gpart4 = nullptr;
-    if (g->jpart4) {   // the four-column scratch is rebuilt with the new slot count on first use
-        cudaFree(g->jpart4);
-        g->jpart4 = nullptr;
-    }
+    g->gpart = nullptr;
     g->n_items = (int32_t)items.size();
     g->n_slots = slots;
     g->items_per_cta = items_per_cta;
@@ -447,7 +442,7 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
 // (J^T partials grow with the items; the J partials do not.)
 fft_status stack_scratch(fft_geom g) {
     int64_t need = 0;
-    for (StackClass& c : g->stk) need = std::max(need, (int64_t)c.sub->n_slots * 4 * TILE_VOX);
+    for (StackClass& c : g->stk) need = std::max(need, (int64_t)c.sub->n_slots * c.sub->batch_cols * TILE_VOX);
     if (need > g->stk_gpart_cap || !g->stk_gpart) {
         cudaFree(g->stk_gpart);
         g->scratch_bytes -= (int64_t)sizeof(float) * g->stk_gpart_cap;
@@ -506,16 +501,17 @@ void build_stack(fft_geom g, const double* tx, const int32_t* rows, const int32_
         return;
     }
     const int64_t plane = (int64_t)g->grid.nx * g->grid.ny;
-    // (an operator's entries: 32 bytes of lists and 128 of partials each, about its slices' share of E)
+    // (an operator's entries: 32 bytes of lists and 256 of partials each, about a slice's share of E)
     double need = 0.0;
     for (const StackPlan& c : plan)
-        need = std::max(need, 160.0 * (double)g->E * (double)c.rows[0].size() / (double)g->M +
-                                  16.0 * (double)plane * (g->grid.nz + c.shift.back()));
+        need = std::max(need, 288.0 * (double)g->E * (double)c.rows[0].size() / (double)g->M +
+                                  32.0 * (double)plane * (g->grid.nz + c.shift.back()));
     if (2.0 * need > 0.5 * (double)mem_free) return;
     const int64_t before = g->scratch_bytes;
     std::vector<int32_t> ids;
     ids.reserve((size_t)g->M);
     int64_t v_max = 0, m_max = 0, e_max = 0;
+    int cols = 4;
     bool ok = true;
     for (const StackPlan& c : plan) {
         const int32_t top = c.shift.back();
@@ -551,6 +547,8 @@ void build_stack(fft_geom g, const double* tx, const int32_t* rows, const int32_
             ids.insert(ids.end(), c.rows[s].begin(), c.rows[s].end());
             for (int z = 0; z < g->grid.nz; ++z) ++zw[z + k.off[s]];
         }
+        k.sub->batch_cols = (c.rows.size() > 4 && k.sub->col8) ? 8 : 4;
+        cols = std::max(cols, k.sub->batch_cols);
         g->stk.push_back(k);
         ok = dmalloc(k.sub, &k.sub->zw, zw.size()) == FFT_OK &&
              cudaMemcpy(k.sub->zw, zw.data(), zw.size(), cudaMemcpyHostToDevice) == cudaSuccess;
@@ -558,21 +556,21 @@ void build_stack(fft_geom g, const double* tx, const int32_t* rows, const int32_
         g->scratch_bytes += k.sub->scratch_bytes;
         v_max = std::max(v_max, k.sub->V);
         m_max = std::max(m_max, k.sub->M);
-        e_max = std::max(e_max, k.sub->E);
+        e_max = std::max(e_max, k.sub->E * k.sub->batch_cols);
     }
     ok = ok && stack_entries(g, 1) <= 0.8 * (double)g->E_used;
     ok = ok && dmalloc(g, &g->stk_rows, ids.size()) == FFT_OK &&
          cudaMemcpy(g->stk_rows, ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
-         dmalloc(g, &g->stk_x, 4 * (size_t)v_max) == FFT_OK && dmalloc(g, &g->stk_d, 4 * (size_t)m_max) == FFT_OK &&
-         dmalloc(g, &g->stk_jpart, 32 * (size_t)e_max) == FFT_OK && stack_scratch(g) == FFT_OK;
+         dmalloc(g, &g->stk_x, cols * (size_t)v_max) == FFT_OK && dmalloc(g, &g->stk_d, cols * (size_t)m_max) == FFT_OK &&
+         dmalloc(g, &g->stk_jpart, 8 * (size_t)e_max) == FFT_OK && stack_scratch(g) == FFT_OK;
     if (!ok) {
         cudaGetLastError();
         drop_stack(g);
         g->scratch_bytes = before;
         return;
     }
-    // n columns at once: the four-column pass over all rows costs 1.45 passes
-    g->stk_batch = stack_entries(g, 4) <= 1.45 * (double)g->E_used;
+    // several columns at once: against passes of the same width over all rows
+    g->stk_batch = stack_entries(g, 8) <= pass_cost(8, g->col8) * (double)g->E_used;
 }
 
 }  // namespace

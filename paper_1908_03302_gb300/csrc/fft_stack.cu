@@ -4,14 +4,14 @@
 // grouped into classes whose members lie whole numbers of layers apart. Each class has one operator (a
 // geometry of its own, `sub`) for the rows of its lowest slice on a grid extended in z so that it
 // holds the layers of every member as that slice sees them, and J and J^T apply it to the members as
-// columns: an entry is evaluated once for four slices by the four-column kernels, and twice as rarely
+// columns: an entry is evaluated once for up to eight slices by the batch kernels, and half as often
 // again where the slice's plane mirrors the extended lattice (find_mirror).
 //
 //   J m on slice s     = sub J (m moved down by the slice's layers)
 //   J^T d              = sum over slices of (sub J^T d_s) moved up by the slice's layers
 //
 // Bound by the evaluations as the plain products are; the moves are one pass over the volume (~0.1 ms
-// of slices3d's 371 ms).
+// of slices3d's 101 ms, which was 371 with each slice's entries evaluated by themselves).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -26,35 +26,32 @@ namespace fftgb {
 
 namespace {
 
-// Up to four (column, slice) jobs that one pass of a class's operator serves.
+// Up to eight (column, slice) jobs that one pass of a class's operator serves.
+constexpr int MAX_JOBS = 8;
 struct StackJobs {
     int n;
-    int32_t col[4];           // column of the call
-    int32_t off[4];           // grid layer z of the slice is layer z + off of the extended grid
-    const int32_t* rows[4];   // the slice's rows in the order of the operator's rows
-    int32_t first[4];         // the first contribution to its column: J^T overwrites
+    int32_t col[MAX_JOBS];           // column of the call
+    int32_t off[MAX_JOBS];           // grid layer z of the slice is layer z + off of the extended grid
+    const int32_t* rows[MAX_JOBS];   // the slice's rows in the order of the operator's rows
+    int32_t first[MAX_JOBS];         // the first contribution to its column: J^T overwrites
 };
 
-// X[c][e] = m[col][e - off layers], 0 outside the grid and in columns past n.
+// X[c][e] = m[col][e - off layers], 0 outside the grid.
 __global__ void __launch_bounds__(256) stack_models_kernel(const StackJobs J, const float* __restrict__ m, int64_t V,
                                                            int64_t plane, int64_t V_ext, float* __restrict__ X) {
     const int c = blockIdx.y;
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= V_ext) return;
-    float v = 0.0f;
-    if (c < J.n) {
-        const int64_t k = e - J.off[c] * plane;
-        if (k >= 0 && k < V) v = __ldg(m + (int64_t)J.col[c] * V + k);
-    }
-    X[(int64_t)c * V_ext + e] = v;
+    const int64_t k = e - J.off[c] * plane;
+    X[(int64_t)c * V_ext + e] = (k >= 0 && k < V) ? __ldg(m + (int64_t)J.col[c] * V + k) : 0.0f;
 }
 
-// D[c][p] = d[col][rows[p]], 0 in columns past n.
+// D[c][p] = d[col][rows[p]].
 __global__ void __launch_bounds__(256) stack_gather_kernel(const StackJobs J, const float* __restrict__ d, int64_t M,
                                                            int64_t M_sub, float* __restrict__ D) {
     const int c = blockIdx.y;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < M_sub) D[(int64_t)c * M_sub + p] = c < J.n ? __ldg(d + (int64_t)J.col[c] * M + J.rows[c][p]) : 0.0f;
+    if (p < M_sub) D[(int64_t)c * M_sub + p] = __ldg(d + (int64_t)J.col[c] * M + J.rows[c][p]);
 }
 
 // d[col][rows[p]] = D[c][p].
@@ -73,7 +70,7 @@ __global__ void __launch_bounds__(256) stack_sum_kernel(const StackJobs J, const
     double s = 0.0;
     bool over = false;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
+    for (int c = 0; c < MAX_JOBS; ++c) {
         if (c >= J.n) break;
         s += (double)__ldg(Y + (int64_t)c * V_ext + v + J.off[c] * plane);
         over = over || J.first[c];
@@ -86,11 +83,6 @@ __global__ void __launch_bounds__(256) stack_sum_kernel(const StackJobs J, const
     }
 }
 
-// Four-column passes cost 1.45 single ones (ring256: 2.8 against 1.93 ms).
-constexpr double PASS4 = 1.45;
-
-double passes(int64_t jobs) { return PASS4 * (double)(jobs / 4) + (jobs % 4 == 1 ? 1.0 : (jobs % 4 ? PASS4 : 0.0)); }
-
 template <class F>
 fft_status for_each_pass(fft_geom g, int n, F&& pass) {
     for (size_t k = 0; k < g->stk.size(); ++k) {
@@ -99,7 +91,7 @@ fft_status for_each_pass(fft_geom g, int n, F&& pass) {
         const int64_t jobs = (int64_t)n * ns;
         for (int64_t j0 = 0; j0 < jobs;) {
             StackJobs J;
-            J.n = (int)std::min<int64_t>(4, jobs - j0);
+            J.n = pass_columns(C.sub, jobs - j0);
             for (int c = 0; c < J.n; ++c) {
                 const int s = (int)((j0 + c) % ns);
                 J.col[c] = (int32_t)((j0 + c) / ns);
@@ -116,6 +108,18 @@ fft_status for_each_pass(fft_geom g, int n, F&& pass) {
 }
 
 }  // namespace
+
+// Cost of a pass over jobs columns in single-column passes (slices3d, J^T: the single-, four- and
+// eight-column kernels take 25.6, 32.5 and 38.9 ms over the same rows).
+double pass_cost(int64_t jobs, bool col8) {
+    double cost = 0.0;
+    for (; jobs > 0;) {
+        const int64_t n = (jobs > 4 && col8) ? std::min<int64_t>(jobs, 8) : std::min<int64_t>(jobs, 4);
+        cost += n > 4 ? 1.52 : (n > 1 ? 1.27 : 1.0);
+        jobs -= n;
+    }
+    return cost;
+}
 
 // Groups the slices of an acquisition into classes (host only). Every row has to lie in one plane z
 // and every slice of a class to hold the same pairs (equal x and y of both transducers) and bands in the
@@ -185,7 +189,7 @@ double stack_cost(const std::vector<StackPlan>& plan, int64_t M, const fft_grid&
     for (const StackPlan& c : plan) {
         const double k = 2.0 * (c.z - gr.origin[2]) / gr.h;
         const bool mirrors = fabs(k - nearbyint(k)) <= 1e-9;
-        cost += passes((int64_t)c.rows.size()) * (double)c.rows[0].size() / (double)M * (mirrors ? 0.5 : 1.0) * (7.0 / 6.0);
+        cost += pass_cost((int64_t)c.rows.size(), true) * (double)c.rows[0].size() / (double)M * (mirrors ? 0.5 : 1.0) * (7.0 / 6.0);
     }
     return cost;
 }
@@ -193,17 +197,16 @@ double stack_cost(const std::vector<StackPlan>& plan, int64_t M, const fft_grid&
 // One J or J^T of n columns in entries evaluated (the measure that decides between the two ways).
 double stack_entries(fft_geom g, int64_t n) {
     double c = 0.0;
-    for (const StackClass& k : g->stk) c += passes(n * (int64_t)k.off.size()) * (double)k.sub->E_used;
+    for (const StackClass& k : g->stk) c += pass_cost(n * (int64_t)k.off.size(), k.sub->batch_cols == 8) * (double)k.sub->E_used;
     return c;
 }
 
 fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st) {
     const int64_t plane = (int64_t)g->grid.nx * g->grid.ny;
     return for_each_pass(g, n, [&](fft_geom sub, const StackJobs& J) -> fft_status {
-        const int nc = J.n == 1 ? 1 : 4;
-        stack_models_kernel<<<dim3((unsigned)ceil_div(sub->V, 256), nc), 256, 0, st>>>(J, m, g->V, plane, sub->V, g->stk_x);
+        stack_models_kernel<<<dim3((unsigned)ceil_div(sub->V, 256), J.n), 256, 0, st>>>(J, m, g->V, plane, sub->V, g->stk_x);
         FFT_CUDA(cudaGetLastError());
-        const fft_status rc = nc == 1 ? launch_J(sub, g->stk_x, g->stk_d, st) : launch_J_batch(sub, g->stk_x, 4, g->stk_d, st);
+        const fft_status rc = launch_J_batch(sub, g->stk_x, J.n, g->stk_d, st);
         if (rc != FFT_OK) return rc;
         stack_scatter_kernel<<<dim3((unsigned)ceil_div(sub->M, 256), J.n), 256, 0, st>>>(J, g->stk_d, sub->M, g->M, d);
         FFT_CUDA(cudaGetLastError());
@@ -214,10 +217,9 @@ fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st)
 fft_status stack_JT(fft_geom g, const float* d, int n, float* gout, cudaStream_t st) {
     const int64_t plane = (int64_t)g->grid.nx * g->grid.ny;
     return for_each_pass(g, n, [&](fft_geom sub, const StackJobs& J) -> fft_status {
-        const int nc = J.n == 1 ? 1 : 4;
-        stack_gather_kernel<<<dim3((unsigned)ceil_div(sub->M, 256), nc), 256, 0, st>>>(J, d, g->M, sub->M, g->stk_d);
+        stack_gather_kernel<<<dim3((unsigned)ceil_div(sub->M, 256), J.n), 256, 0, st>>>(J, d, g->M, sub->M, g->stk_d);
         FFT_CUDA(cudaGetLastError());
-        const fft_status rc = nc == 1 ? launch_JT(sub, g->stk_d, g->stk_x, st) : launch_JT_batch(sub, g->stk_d, 4, g->stk_x, st);
+        const fft_status rc = launch_JT_batch(sub, g->stk_d, J.n, g->stk_x, st);
         if (rc != FFT_OK) return rc;
         stack_sum_kernel<<<(unsigned)ceil_div(g->V, 256), 256, 0, st>>>(J, g->stk_x, sub->V, g->V, plane, gout);
         FFT_CUDA(cudaGetLastError());
