@@ -189,7 +189,7 @@ size_t apply_smem(fft_geom g, int warps) {
 
 size_t apply_smem(fft_geom g) { return apply_smem(g, APPLY_WARPS); }
 
-size_t apply_smem8(fft_geom g) { return apply_smem(g, 0) + (size_t)COL8_WARPS * STG_PER_WARP8 * sizeof(float4); }
+size_t apply_smem8(fft_geom g, int warps) { return apply_smem(g, 0) + (size_t)warps * STG_PER_WARP8 * sizeof(float4); }
 
 // Most warps (a multiple of 8, at most 24) one sharp-variant CTA can stage for.
 static int sharp_max_warps(fft_geom g) {
@@ -228,10 +228,11 @@ fft_status set_apply_attributes(fft_geom g) {
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, dev);
     g->sms = std::max(g->sms, 1);
-    g->col8 = g->dt_mode == FFT_DT_STABLE && apply_smem8(g) <= (size_t)optin;
+    const size_t smem8 = apply_smem8(g, col8_warps<false>());
+    g->col8 = g->dt_mode == FFT_DT_STABLE && smem8 <= (size_t)optin;
     if (g->col8) {
-        if ((rc = set_attr_mode<MODE_JT8>(apply_smem8(g))) != FFT_OK) return rc;
-        if ((rc = set_attr_mode<MODE_J8>(apply_smem8(g))) != FFT_OK) return rc;
+        if ((rc = set_attr_mode<MODE_JT8>(smem8)) != FFT_OK) return rc;
+        if ((rc = set_attr_mode<MODE_J8>(smem8)) != FFT_OK) return rc;
     }
     return set_attr_mode<MODE_FROB>(smem);
 }

@@ -45,10 +45,14 @@ enum { MODE_JT = 0, MODE_J = 1, MODE_COUNT = 2, MODE_FROB = 3, MODE_COV = 4, MOD
        MODE_J8 = 8 };
 constexpr int STG_PER_WARP = 128;    // staged float4 per warp: 32 rows x (3 or 4)
 constexpr int STG_PER_WARP8 = 160;   // the eight-column J^T: 32 rows x 5
-// CTA of the eight-column kernels: one of 12 warps per SM, up to 168 registers (64 of them hold a lane's
-// accumulators or model values: 8 voxels x 8 columns). Fewer warps than the four-column kernels' 16
-// hide less latency, yet an entry's evaluation serves twice the columns: 1.2 times the time a pass.
-constexpr int COL8_WARPS = 12;
+// CTA of the eight-column kernels: one per SM, of 16 warps at 128 registers (64 of them hold a lane's
+// accumulators or model values: 8 voxels x 8 columns), the sharp-band ones of 12 at 168, which
+// would spill 600 bytes at 128. With 12 warps the plain ones were bound by latency (issue slots 59 %
+// active): ring256, block of 8 columns, J and J^T 6.91 -> 6.13 ms, slices3d J^T 100.9 -> 96.4 ms.
+template <bool SHARP>
+constexpr int col8_warps() {
+    return SHARP ? 12 : 16;
+}
 
 template <int MODE>
 constexpr int apply_ncol() {
@@ -450,7 +454,7 @@ constexpr int PLAIN_MAX_WARPS = 24;
 
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr int apply_block_bound() {
-    return apply_ncol<MODE>() == 8                    ? 32 * COL8_WARPS
+    return apply_ncol<MODE>() == 8                    ? 32 * col8_warps<SHARP>()
            : apply_sharp_wide<MODE, DT, SHARP, PHI>() ? 32 * SHARP_MAX_WARPS
            : apply_plain_wide<MODE, DT, SHARP, PHI>() ? 32 * PLAIN_MAX_WARPS
                                                       : APPLY_THREADS;
@@ -1022,7 +1026,7 @@ inline fft_status set_attr_mode_impl(size_t smem) {
 }
 
 size_t apply_smem(fft_geom g, int warps);
-size_t apply_smem8(fft_geom g);
+size_t apply_smem8(fft_geom g, int warps);
 // Resident CTAs per SM of the J^T kernel (stable detour, tables; plain or sharp).
 int apply_blocks_per_sm(bool sharp, int threads, size_t smem);
 
@@ -1032,7 +1036,7 @@ int apply_blocks_per_sm(bool sharp, int threads, size_t smem);
 template <int MODE, int DT, bool G, bool S, int PHI>
 inline void launch_apply(fft_geom g, const ApplyParams& P, cudaStream_t st) {
     if (apply_ncol<MODE>() == 8) {
-        apply_kernel<MODE, DT, G, S, PHI><<<g->sms, 32 * COL8_WARPS, apply_smem8(g), st>>>(P);
+        apply_kernel<MODE, DT, G, S, PHI><<<g->sms, 32 * col8_warps<S>(), apply_smem8(g, col8_warps<S>()), st>>>(P);
     } else if (apply_sharp_wide<MODE, DT, S, PHI>()) {
         apply_kernel<MODE, DT, G, S, PHI><<<g->sharp_ctas, 32 * g->sharp_warps, apply_smem(g, g->sharp_warps), st>>>(P);
     } else if (apply_plain_wide<MODE, DT, S, PHI>() && g->plain_warps > APPLY_WARPS) {
