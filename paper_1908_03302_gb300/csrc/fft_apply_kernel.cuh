@@ -211,7 +211,8 @@ enum { FORM_GENERAL = 0, FORM_INNER = 1, FORM_DEEP = 2 };
 
 // Staged flag word: band (bits 0-7), sharp band (8), planar pair (9), and per sub-brick s of the
 // unit: the row may reach it (12 + s), it is inner (16 + s), it is deep (20 + s); and per z layer h
-// of the unit (sub-bricks 2 h and 2 h + 1): both are reached and deep (24 + h).
+// of the unit (sub-bricks 2 h and 2 h + 1): both are reached and deep (24 + h). In the support count also:
+// the support holds the sub-brick whole (28 + s).
 __device__ __forceinline__ int form_of(uint32_t cw, int s) {
     return ((cw >> (20 + s)) & 1u) ? FORM_DEEP : (((cw >> (16 + s)) & 1u) ? FORM_INNER : FORM_GENERAL);
 }
@@ -627,18 +628,23 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const float lam = 2.0f * hl;
                 const float rim = hl - (4.1f + DEEP_MARGIN) * hb;
                 const float rim2 = (DT == FFT_DT_STABLE && lam >= DEEP_MIN_L && rim > 0.0f) ? rim * rim : -1.0f;
-                uint32_t inb = 0, dpb = 0;
+                uint32_t inb = 0, dpb = 0, full = 0;
 #pragma unroll
                 for (int s = 0; s < NSUB; ++s) {
                     const float cy = fmaf(8.0f * wy + (float)sub_dy<NSUB>(s) + 1.5f, hb, dy);
                     const float cz = fmaf(4.0f * wz + (float)sub_dz<NSUB>(s) + 1.5f, hb, dz);
                     if (live && ((sub_ok >> s) & 1u) && box_may_touch(cx, cy, cz, ex, ey, ez, hl, hxx, hyy, hyy))
                         okb |= 1u << s;
+                    // the support count takes sub-bricks that the support holds whole as they are
+                    // (a ring of 256 calibrated elements: 3.41 -> 2.63 ms)
+                    if (MODE == MODE_COUNT && DT != FFT_DT_FP64 && ((okb >> s) & 1u) &&
+                        box_inside(cx, cy, cz, ex, ey, ez, hl, hxx, hyy, hyy))
+                        full |= 1u << s;
                     // sub-bricks whose voxels all satisfy |p| <= hl (between the transducer planes)
                     if (fabsf(fmaf(cx, ex, fmaf(cy, ey, cz * ez))) + pext <= hl) inb |= 1u << s;
                     if (fmaf(cx, cx, fmaf(cy, cy, cz * cz)) <= rim2) dpb |= 1u << s;
                 }
-                const uint32_t od = okb & dpb, both = ((od & 3u) == 3u ? 1u : 0u) | ((od & 12u) == 12u ? 2u : 0u);
+                const uint32_t od = okb & dpb & ~full, both = ((od & 3u) == 3u ? 1u : 0u) | ((od & 12u) == 12u ? 2u : 0u);
                 stg[lane * SR + 0] = base;
                 stg[lane * SR + 1] = make_float4(r.c.x, r.c.y, r.c.z, base3);
                 // planar pair (both transducers at one z): stepping along x changes only c3
@@ -650,7 +656,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                                     : fmaf((float)(b * (PHI == PHI_SEG ? P.seg_n + SEG_PAD : P.n_tab)), MAGIC2_ULP, MAGIC2);
                 stg[lane * SR + 2] = make_float4(W, row_m, DT == FFT_DT_FP64 ? __int_as_float(p) : lam,
                                                  __int_as_float(b | (bc.sharp << 8) | (planar << 9) |
-                                                                (int)((okb << 12) | (inb << 16) | (dpb << 20) | (both << 24))));
+                                                                (int)((okb << 12) | (inb << 16) | (dpb << 20) | (both << 24) | (full << 28))));
                 if (JTN) {
 #pragma unroll
                     for (int k = 0; k < NC / 4; ++k)
@@ -790,6 +796,10 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         for (int q = 0; q < 2; ++q) {
                             const int s = 2 * h + q;
                             if (!((cw >> (12 + s)) & 1u)) continue;
+                            if (MODE == MODE_COUNT && ((cw >> (28 + s)) & 1u)) {
+                                n_in += (uint32_t)__popc((vmask >> (4 * s)) & 15u) * 0x10001u * ((mult >> (8 * s)) & 255u);
+                                continue;
+                            }
                             f2 v[2], w[2];
                             if (DT == FFT_DT_FP64) {
                                 const RowRec64 r64 = P.rec64[__float_as_int(C.z)];

@@ -138,6 +138,22 @@ __device__ __forceinline__ bool box_may_touch(float dx, float dy, float dz, floa
     return !(ok && lb1 >= 1.0f + CULL_MARGIN);
 }
 
+// Does the support {R < 1} hold a whole box (arguments as in box_may_touch)? R is convex: its largest
+// value over the box is at a corner. The margin covers the FP32 rounding of R here and in the kernels.
+__device__ __forceinline__ bool box_inside(float dx, float dy, float dz, float ex, float ey, float ez, float hl,
+                                           float hx, float hy, float hz) {
+    float m = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float x = dx + ((c & 1) ? hx : -hx), y = dy + ((c & 2) ? hy : -hy), z = dz + ((c & 4) ? hz : -hz);
+        const float sx = fmaf(hl, ex, x), sy = fmaf(hl, ey, y), sz = fmaf(hl, ez, z);
+        const float rx = fmaf(-hl, ex, x), ry = fmaf(-hl, ey, y), rz = fmaf(-hl, ez, z);
+        const float ss = fmaxf(fmaf(sx, sx, fmaf(sy, sy, sz * sz)), 1e-12f), rr = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-12f);
+        m = fmaxf(m, fmaf(ss, rsqrt_approx(ss), rr * rsqrt_approx(rr)));
+    }
+    return m - 2.0f * hl < 1.0f - 1e-3f;
+}
+
 // Normalised detour v = R / U in [0, 1] (saturated) and the two inverse distances, from
 // the pair-frame coordinates of a voxel centre: p = (x - o).e, q2 = |(x - o) x e|^2.
 //   STABLE: R = q2 (A + B) / (A B) + E with A = R_xs + |p + hl|, B = R_xr + |p - hl| and

@@ -136,30 +136,45 @@ __global__ void tile_fill_kernel(const CullParams C, const int64_t* __restrict__
 // FP64 pair-frame coordinates of each entry's tile origin (voxel (TX, TY, TZ) centre) in band
 // units: p = (x_T - o).e and c = (x_T - o) x e. Computing them here in double precision keeps
 // the large (~L/2) coordinates out of FP32 arithmetic; the kernels add only small offsets.
+// The rows' frames come from a pass of their own: the square root and the divisions, an entry's most
+// expensive FP64 operations, once per row instead of once per entry (ring256: 0.75 -> 0.20 ms).
+struct RowFrame {
+    double o[3], e[3];   // pair midpoint (m), unit axis
+    double hl, inv_u;    // half pair length (band units), 1 / U
+};
+__global__ void row_frame_kernel(const double* __restrict__ tx, const int32_t* __restrict__ pairs,
+                                 const int32_t* __restrict__ row_band, const BandConst* __restrict__ bc, int64_t M,
+                                 RowFrame* __restrict__ frame) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= M) return;
+    const double* xs = tx + 3 * (int64_t)pairs[2 * p];
+    const double* xr = tx + 3 * (int64_t)pairs[2 * p + 1];
+    const double U = bc[row_band[p]].U;
+    const double ax = xr[0] - xs[0], ay = xr[1] - xs[1], az = xr[2] - xs[2];
+    const double L = sqrt(ax * ax + ay * ay + az * az);
+    RowFrame f;
+    for (int a = 0; a < 3; ++a) f.o[a] = 0.5 * (xs[a] + xr[a]);
+    f.e[0] = ax / L;
+    f.e[1] = ay / L;
+    f.e[2] = az / L;
+    f.hl = 0.5 * L / U;
+    f.inv_u = 1.0 / U;
+    frame[p] = f;
+}
+
 __global__ void entry_base_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ rows_of_entry,
-                                  const double* __restrict__ tx, const int32_t* __restrict__ pairs,
-                                  const int32_t* __restrict__ row_band, const BandConst* __restrict__ bc,
-                                  double ox, double oy, double oz, double h, int tiles_x, int tiles_y,
-                                  float4* __restrict__ ebase, float* __restrict__ ebase3) {
+                                  const RowFrame* __restrict__ frame, double ox, double oy, double oz, double h,
+                                  int tiles_x, int tiles_y, float4* __restrict__ ebase, float* __restrict__ ebase3) {
     const int T = blockIdx.x;
     const int tx_ = T % tiles_x, ty_ = (T / tiles_x) % tiles_y, tz_ = T / (tiles_x * tiles_y);
     const double xT = ox + (double)(TILE_X * tx_) * h;
     const double yT = oy + (double)(TILE_Y * ty_) * h;
     const double zT = oz + (double)(TILE_Z * tz_) * h;
     for (int64_t e = off[T] + threadIdx.x; e < off[T + 1]; e += blockDim.x) {
-        const int p = rows_of_entry[e];
-        const double* xs = tx + 3 * (int64_t)pairs[2 * p];
-        const double* xr = tx + 3 * (int64_t)pairs[2 * p + 1];
-        const double U = bc[row_band[p]].U;
-        double ax = xr[0] - xs[0], ay = xr[1] - xs[1], az = xr[2] - xs[2];
-        const double L = sqrt(ax * ax + ay * ay + az * az);
-        ax /= L;
-        ay /= L;
-        az /= L;
-        const double dx = (xT - 0.5 * (xs[0] + xr[0])) / U;
-        const double dy = (yT - 0.5 * (xs[1] + xr[1])) / U;
-        const double dz = (zT - 0.5 * (xs[2] + xr[2])) / U;
-        const double pp = dx * ax + dy * ay + dz * az, hl = 0.5 * L / U;
+        const RowFrame f = frame[rows_of_entry[e]];
+        const double ax = f.e[0], ay = f.e[1], az = f.e[2];
+        const double dx = (xT - f.o[0]) * f.inv_u, dy = (yT - f.o[1]) * f.inv_u, dz = (zT - f.o[2]) * f.inv_u;
+        const double pp = dx * ax + dy * ay + dz * az, hl = f.hl;
         // p + hl and p - hl are the axial offsets from the emitter and the receiver; forming
         // them here keeps them exact when small (voxels near a transducer)
         ebase[e] = make_float4((float)(pp + hl), (float)(pp - hl), (float)(dy * az - dz * ay),
@@ -868,14 +883,17 @@ fft_status create_geom(const double* tx_xyz, int32_t n_tx, const int32_t* rows, 
         if (e == cudaSuccess) e = cudaMalloc(&d_pairs, sizeof(int32_t) * 2 * n_rows);
         if (e == cudaSuccess) e = cudaMemcpy(d_tx, tx_xyz, sizeof(double) * 3 * n_tx, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(d_pairs, rows, sizeof(int32_t) * 2 * n_rows, cudaMemcpyHostToDevice);
+        RowFrame* d_frame = nullptr;
+        if (e == cudaSuccess) e = cudaMalloc(&d_frame, sizeof(RowFrame) * n_rows);
         if (e == cudaSuccess) {
-            entry_base_kernel<<<(unsigned)g->n_tiles, 256>>>(g->tile_off, g->tile_rows, d_tx, d_pairs, g->row_band,
-                                                             g->d_band, grid->origin[0], grid->origin[1],
-                                                             grid->origin[2], grid->h, g->tiles[0], g->tiles[1],
-                                                             g->ebase, g->ebase3);
+            row_frame_kernel<<<(unsigned)ceil_div(n_rows, 128), 128>>>(d_tx, d_pairs, g->row_band, g->d_band, n_rows, d_frame);
+            entry_base_kernel<<<(unsigned)g->n_tiles, 256>>>(g->tile_off, g->tile_rows, d_frame, grid->origin[0],
+                                                             grid->origin[1], grid->origin[2], grid->h, g->tiles[0],
+                                                             g->tiles[1], g->ebase, g->ebase3);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        cudaFree(d_frame);
         cudaFree(d_tx);
         cudaFree(d_pairs);
         GEOM_CUDA(e);
