@@ -72,13 +72,10 @@ constexpr int D_LANES = 16;            // lanes that scatter one row's D entries
 constexpr long long WAIT_BUDGET = 4000000000ll;   // cycles (~2 s)
 constexpr int HDR_UFIRST = 1, HDR_LAST = 2, HDR_GFIRST = 4;   // chunk header flags
 constexpr int MAX_NG = 256;            // MMA N (spikes of one launch, rounded up to 16)
-// Stand-in for a row past a chunk's end: a voxel line at distance FAR from the axis of a pair of
-// length 2 FAR_HL and at its midplane (in band units), so that every detour form gives v >> 1, saturated
-// to the cut-off: Phi = 0, and the geometric factor stays finite. (R = 181; the deep form's y is 50, its
-// polynomial positive.)
-constexpr float FAR = 100.0f, FAR_HL = 10.0f;
-// Form flags in the low bits of a staged row's table address (a multiple of 8)
-constexpr uint32_t ROW_INNER = 1u, ROW_PLANAR = 2u, ROW_DEEP = 4u;
+// Stand-in for a row past a chunk's end: a voxel line at distance FAR from the pair's axis and
+// at its midplane (in band units), so that every detour form gives v = 2 FAR, saturated to the
+// cut-off: Phi = 0, and the geometric factor stays finite.
+constexpr float FAR = 1.0e4f;
 static_assert(GEN_WARPS == 2 * ROW_OCTETS && D_ROWS == 4, "generator warps: 8 rows x 64 voxels");
 
 // Zero page the MMA warp copies over a consumed B tile (static storage: zero-initialised).
@@ -179,14 +176,14 @@ __device__ __forceinline__ bool warp_wait(uint32_t mbar, uint32_t parity, int32_
 // Producer side, called by the scan warp that holds the turn (whole warp): publish chunk
 // `chunk` (lane 0 writes the header and arrives on its "ring full" barrier). The rows past
 // n_rows get the stand-in record (a voxel line FAR from the pair's axis, no D entries, table
-// base `tb_safe` with every form flag), so that the generators load every row of a
+// base `tb_safe` with both detour-form flags), so that the generators load every row of a
 // chunk alike and the stand-ins contribute exact zeros.
 __device__ __forceinline__ void publish_chunk(TcShared& S, float4* s_ring, uint32_t ring_full0, int chunk, int unit,
                                               int n_rows, int flags, int group, uint32_t tb_safe, int lane) {
     if (n_rows >= 0) {
         float4* dst = s_ring + (size_t)(chunk % RING) * KC * 3;
         for (int r = n_rows + lane; r < KC; r += 32) {
-            dst[3 * r + 0] = make_float4(FAR_HL, -FAR_HL, FAR, 0.f);
+            dst[3 * r + 0] = make_float4(0.f, 0.f, FAR, 0.f);
             dst[3 * r + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
             dst[3 * r + 2] = make_float4(0.f, __uint_as_float(tb_safe), 0.f, 0.f);
         }
@@ -323,53 +320,6 @@ __global__ void __launch_bounds__(MASK_THREADS) psf_mask_kernel(const PsfTcParam
     if (threadIdx.x == 0) c_or[T] = (uint16_t)s_or;
 }
 
-// Two rows (a, b) on the eight voxels of an x line, deep inside both pairs' spheres: the form of
-// eval_deep, two rows per packed instruction, so that a packed value is the K pair the A tile stores.
-// The axis offset c3 (and c2), -X and its difference are stepped along the line (eight steps of FP32
-// rounding, far below the BF16 of the entries). Issue-bound: 15.5 instructions per entry against 23;
-// 384 PSFs of ring256 with three bands 12.3 -> 11.8 ms.
-template <bool PL>
-__device__ __forceinline__ void deep_line(f2 ps, f2 pr, f2 c1q, f2 c2, f2 c3, f2 hx, f2 hy, f2 hz, uint32_t tba,
-                                          uint32_t tbb, float nm1, unsigned char* aw) {
-    const f2 lam = add2(ps, neg2(pr)), l2 = mul2(lam, lam);
-    // c2 and c3 at the voxels t step by -h_z and h_y; X by b + h^2 (2 t + 1)
-    f2 g = mul2(c3, hy), hh = fma2(hx, hx, mul2(hy, hy));
-    f2 c12 = c1q;
-    if (PL) {
-        c12 = fma2(c2, c2, c1q);
-    } else {
-        g = fma2(neg2(c2), hz, g);
-        hh = fma2(hz, hz, hh);
-    }
-    const f2 q20 = PL ? fma2(c3, c3, c12) : fma2(c3, c3, fma2(c2, c2, c12));
-    f2 Xn = neg2(fma2(ps, pr, q20));
-    f2 dX = neg2(add2(fma2(pk1(2.0f), g, mul2(hx, add2(ps, pr))), hh));
-    const f2 ddX = mul2(pk1(-2.0f), hh);
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        const f2 q2 = PL ? fma2(c3, c3, c12) : fma2(c3, c3, fma2(c2, c2, c12));
-        const f2 D = fma2(Xn, Xn, mul2(l2, q2));
-        const f2 w = rsqrt2(D);
-        const f2 y = mul2(q2, rcp2(fma2(D, w, Xn)));
-        f2 Q = fma2(pk1(DEEP_C5), y, pk1(DEEP_C4));
-        Q = fma2(Q, y, pk1(DEEP_C3));
-        Q = fma2(Q, y, pk1(DEEP_C2));
-        Q = fma2(Q, y, pk1(1.0f));
-        const float2 ly = up(mul2(lam, y)), q = up(Q);
-        const float va = __saturatef(ly.x * q.x), vb = __saturatef(ly.y * q.y);
-        const float2 tt = up(fma2_rd(pk(va, vb), pk1(nm1), pk1(MAGIC)));
-        const float2 Ta = lds_f2(tba + (__float_as_uint(tt.x) << 3)), Tb = lds_f2(tbb + (__float_as_uint(tt.y) << 3));
-        const float2 val = up(mul2(pk(fmaf(va, Ta.y, Ta.x), fmaf(vb, Tb.y, Tb.x)), w));
-        *reinterpret_cast<uint32_t*>(aw + t * 16 * KC) = pack_bf16x2(val.x, val.y);
-        if (t < 7) {
-            c3 = add2(c3, hy);
-            if (!PL) c2 = add2(c2, neg2(hz));
-            Xn = add2(Xn, dX);
-            dX = add2(dX, ddX);
-        }
-    }
-}
-
 // GUARD: some voxel centre lies on a transducer (the geometry's flag): the guarded detour.
 template <bool GUARD>
 __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_constant__ PsfTcParams P) {
@@ -394,7 +344,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
         for (uint32_t i = tid; i < NSTAGE * b_bytes / 16; i += TC_THREADS) b4[i] = make_uint4(0, 0, 0, 0);
     }
     const uint32_t tab_addr = smem_addr(s_tab);
-    const uint32_t tb_safe = (tab_addr - MAGIC_BITS_X8) | ROW_INNER | ROW_PLANAR | ROW_DEEP;   // band 0
+    const uint32_t tb_safe = (tab_addr - MAGIC_BITS_X8) | 3u;   // band 0, both detour-form flags
     const float nm1 = (float)(P.n_tab - 1);
     const uint32_t full0 = smem_addr(&S.full[0]), empty0 = smem_addr(&S.empty[0]), done0 = smem_addr(&S.done[0]);
     const uint32_t ring_full0 = smem_addr(&S.ring_full[0]), ring_empty0 = smem_addr(&S.ring_empty[0]);
@@ -527,18 +477,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
                     const float pc = fmaf((float)(SXo + 3.5f), hx, fmaf((float)(SYo + 1.5f), hy, fmaf((float)(SZo + 1.5f), hz, p0)));
                     const float pext = 3.5f * fabsf(hx) + 1.5f * (fabsf(hy) + fabsf(hz)) + 1e-3f;
                     const bool inner = fabsf(pc) + pext <= hl;
-                    // deep inside the pair's sphere (the test of the J / J^T kernels)? c at the
-                    // centre gives its distance from the axis
+                    // table base (a multiple of 8) with the inner / planar flags in bits 0, 1
                     const uint32_t bnd = (uint32_t)__float_as_int(s2.y);
-                    const float c1 = fmaf(SYo + 1.5f, hz, fmaf(-(SZo + 1.5f), hy, s0.z));
-                    const float c2 = fmaf(SZo + 1.5f, hx, fmaf(-(SXo + 3.5f), hz, s0.w));
-                    const float c3 = fmaf(SXo + 3.5f, hy, fmaf(-(SYo + 1.5f), hx, s1.w));
-                    const float rim = hl - (4.1f + DEEP_MARGIN) * S.bc[bnd].h;
-                    const bool deep = !GUARD && 2.0f * hl >= DEEP_MIN_L && rim > 0.0f &&
-                                      fmaf(pc, pc, fmaf(c1, c1, fmaf(c2, c2, c3 * c3))) <= rim * rim;
-                    // table base (a multiple of 8) with the form flags
-                    const uint32_t tb = (tab_addr + bnd * (uint32_t)P.n_tab * 8u - MAGIC_BITS_X8) |
-                                        (inner ? ROW_INNER : 0u) | (hz == 0.0f ? ROW_PLANAR : 0u) | (deep ? ROW_DEEP : 0u);
+                    const uint32_t tb = (tab_addr + bnd * (uint32_t)P.n_tab * 8u - MAGIC_BITS_X8) | (inner ? 1u : 0u) |
+                                        (hz == 0.0f ? 2u : 0u);
                     s2.y = __uint_as_float(tb);
                 }
                 const uint32_t bal = __ballot_sync(0xffffffffu, keep);
@@ -672,7 +614,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
             const uint32_t ta = __float_as_uint(stg[ra * 3 + 2].y);
             const float4 Ab = stg[ra * 3 + 3], Bb = stg[ra * 3 + 4];
             const uint32_t tbb = __float_as_uint(stg[ra * 3 + 5].y);
-            const uint32_t wfl = __reduce_and_sync(0xffffffffu, ta & tbb) & (ROW_INNER | ROW_PLANAR | ROW_DEEP);
+            const uint32_t fl = ta & tbb & 3u;
+            const uint32_t wfl = (__all_sync(0xffffffffu, fl & 1u) ? 1u : 0u) | (__all_sync(0xffffffffu, fl & 2u) ? 2u : 0u);
             const float Xv = (float)SX, Yv = (float)SY + Yv0, Zv = (float)SZ + Zv0;
             // pair-frame values of each row at voxel t = 0 of the lane's line
             const float oa = fmaf(Xv, Ba.x, fmaf(Yv, Ba.y, Zv * Ba.z)), ob = fmaf(Xv, Bb.x, fmaf(Yv, Bb.y, Zv * Bb.z));
@@ -681,7 +624,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
             const float c2a = fmaf(Zv, Ba.x, fmaf(-Xv, Ba.z, Aa.w)), c2b = fmaf(Zv, Bb.x, fmaf(-Xv, Bb.z, Ab.w));
             const float c3a = fmaf(Xv, Ba.y, fmaf(-Yv, Ba.x, Ba.w)), c3b = fmaf(Xv, Bb.y, fmaf(-Yv, Bb.x, Bb.w));
             const float c1qa = c1a * c1a, c1qb = c1b * c1b;
-            const uint32_t tba = ta & ~7u, tbbb = tbb & ~7u;
+            const float c12a = fmaf(c2a, c2a, c1qa), c12b = fmaf(c2b, c2b, c1qb);
+            const uint32_t tba = ta & ~3u, tbbb = tbb & ~3u;
             unsigned char* aw = sA + a_off0;
             // warp-uniform choice of the detour form for the whole line
 #define FFT_TC_LINE(INNER_V, PLANAR_V)                                                                 \
@@ -690,8 +634,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
         float q2a, q2b;                                                                               \
         const float c3ta = fmaf(ft, Ba.y, c3a), c3tb = fmaf(ft, Bb.y, c3b);                           \
         if (PLANAR_V) {                                                                               \
-            q2a = fmaf(c3ta, c3ta, fmaf(c2a, c2a, c1qa));                                                             \
-            q2b = fmaf(c3tb, c3tb, fmaf(c2b, c2b, c1qb));                                                             \
+            q2a = fmaf(c3ta, c3ta, c12a);                                                             \
+            q2b = fmaf(c3tb, c3tb, c12b);                                                             \
         } else {                                                                                      \
             const float c2ta = fmaf(-ft, Ba.z, c2a), c2tb = fmaf(-ft, Bb.z, c2b);                     \
             q2a = fmaf(c2ta, c2ta, fmaf(c3ta, c3ta, c1qa));                                           \
@@ -706,21 +650,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
         const float yb = phi_lookup(vib, tbbb, nm1) * (isb * irb);                                   \
         *reinterpret_cast<uint32_t*>(aw + t * 16 * KC) = pack_bf16x2(ya, yb);                        \
     }
-            if (wfl & ROW_DEEP) {
-                const f2 hy = pk(Ba.y, Bb.y), hx = pk(Ba.x, Bb.x), hz = pk(Ba.z, Bb.z);
-                const f2 ps = pk(psa, psb), pr = pk(pra, prb);
-                if (wfl & ROW_PLANAR)
-                    deep_line<true>(ps, pr, pk(c1qa, c1qb), pk(c2a, c2b), pk(c3a, c3b), hx, hy, hz, tba, tbbb, nm1, aw);
-                else
-                    deep_line<false>(ps, pr, pk(c1qa, c1qb), pk(c2a, c2b), pk(c3a, c3b), hx, hy, hz, tba, tbbb, nm1, aw);
-            } else if (wfl & ROW_INNER) {
-                if (wfl & ROW_PLANAR) {
+            if (wfl & 1u) {
+                if (wfl & 2u) {
                     FFT_TC_LINE(true, true)
                 } else {
                     FFT_TC_LINE(true, false)
                 }
             } else {
-                if (wfl & ROW_PLANAR) {
+                if (wfl & 2u) {
                     FFT_TC_LINE(false, true)
                 } else {
                     FFT_TC_LINE(false, false)
