@@ -102,7 +102,6 @@ struct PsfTcParams {
     int32_t* counter;
     int tiles_x, tiles_y;
     int nx, ny, nz;
-    int z_lo, z_end, mirror;   // layers to generate, mirror plane (fft_geom_s)
     const int64_t* d_off;      // sparse D rows: [M + 1]
     const uint32_t* d_ent;     // entry: spike index k (bits 0-15) | BF16 of C_p J[p, spike_k] (16-31)
     int ng;                    // MMA N: columns of one group (multiple of 16, <= MAX_NG)
@@ -210,14 +209,6 @@ __device__ __forceinline__ bool ring_slot_free(uint32_t ring_empty0, int chunk, 
 
 constexpr int MASK_THREADS = 256;
 
-// Does tile T hold layers that are generated? (Y = J^T D is the same on a layer and its mirror image, as
-// J's entries are: fft_geom_s. Generating one of the two halves the units and the candidate lists: 384
-// PSFs of ring256 with three bands 22.4 -> 12.3 ms.)
-__device__ __forceinline__ bool tile_generated(const PsfTcParams& P, int T) {
-    const int Z0 = TILE_Z * (T / (P.tiles_x * P.tiles_y));
-    return Z0 < P.z_end && Z0 + TILE_Z > P.z_lo;
-}
-
 // Capacity of each (tile, group) candidate segment: the tile's entries whose row has D
 // entries, by the row's group (an upper bound of the compact candidates psf_mask_kernel keeps).
 __global__ void __launch_bounds__(MASK_THREADS) psf_cap_kernel(const PsfTcParams P, int32_t* __restrict__ cap) {
@@ -225,8 +216,7 @@ __global__ void __launch_bounds__(MASK_THREADS) psf_cap_kernel(const PsfTcParams
     const int T = P.tile_order[blockIdx.x], G = P.n_groups;
     if (threadIdx.x < PSF_TC_MAX_GROUPS) s_cnt[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t e_end = tile_generated(P, T) ? P.tile_off[T + 1] : P.tile_off[T];
-    for (int64_t e = P.tile_off[T] + threadIdx.x; e < e_end; e += MASK_THREADS) {
+    for (int64_t e = P.tile_off[T] + threadIdx.x; e < P.tile_off[T + 1]; e += MASK_THREADS) {
         const int p = P.tile_rows[e];
         if (P.d_off[p + 1] > P.d_off[p]) atomicAdd(&s_cnt[P.grp[p]], 1);
     }
@@ -235,7 +225,7 @@ __global__ void __launch_bounds__(MASK_THREADS) psf_cap_kernel(const PsfTcParams
 }
 
 // Compact candidate lists, one CTA per tile: the tile's candidate rows that have D entries,
-// each with the mask of its 16 sub-bricks (8 x 4 x 4, inside the grid, layers to generate) that the row's support
+// each with the mask of its 16 sub-bricks (8 x 4 x 4, inside the grid) that the row's support
 // may reach (tangent-plane bound of the convex detour, as in the J^T kernel), written by group
 // from seg_off[T * G + g] in candidate order; c_cnt[T * G + g] their number and c_or[T] the
 // union of the masks. With each candidate goes its staging record, so that the scan warps
@@ -252,7 +242,7 @@ __global__ void __launch_bounds__(MASK_THREADS) psf_mask_kernel(const PsfTcParam
     const int T = P.tile_order[blockIdx.x], G = P.n_groups;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tx = T % P.tiles_x, ty = (T / P.tiles_x) % P.tiles_y, tz = T / (P.tiles_x * P.tiles_y);
-    const int64_t e_begin = P.tile_off[T], e_end = tile_generated(P, T) ? P.tile_off[T + 1] : e_begin;
+    const int64_t e_begin = P.tile_off[T], e_end = P.tile_off[T + 1];
     if (threadIdx.x == 0) s_or = 0u;
     if (threadIdx.x < PSF_TC_MAX_GROUPS) run[threadIdx.x] = 0;
     __syncthreads();
@@ -278,7 +268,7 @@ __global__ void __launch_bounds__(MASK_THREADS) psf_mask_kernel(const PsfTcParam
                 for (int sb = 0; sb < 16; ++sb) {
                     const int X0 = TILE_X * tx + 8 * (sb & 1), Y0 = TILE_Y * ty + 4 * ((sb >> 1) & 3),
                               Z0 = TILE_Z * tz + 4 * (sb >> 3);
-                    if (X0 >= P.nx || Y0 >= P.ny || Z0 >= P.z_end || Z0 + 3 < P.z_lo) continue;
+                    if (X0 >= P.nx || Y0 >= P.ny || Z0 >= P.nz) continue;
                     const float cx = fmaf((float)(X0) + 3.5f, hb, bc.org[0]) - r.a.x;
                     const float cy = fmaf((float)(Y0) + 1.5f, hb, bc.org[1]) - r.a.y;
                     const float cz = fmaf((float)(Z0) + 1.5f, hb, bc.org[2]) - r.a.z;
@@ -703,8 +693,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
                 const int eg = lane & 7;
                 const int x = X0 + 4 * (quarter & 1) + (lane >> 3), y = Y0 + (eg & 3),
                           z = Z0 + 2 * (quarter >> 1) + (eg >> 2);
-                const bool valid = x < P.nx && y < P.ny && z >= P.z_lo && z < P.z_end;
-                const int64_t mo = (int64_t)mirror_step(P.mirror, z, P.nz) * P.ny * P.nx;   // (0: no image)
+                const bool valid = x < P.nx && y < P.ny && z < P.nz;
                 const int64_t v = ((int64_t)z * P.ny + y) * P.nx + x;
                 const uint32_t lane_base = taddr + ((uint32_t)(32 * quarter) << 16);
                 for (int c = 8 * (warp >> 2); c < P.nk; c += 8 * (GEN_WARPS / 4)) {
@@ -723,10 +712,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
                             float* o = P.out + ((int64_t)s * P.n_spike + P.k0 + c) * P.V + v;
 #pragma unroll
                             for (int i = 0; i < 8; ++i)
-                                if (c + i < P.nk) {
-                                    o[(int64_t)i * P.V] = acc[i];
-                                    if (mo != 0) o[(int64_t)i * P.V + mo] = acc[i];
-                                }
+                                if (c + i < P.nk) o[(int64_t)i * P.V] = acc[i];
                         }
                     }
                 }
@@ -909,9 +895,6 @@ fft_status launch_psf_tc(fft_geom g, const int64_t* d_off, const uint32_t* d_ent
     P.nx = g->grid.nx;
     P.ny = g->grid.ny;
     P.nz = g->grid.nz;
-    P.z_lo = g->z_lo;
-    P.z_end = g->z_end;
-    P.mirror = g->mirror;
     P.d_off = d_off;
     P.d_ent = d_ent;
     P.ng = ng;

@@ -59,9 +59,7 @@ def test_mirrored_products(plane, nz, mirrors):
     subs = [np.arange(0, geo.M, 2, dtype=np.int32), np.arange(geo.M, dtype=np.int32)]
     for mode in (0, 1, 2):
         a, b = to_np(geo.psf_batch(spikes, subs, mode=mode)), to_np(gen.psf_batch(spikes, subs, mode=mode))
-        # mode 1 rounds J to BF16: entries of a layer and of its image agree to FP32 rounding (1e-6 of an
-        # entry), so that fewer than 1e-3 of them round to neighbouring BF16 values, 2^-8 apart
-        assert rel_l2(a, b) <= (1e-3 ** 0.5 * 2.0 ** -8 if mode == 1 else 2e-6)
+        assert rel_l2(a, b) <= 2e-6
     if (plane, nz) in ((8.5, 18), (4.0, 19)):
         og = oracle.Geometry(tx, rows, bor, [oracle.phi_table_gauss(f, s, 4096, t) for f, s, t in BANDS],
                              [b[2] for b in BANDS], grid, 1500.0)
