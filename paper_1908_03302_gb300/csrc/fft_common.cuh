@@ -115,7 +115,7 @@ struct fft_table_s {
 namespace fftgb {
 // Elevation stacks (fft_stack.cu): slices of equal rows whole numbers of layers apart.
 constexpr size_t STACK_MAX_SLICES = 64, STACK_MAX_CLASSES = 8;
-constexpr int64_t STACK_MIN_ENTRIES = 1 << 18;   // see build_stack
+constexpr int64_t STACK_MIN_ENTRIES = 1 << 20;   // see build_stack
 struct StackPlan {                               // host: a class as find_stack sees it
     double z;                                    // plane of its lowest slice
     std::vector<int32_t> shift;                  // each slice's layers above that

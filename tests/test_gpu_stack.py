@@ -1,6 +1,6 @@
 """Elevation stacks: slices a whole number of layers apart share one evaluation. Against the general
 path (the same rows plus one out-of-plane row far outside the grid, which is no stack) to 2e-6
-relative L2 (each is within 1e-6 of the exact product) and, for two of them, against the FP64 oracle
+relative L2 (each is within 1e-6 of the exact product) and, for one of them, against the FP64 oracle
 to 1e-5; 2 to 9 slices (every remainder of the four-column passes), one and several classes, planes on
 layers and between them, slices outside the grid, rows in slice, interleaved and descending order,
 tables and sine series, and slices that are not alike."""
@@ -19,7 +19,7 @@ BANDS = [(1.0e6, 0.3e6, 3e-6), (1.4e6, 0.2e6, 3 / 1.4e6)]   # the second is shar
 H = 1.5e-3
 
 
-def acquisition(layers, order, odd=None, n=128):
+def acquisition(layers, order, odd=None, n=256):
     """One ring per entry of `layers` (in voxel layers from the middle); rows of both bands."""
     ring = wl.ring(n, 36e-3)
     tx = np.concatenate([ring + [0.0, 0.0, z * H] for z in layers])
@@ -74,7 +74,7 @@ def test_stacked_products(layers, nz, order, odd, stack, series):
     geo = fg.Geometry(tx, rows, grid, 1500.0, tabs, band_of_row=bor)
     gen = fg.Geometry(np.concatenate([tx, far]), np.concatenate([rows, [[len(tx), len(tx) + 1]]]).astype(np.int32), grid,
                       1500.0, tabs, band_of_row=np.append(bor, 0).astype(np.int32))
-    assert geo.info().n_entries == gen.info().n_entries >= 1 << 18
+    assert geo.info().n_entries == gen.info().n_entries > 1 << 20
     rng = np.random.default_rng(5)
     m, d, w = (to_dev(rng.normal(size=n)) for n in (geo.V, geo.M, geo.M))
     more = lambda x: torch.cat([x, torch.zeros_like(x[..., :1])], dim=-1).contiguous()   # noqa: E731
@@ -109,7 +109,7 @@ def test_stacked_products(layers, nz, order, odd, stack, series):
         for mode in (0, 2):
             a, b = to_np(geo.psf_batch(spikes, subs, mode=mode)), to_np(gen.psf_batch(spikes, subs, mode=mode))
             assert rel_l2(a, b) <= 2e-6
-        if len(layers) in (2, 3):
+        if len(layers) == 2:
             og = oracle.Geometry(tx, rows, bor, [oracle.phi_table_gauss(f, s, 4096, t) for f, s, t in BANDS],
                                  [b[2] for b in BANDS], grid, 1500.0)
             assert rel_l2(J, og.J(to_np(m))) <= 1e-5
