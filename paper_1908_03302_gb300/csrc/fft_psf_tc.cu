@@ -310,6 +310,36 @@ __global__ void __launch_bounds__(MASK_THREADS) psf_mask_kernel(const PsfTcParam
     if (threadIdx.x == 0) c_or[T] = (uint16_t)s_or;
 }
 
+// Two rows (a, b) on the eight voxels of an x line between both pairs' transducer planes: detour_v's
+// inner form with two rows per packed instruction, by the same operations in the same order (the same
+// bits, so the same BF16 entries); a packed value is the K pair that the A tile stores. The generators are
+// bound by issue slots: about 31 instructions for the two entries against 46. TC_FIGURES
+template <bool PL>
+__device__ __forceinline__ void inner_line(f2 ps, f2 nr, f2 c1q, f2 c2, f2 c3, f2 hx, f2 hy, f2 hz, uint32_t tba,
+                                           uint32_t tbb, float nm1, unsigned char* aw) {
+    const f2 c12 = PL ? fma2(c2, c2, c1q) : c1q, nhx = neg2(hx), nhz = neg2(hz);
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const f2 ft = pk1((float)t);
+        const f2 c3t = fma2(ft, hy, c3);
+        f2 q2 = fma2(c3t, c3t, c12);
+        if (!PL) {
+            const f2 c2t = fma2(ft, nhz, c2);
+            q2 = fma2(c2t, c2t, q2);
+        }
+        const f2 pst = fma2(ft, hx, ps), nrt = fma2(ft, nhx, nr);   // p + L / 2 and L / 2 - p
+        const f2 ss = fma2(pst, pst, q2), rr = fma2(nrt, nrt, q2);
+        const f2 is = rsqrt2(ss), ir = rsqrt2(rr);
+        const f2 A = fma2(ss, is, pst), B = fma2(rr, ir, nrt);
+        const float2 N = up(mul2(q2, add2(A, B))), Q = up(rcp2(mul2(A, B)));
+        const float va = __saturatef(N.x * Q.x), vb = __saturatef(N.y * Q.y);
+        const float2 tt = up(fma2_rd(pk(va, vb), pk1(nm1), pk1(MAGIC)));
+        const float2 Ta = lds_f2(tba + (__float_as_uint(tt.x) << 3)), Tb = lds_f2(tbb + (__float_as_uint(tt.y) << 3));
+        const float2 y = up(mul2(pk(fmaf(va, Ta.y, Ta.x), fmaf(vb, Tb.y, Tb.x)), mul2(is, ir)));
+        *reinterpret_cast<uint32_t*>(aw + t * 16 * KC) = pack_bf16x2(y.x, y.y);
+    }
+}
+
 // GUARD: some voxel centre lies on a transducer (the geometry's flag): the guarded detour.
 template <bool GUARD>
 __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_constant__ PsfTcParams P) {
@@ -640,7 +670,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) psf_tc_kernel(const __grid_cons
         const float yb = phi_lookup(vib, tbbb, nm1) * (isb * irb);                                   \
         *reinterpret_cast<uint32_t*>(aw + t * 16 * KC) = pack_bf16x2(ya, yb);                        \
     }
-            if (wfl & 1u) {
+            if (!GUARD && (wfl & 1u)) {
+                const f2 ps = pk(psa, psb), nr = pk(-pra, -prb), c1q = pk(c1qa, c1qb), c2 = pk(c2a, c2b), c3 = pk(c3a, c3b);
+                const f2 hx = pk(Ba.x, Bb.x), hy = pk(Ba.y, Bb.y), hz = pk(Ba.z, Bb.z);
+                if (wfl & 2u)
+                    inner_line<true>(ps, nr, c1q, c2, c3, hx, hy, hz, tba, tbbb, nm1, aw);
+                else
+                    inner_line<false>(ps, nr, c1q, c2, c3, hx, hy, hz, tba, tbbb, nm1, aw);
+            } else if (wfl & 1u) {
                 if (wfl & 2u) {
                     FFT_TC_LINE(true, true)
                 } else {
