@@ -205,13 +205,14 @@ fft_status fft_JT_apply(fft_geom g, const float* d_dev, float* g_dev, void* stre
 /*
  * fft_J_apply_batch / fft_JT_apply_batch - J or J^T applied to n vectors at once (the
  * operator of Eq. forward_compact and its adjoint, for block methods such as the low-rank
- * eigensolver): every evaluated entry J[p, v] is used for four columns, so a group of four
- * costs little more than one application.
+ * eigensolver): every evaluated entry J[p, v] is used for up to eight columns, so a group of
+ * eight costs about one and a half applications, a group of four one and a quarter.
  *   m_dev  device float32, n columns of length V (column c at m_dev + c * V);
  *   d_dev  device float32, n columns of length M (column c at d_dev + c * M);
  *   g_dev  device float32, n columns of length V.
- * Columns are processed in groups of four; a remainder (and every column of geometries with
- * a non-stable detour mode) goes through the single-vector kernels. Each column matches the
+ * From four columns on they are processed in groups of up to eight (four where the scratch for
+ * eight is not there); fewer, and every column of geometries with a non-stable detour mode, go
+ * through the single-vector kernels. Each column matches the
  * single-vector call to rounding (same entries, same summation order). The first call
  * allocates the handle's batch scratch (E * 32 + slots * 4 * 2048 floats; twice that
  * from five columns on, where it takes at most half of the free memory).

@@ -313,7 +313,8 @@ __global__ void __launch_bounds__(MASK_THREADS) psf_mask_kernel(const PsfTcParam
 // Two rows (a, b) on the eight voxels of an x line between both pairs' transducer planes: detour_v's
 // inner form with two rows per packed instruction, by the same operations in the same order (the same
 // bits, so the same BF16 entries); a packed value is the K pair that the A tile stores. The generators are
-// bound by issue slots: about 31 instructions for the two entries against 46. TC_FIGURES
+// bound by issue slots: about 31 instructions for the two entries against 46 (384 PSFs of ring256 with
+// three bands 22.4 -> 21.4 ms).
 template <bool PL>
 __device__ __forceinline__ void inner_line(f2 ps, f2 nr, f2 c1q, f2 c2, f2 c3, f2 hx, f2 hy, f2 hz, uint32_t tba,
                                            uint32_t tbb, float nm1, unsigned char* aw) {
