@@ -297,9 +297,10 @@ fft_status fft_frob2(fft_geom g, double* out);
  *   m_dev     device float32[V]: in = starting model (zeros for m0 = 0), out = solution.
  *   hist_host nullable host double[n_iter + 1]: |J^T r - lambda m|^2 before each iteration
  *             and after the last.
- * Vectors are FP32; inner products, alpha, beta and gamma are FP64 on the device (no host
- * round trip). The iteration loop is captured once per handle into a CUDA graph and
- * replayed. A vanishing gradient (|J^T r - lambda m|^2 = 0) means m already minimises the
+ * Vectors are FP32, but up to 2^19 evaluated entries the products J p and J^T r come with
+ * compensated sums as two floats each (CGLS amplifies their rounding); inner products, alpha,
+ * beta and gamma are FP64 on the device (no host round trip). The iteration loop is captured
+ * once per handle into a CUDA graph and replayed. A vanishing gradient (|J^T r - lambda m|^2 = 0) means m already minimises the
  * misfit: the remaining iterations keep it, and that is not a breakdown.
  * Asynchronous on `stream` when hist_host is NULL: the call returns once the solve is
  * enqueued, and fft_cg_status gives its outcome. With hist_host the call synchronises and

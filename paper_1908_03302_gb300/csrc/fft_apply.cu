@@ -11,32 +11,41 @@
 namespace fftgb {
 
 // d_p = sum over the row's entries (ascending tile order) and the 4 regions of the partials.
+// LOW (the compensated form): the partials are FP64 and summed in it, and what d_p lacks after rounding goes to low.
+template <bool LOW>
 __global__ void __launch_bounds__(256) j_reduce_kernel(const int64_t* __restrict__ row_off,
                                                        const int64_t* __restrict__ row_ent,
-                                                       const float* __restrict__ jpart, int64_t M,
-                                                       float* __restrict__ d) {
+                                                       const void* __restrict__ jpart, int64_t M,
+                                                       float* __restrict__ d, float* __restrict__ low) {
     // one warp per row: lane l takes the row's entries l, l + 32, ... in order (the 4 region
     // partials of an entry pairwise in FP32, entries accumulated in FP64), then a fixed
     // butterfly over the lanes; the order never depends on scheduling
     const int lane = threadIdx.x & 31;
     const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (p >= M) return;
+    auto four = [&](int64_t j) {
+        if (LOW) {
+            const double2* a = reinterpret_cast<const double2*>(jpart) + row_ent[j] * 2;
+            const double2 a0 = __ldg(a), a1 = __ldg(a + 1);
+            return (a0.x + a0.y) + (a1.x + a1.y);
+        }
+        const float4 a = __ldg(reinterpret_cast<const float4*>(jpart) + row_ent[j]);
+        return (double)((a.x + a.y) + (a.z + a.w));
+    };
     double s = 0.0;
     const int64_t j1 = row_off[p + 1];
     int64_t j = row_off[p] + lane;
     for (; j + 32 < j1; j += 64) {   // two entries in flight, added in the same order
-        const float4 a0 = __ldg(reinterpret_cast<const float4*>(jpart + row_ent[j] * 4));
-        const float4 a1 = __ldg(reinterpret_cast<const float4*>(jpart + row_ent[j + 32] * 4));
-        s += (double)((a0.x + a0.y) + (a0.z + a0.w));
-        s += (double)((a1.x + a1.y) + (a1.z + a1.w));
+        const double a0 = four(j), a1 = four(j + 32);
+        s += a0;
+        s += a1;
     }
-    if (j < j1) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(jpart + row_ent[j] * 4));
-        s += (double)((a.x + a.y) + (a.z + a.w));
-    }
+    if (j < j1) s += four(j);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) d[p] = (float)s;
+    if (lane != 0) return;
+    d[p] = (float)s;
+    if (LOW) low[p] = (float)(s - (double)(float)s);
 }
 
 // The batch form of j_reduce_kernel: jpart[(entry * 8 + region) * NC + r]; the same lane order,
@@ -82,16 +91,19 @@ __global__ void __launch_bounds__(256) j_reduce_n_kernel(const int64_t* __restri
 // as many loads in flight as with one thread per run, which a tile cut into many small items
 // needs (32-element ring: about 45 slots per tile).
 // NCOL = 4, 8: the batch forms, slot q of column r at gpart[((s0 + q) * NCOL + r) * TILE_VOX],
-// g[r * V + v], columns r < ncol.
+// g[r * V + v], columns r < ncol. LOW (the compensated form, one column): the partials have low
+// parts (gpart_low), and what g lacks after rounding goes to g_low.
 constexpr int RED_WARPS = 8;
-template <int NCOL>
+template <int NCOL, bool LOW>
 __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t* __restrict__ slot0,
                                                                    const int32_t* __restrict__ nslot,
                                                                    const float* __restrict__ gpart, int nx, int ny,
                                                                    int nz, int z_lo, int z_end, int mirror,
                                                                    int tiles_x, int tiles_y, int ncol,
-                                                                   float* __restrict__ g) {
-    __shared__ float4 sh[RED_WARPS][32];
+                                                                   float* __restrict__ g,
+                                                                   const float* __restrict__ gpart_low,
+                                                                   float* __restrict__ g_low) {
+    __shared__ float4 sh[RED_WARPS][32], sh_low[LOW ? RED_WARPS : 1][32];
     constexpr int PER_TILE = TILE_VOX / (4 * 32);   // CTAs per tile
     const int T = blockIdx.x / PER_TILE, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int s0 = slot0[T];
@@ -128,15 +140,36 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
         }
         for (; q < ns; q += RED_WARPS)
             add(__ldcs(reinterpret_cast<const float4*>(base + (int64_t)q * NCOL * TILE_VOX)));
+        if (LOW && ns > 0) {   // low[k]: so far what acc lacks, with the opposite sign
+            const float* lbase = gpart_low + (int64_t)s0 * TILE_VOX + loc;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) low[k] = -low[k];
+            for (q = w; q < ns; q += RED_WARPS) {
+                const float4 x = __ldcs(reinterpret_cast<const float4*>(lbase + (int64_t)q * TILE_VOX));
+                low[0] += x.x;
+                low[1] += x.y;
+                low[2] += x.z;
+                low[3] += x.w;
+            }
+        }
         sh[w][lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        if (LOW) sh_low[w][lane] = make_float4(low[0], low[1], low[2], low[3]);
         __syncthreads();
         if (w < 4) {   // warp w: component w of the 32 runs
             double s = 0.0;
 #pragma unroll
-            for (int k = 0; k < RED_WARPS; ++k) s += (double)reinterpret_cast<const float*>(&sh[k][lane])[w];
+            for (int k = 0; k < RED_WARPS; ++k) {
+                s += (double)reinterpret_cast<const float*>(&sh[k][lane])[w];
+                if (LOW) s += (double)reinterpret_cast<const float*>(&sh_low[k][lane])[w];
+            }
             if (inside && ix + w < nx) {
                 g[(int64_t)r * V + v + w] = (float)s;
                 if (mo != 0) g[(int64_t)r * V + v + mo + w] = (float)s;
+                if (LOW) {
+                    const float l = (float)(s - (double)(float)s);
+                    g_low[v + w] = l;
+                    if (mo != 0) g_low[v + mo + w] = l;
+                }
             }
         }
         if (NCOL > 1) __syncthreads();
@@ -172,6 +205,8 @@ static ApplyParams make_params(fft_geom g) {
     P.vin = nullptr;
     P.vout = nullptr;
     P.gpart = g->gpart;
+    P.vlow = P.gpart_low = nullptr;
+    P.vpart = nullptr;
     P.dsum = nullptr;
     P.icount = nullptr;
     P.trig_nq = g->trig_nq;
@@ -218,6 +253,8 @@ fft_status set_apply_attributes(fft_geom g) {
     fft_status rc;
     if ((rc = set_attr_mode<MODE_JT>(smem)) != FFT_OK) return rc;
     if ((rc = set_attr_mode<MODE_J>(smem)) != FFT_OK) return rc;
+    if ((rc = set_attr_mode<MODE_JTC>(smem)) != FFT_OK) return rc;
+    if ((rc = set_attr_mode<MODE_JC>(smem)) != FFT_OK) return rc;
     if ((rc = set_attr_mode<MODE_COUNT>(smem)) != FFT_OK) return rc;
     if ((rc = set_attr_mode<MODE_COV>(smem)) != FFT_OK) return rc;
     // batch modes: stable detour only (other geometries apply the columns one by one)
@@ -360,12 +397,13 @@ static fft_status j_pass(fft_geom g, const float* m, int nc, float* d, cudaStrea
     return FFT_OK;
 }
 
-template <int NCOL>
-static fft_status launch_jt_reduce(fft_geom g, const float* gpart, int ncol, float* gout, cudaStream_t st) {
+template <int NCOL, bool LOW = false>
+static fft_status launch_jt_reduce(fft_geom g, const float* gpart, int ncol, float* gout, cudaStream_t st,
+                                   const float* gpart_low = nullptr, float* g_low = nullptr) {
     if (g->n_tiles == 0) return FFT_OK;
-    jt_reduce_kernel<NCOL><<<(unsigned)(g->n_tiles * (TILE_VOX / 128)), 32 * RED_WARPS, 0, st>>>(
+    jt_reduce_kernel<NCOL, LOW><<<(unsigned)(g->n_tiles * (TILE_VOX / 128)), 32 * RED_WARPS, 0, st>>>(
         g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->z_lo, g->z_end, g->mirror, g->tiles[0],
-        g->tiles[1], ncol, gout);
+        g->tiles[1], ncol, gout, gpart_low, g_low);
     FFT_CUDA(cudaGetLastError());
     return FFT_OK;
 }
@@ -422,7 +460,7 @@ fft_status launch_J(fft_geom g, const float* m, float* d, cudaStream_t st) {
     if (rc != FFT_OK) return rc;
     if (g->M > 0) {
         int64_t blocks = ceil_div(g->M, 8);   // 8 rows (warps) per block
-        j_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(g->row_off, g->row_ent, g->jpart, g->M, d);
+        j_reduce_kernel<false><<<(unsigned)blocks, 256, 0, st>>>(g->row_off, g->row_ent, g->jpart, g->M, d, nullptr);
         FFT_CUDA(cudaGetLastError());
     }
     return FFT_OK;
@@ -436,6 +474,35 @@ fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st)
     fft_status rc = launch_mode<MODE_JT>(g, P, st);
     if (rc != FFT_OK) return rc;
     return launch_jt_reduce<1>(g, g->gpart, 1, gout, st);
+}
+
+// J and J^T with compensated sums (MODE_JC, MODE_JTC), the result as the sum of two floats: d + d_low, g + g_low.
+// The caller's scratch: jpart64 [E * 4], gpart_low [n_slots * TILE_VOX].
+bool has_compensated(fft_geom g) {
+    return g->dt_mode == FFT_DT_STABLE && g->stk.empty() && g->E_used <= COMP_MAX_ENTRIES;
+}
+
+fft_status launch_J_comp(fft_geom g, const float* m, float* d, float* d_low, double* jpart64, cudaStream_t st) {
+    ApplyParams P = make_params(g);
+    P.vin = m;
+    P.vpart = jpart64;
+    const fft_status rc = launch_mode<MODE_JC>(g, P, st);
+    if (rc != FFT_OK || g->M == 0) return rc;
+    j_reduce_kernel<true><<<(unsigned)ceil_div(g->M, 8), 256, 0, st>>>(g->row_off, g->row_ent, jpart64, g->M, d, d_low);
+    FFT_CUDA(cudaGetLastError());
+    return FFT_OK;
+}
+
+fft_status launch_JT_comp(fft_geom g, const float* din, float* gout, float* g_low, float* gpart_low,
+                          cudaStream_t st) {
+    ApplyParams P = make_params(g);
+    P.vin = din;
+    P.vout = gout;
+    P.vlow = g_low;
+    P.gpart_low = gpart_low;
+    const fft_status rc = launch_mode<MODE_JTC>(g, P, st);
+    if (rc != FFT_OK) return rc;
+    return launch_jt_reduce<1, true>(g, g->gpart, 1, gout, st, gpart_low, g_low);
 }
 
 // cov_v = sum_p |J[p, v] w_p| (w null: all ones), gathered like J^T.

@@ -41,8 +41,11 @@ namespace fftgb {
 // MODE_COV: sensitivity coverage sum_p |J[p, v] w_p| (J^T of |J|, same gather as MODE_JT).
 // MODE_JT4 / MODE_J4, MODE_JT8 / MODE_J8: J^T and J for up to four or eight right-hand sides at once
 // (every evaluated entry is applied to all; blocks are column-major: column r at r * V or r * M).
+// MODE_JTC / MODE_JC: J^T and J with compensated FP32 sums, for the solver (fft_cg.cu says why): an
+// entry's product goes into a pair of floats (fma2_comp), rows' weights are pairs as well, J folds the
+// pairs, and the partials are stored as pairs (J^T) or in FP64 (J).
 enum { MODE_JT = 0, MODE_J = 1, MODE_COUNT = 2, MODE_FROB = 3, MODE_COV = 4, MODE_JT4 = 5, MODE_J4 = 6, MODE_JT8 = 7,
-       MODE_J8 = 8 };
+       MODE_J8 = 8, MODE_JTC = 9, MODE_JC = 10 };
 constexpr int STG_PER_WARP = 128;    // staged float4 per warp: 32 rows x (3 or 4)
 constexpr int STG_PER_WARP8 = 160;   // the eight-column J^T: 32 rows x 5
 // CTA of the eight-column kernels: one per SM, of 16 warps at 128 registers (64 of them hold a lane's
@@ -86,6 +89,9 @@ struct ApplyParams {
     const float* vin;        // J: m [V]; J^T: d [M]
     float* vout;             // J: jpart [E * 4]; J^T: g [V]
     float* gpart;            // J^T partials of multi-item tiles
+    float* vlow;             // JTC: what a voxel's value lacks after rounding (written beside vout)
+    float* gpart_low;        // JTC: the same of the J^T partials
+    double* vpart;           // JC: jpart in FP64 [E * 4]
     double* dsum;            // FROB: one per unit [n_items * 4]
     unsigned long long* icount;   // COUNT
     int trig_nq;             // PHI_TRIG: coefficient groups of 4 per band
@@ -442,6 +448,11 @@ constexpr bool apply_sharp_wide() {
     return SHARP && DT == FFT_DT_STABLE && PHI != PHI_TRIG && apply_ncol<MODE>() == 1;
 }
 constexpr int SHARP_MAX_WARPS = 20;
+// (the compensated J^T, 16 more registers a lane, for 16 warps at 128: it would spill 336 bytes at 96)
+template <int MODE>
+constexpr int sharp_bound_warps() {
+    return MODE == MODE_JTC ? 16 : SHARP_MAX_WARPS;
+}
 
 // The plain stable-detour table variants (single column) are built for blocks of up to 24
 // warps at one per SM, i.e. 80 registers: their 16 per-lane voxels (8 x 8 x 8 units) want more
@@ -456,7 +467,7 @@ constexpr int PLAIN_MAX_WARPS = 24;
 template <int MODE, int DT, bool SHARP, int PHI>
 constexpr int apply_block_bound() {
     return apply_ncol<MODE>() == 8                    ? 32 * col8_warps<SHARP>()
-           : apply_sharp_wide<MODE, DT, SHARP, PHI>() ? 32 * SHARP_MAX_WARPS
+           : apply_sharp_wide<MODE, DT, SHARP, PHI>() ? 32 * sharp_bound_warps<MODE>()
            : apply_plain_wide<MODE, DT, SHARP, PHI>() ? 32 * PLAIN_MAX_WARPS
                                                       : APPLY_THREADS;
 }
@@ -486,7 +497,8 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
     constexpr int NC = apply_ncol<MODE>();
     constexpr bool JTN = (MODE == MODE_JT4 || MODE == MODE_JT8), JN = (MODE == MODE_J4 || MODE == MODE_J8);
     constexpr bool BATCH = NC > 1;
-    constexpr int SR = JTN ? 3 + NC / 4 : 3;   // staged float4 per row
+    constexpr bool JT1 = (MODE == MODE_JT || MODE == MODE_JTC), J1 = (MODE == MODE_J || MODE == MODE_JC);
+    constexpr int SR = JTN ? 3 + NC / 4 : (MODE == MODE_JTC ? 4 : 3);   // staged float4 per row
     constexpr int NSUB = apply_nsub<MODE>();
     constexpr int NREG = apply_regions<MODE>();
     float4* stg = s_stage + warp * apply_stage<MODE>();
@@ -532,7 +544,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 TZ + 4 * wz + sub_dz<NSUB>(s) + 3 >= P.z_lo)
                 sub_ok |= 1u << s;
         // the gather modes need the mask only for their stores: recomputed there
-        constexpr bool VM_LIVE = !(MODE == MODE_JT || MODE == MODE_COV || JTN);
+        constexpr bool VM_LIVE = !(JT1 || MODE == MODE_COV || JTN);
         const uint32_t vmask = VM_LIVE ? lane_vmask() : 0u;
         const int64_t vbase = ((int64_t)(TZ + ozi) * P.ny + TY + oyi) * P.nx + TX + oxi;
         // voxels from this lane's run in sub-brick s to its mirror image (0: none)
@@ -556,7 +568,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
 
         // accumulators (J^T) or model values (J) of the lane's voxels, as pairs (0, 1), (2, 3) of
         // each run
-        f2 acc[NSUB][2], mv[NSUB][2];
+        f2 acc[NSUB][2], accl[NSUB][2], mv[NSUB][2];   // (accl: low parts, JTC only)
         f2 accn[2][2][NC], mvn[2][2][NC];   // batch modes only (NSUB = 2)
         double dacc = 0.0;
         unsigned long long cnt = 0, cnt_eval = 0;
@@ -566,8 +578,8 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
             for (int j = 0; j < 2; ++j) {
                 const int64_t vo = vbase + ((int64_t)sub_dz<NSUB>(s) * P.ny + sub_dy<NSUB>(s)) * P.nx + 2 * j;
                 const bool ok0 = (vmask >> (4 * s + 2 * j)) & 1u, ok1 = (vmask >> (4 * s + 2 * j + 1)) & 1u;
-                acc[s][j] = mv[s][j] = 0ull;
-                if (MODE == MODE_J) {
+                acc[s][j] = accl[s][j] = mv[s][j] = 0ull;
+                if (J1) {
                     mv[s][j] = pk(ok0 ? __ldg(P.vin + vo) : 0.0f, ok1 ? __ldg(P.vin + vo + 1) : 0.0f);
                     if (const int64_t mo = mirror_off(s))
                         mv[s][j] = add2(mv[s][j], pk(ok0 ? __ldg(P.vin + vo + mo) : 0.0f,
@@ -602,7 +614,12 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const BandConst bc = P.bc[b];
                 const float hb = bc.h;
                 float W = r.b.w;
-                if (MODE == MODE_JT) W *= __ldg(P.vin + p);
+                float Wlow = 0.0f;   // what W lacks after rounding
+                if (JT1) {
+                    const float x = __ldg(P.vin + p), C = W;
+                    W *= x;
+                    if (MODE == MODE_JTC) Wlow = fmaf(C, x, -W);
+                }
                 if (MODE == MODE_COV) W = fabsf(W) * (P.vin ? fabsf(__ldg(P.vin + p)) : 1.0f);
                 float Wn[NC];
                 bool any_w = false;
@@ -621,7 +638,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 const float cx = fmaf(8.0f * wx + 3.5f, hb, dx);
                 const float hxx = 3.5f * hb, hyy = 1.5f * hb;
                 // rows with zero weight add exactly nothing to J^T: skip them
-                const bool live = JTN ? any_w : ((MODE != MODE_JT && MODE != MODE_COV) || (W != 0.0f));
+                const bool live = JTN ? any_w : ((!JT1 && MODE != MODE_COV) || (W != 0.0f));
                 const float pext = hxx * fabsf(ex) + hyy * (fabsf(ey) + fabsf(ez)) + 1e-3f;
                 // deep sub-bricks: their voxel centres (half diagonal sqrt(3.5^2 + 2 1.5^2) = 4.1 steps)
                 // keep DEEP_MARGIN steps off the pair's sphere
@@ -657,6 +674,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 stg[lane * SR + 2] = make_float4(W, row_m, DT == FFT_DT_FP64 ? __int_as_float(p) : lam,
                                                  __int_as_float(b | (bc.sharp << 8) | (planar << 9) |
                                                                 (int)((okb << 12) | (inb << 16) | (dpb << 20) | (both << 24) | (full << 28))));
+                if (MODE == MODE_JTC) stg[lane * SR + 3].x = Wlow;
                 if (JTN) {
 #pragma unroll
                     for (int k = 0; k < NC / 4; ++k)
@@ -666,6 +684,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
             uint32_t mm = __ballot_sync(0xffffffffu, okb != 0u);
             __syncwarp();
             float mypart = 0.0f;
+            double mypart64 = 0.0;   // JC
             while (mm) {
                 const int bit = __ffs(mm) - 1;
                 mm &= mm - 1;
@@ -684,13 +703,14 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     }
                 }
                 const float hx = B.x, hy = B.y, hz = B.z, W = C.x, row_m = C.y;
+                const float Wlow = MODE == MODE_JTC ? stg[bit * SR + 3].x : 0.0f;
                 const float hl = 0.5f * (A.x - A.y);   // used by the textbook (NAIVE) detour only
                 const uint32_t cw = (uint32_t)__float_as_int(C.w);
                 const bool planar = (DT != FFT_DT_FP64) && ((cw >> 9) & 1u);
                 DeepRow dr;
                 deep_init(dr, C.z);
                 float near = 2.0f;   // smallest |v - 1| of this lane's voxels (sharp bands)
-                f2 part = 0ull;
+                f2 part = 0ull, partl = 0ull;   // (partl: low part, JC only)
                 f2 partn[NC];
 #pragma unroll
                 for (int r = 0; r < NC; ++r) partn[r] = 0ull;
@@ -729,11 +749,16 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     for (int j = 0; j < 2; ++j) {
                         const f2 val = mul2(pk(ph[2 * j], ph[2 * j + 1]), w[j]);
                         if (MODE == MODE_JT) acc[s][j] = fma2(val, pk1(W), acc[s][j]);
+                        if (MODE == MODE_JTC) {
+                            fma2_comp(val, pk1(W), acc[s][j], accl[s][j]);
+                            accl[s][j] = fma2(val, pk1(Wlow), accl[s][j]);
+                        }
                         if (MODE == MODE_COV) {
                             const float2 x = up(val);
                             acc[s][j] = fma2(pk(fabsf(x.x), fabsf(x.y)), pk1(W), acc[s][j]);
                         }
                         if (MODE == MODE_J) part = fma2(val, mv[s][j], part);
+                        if (MODE == MODE_JC) fma2_comp(val, mv[s][j], part, partl);
                         if (JTN) {
 #pragma unroll
                             for (int r = 0; r < NC; ++r) accn[s & 1][j][r] = fma2(val, pk1(Wr[r]), accn[s & 1][j][r]);
@@ -855,8 +880,8 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                             const bool ok0 = (vmask >> (4 * s + 2 * j)) & 1u, ok1 = (vmask >> (4 * s + 2 * j + 1)) & 1u;
                             const int f = (int)((mult >> (8 * s)) & 255u);   // count, Frobenius
                             if (MODE == MODE_COUNT) n_in += f * ((ok0 ? (int)d0 : 0) + (ok1 ? (int)d1 : 0));
-                            if (MODE == MODE_JT || MODE == MODE_COV) acc[s][j] = fma2(dk, pk1(W), acc[s][j]);
-                            if (MODE == MODE_J) part = fma2(dk, mv[s][j], part);
+                            if (JT1 || MODE == MODE_COV) acc[s][j] = fma2(dk, pk1(W), acc[s][j]);
+                            if (J1) part = fma2(dk, mv[s][j], part);
                             if (JTN) {
 #pragma unroll
                                 for (int r = 0; r < NC; ++r) accn[s & 1][j][r] = fma2(dk, pk1(Wr[r]), accn[s & 1][j][r]);
@@ -884,6 +909,19 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     __syncwarp();
                     if (lane < 8) reinterpret_cast<float*>(stg + bit * SR)[lane] = ps;
                 }
+                if (MODE == MODE_JC) {
+                    // the same with (sum, low part) pairs, to 4 lanes; the row's lane adds those in FP64
+                    const float2 p2 = up(part), l2 = up(partl);
+                    float ps, pl = two_sum(p2.x, p2.y, ps) + (l2.x + l2.y);
+#pragma unroll
+                    for (int o = 16; o >= 4; o >>= 1) {
+                        const float qs = __shfl_xor_sync(0xffffffffu, ps, o), ql = __shfl_xor_sync(0xffffffffu, pl, o);
+                        const float low = two_sum(ps, qs, ps);
+                        pl = low + (pl + ql);
+                    }
+                    __syncwarp();
+                    if (lane < 4) reinterpret_cast<float2*>(stg + bit * SR)[lane] = make_float2(ps, pl);
+                }
                 if (JN) {
                     // Transposing fold: each exchange halves the columns a lane carries (NC / 2 + .. + 1
                     // shuffles), the others add the lanes that hold one column; the first of them
@@ -910,16 +948,23 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                 }
                 if (MODE == MODE_FROB) dacc += (double)fsum * (double)W * (double)W;
             }
-            if (MODE == MODE_J) {
+            if (J1) {
                 __syncwarp();
                 if (have) {
                     if (okb) {
                         const float4 r0 = stg[lane * SR + 0];
                         const float4 r1 = stg[lane * SR + 1];
                         const float Wl = stg[lane * SR + 2].x;
-                        mypart = (r0.x + r0.y + r0.z + r0.w + r1.x + r1.y + r1.z + r1.w) * Wl;
+                        if (MODE == MODE_JC)
+                            mypart64 = (((double)r0.x + (double)r0.z) + ((double)r1.x + (double)r1.z) +
+                                        (double)((r0.y + r0.w) + (r1.y + r1.w))) * (double)Wl;
+                        else
+                            mypart = (r0.x + r0.y + r0.z + r0.w + r1.x + r1.y + r1.z + r1.w) * Wl;
                     }
-                    P.vout[e * NREG + region] = mypart;
+                    if (MODE == MODE_JC)
+                        P.vpart[e * NREG + region] = mypart64;
+                    else
+                        P.vout[e * NREG + region] = mypart;
                 }
             }
             if (JN) {
@@ -940,27 +985,40 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
             __syncwarp();
         }
 
-        if (MODE == MODE_JT || MODE == MODE_COV) {
+        if (JT1 || MODE == MODE_COV) {
             const uint32_t vm = lane_vmask();
 #pragma unroll
             for (int s = 0; s < NSUB; ++s) {
                 const int dy = sub_dy<NSUB>(s), dz = sub_dz<NSUB>(s);
                 const float2 a0 = up(acc[s][0]), a1 = up(acc[s][1]);
-                const float av[NX_LANE] = {a0.x, a0.y, a1.x, a1.y};
+                float av[NX_LANE] = {a0.x, a0.y, a1.x, a1.y}, lv[NX_LANE];
+                if (MODE == MODE_JTC) {
+                    const float2 l0 = up(accl[s][0]), l1 = up(accl[s][1]);
+                    const float low[NX_LANE] = {l0.x, l0.y, l1.x, l1.y};
+#pragma unroll
+                    for (int t = 0; t < NX_LANE; ++t) lv[t] = two_sum(av[t], low[t], av[t]);
+                }
                 if (item.slot < 0) {
                     const int64_t mo = mirror_off(s);
 #pragma unroll
                     for (int t = 0; t < NX_LANE; ++t)
                         if ((vm >> (4 * s + t)) & 1u) {
-                            float* o = P.vout + vbase + ((int64_t)dz * P.ny + dy) * P.nx + t;
-                            o[0] = av[t];
-                            if (mo != 0) o[mo] = av[t];
+                            const int64_t at_v = vbase + ((int64_t)dz * P.ny + dy) * P.nx + t;
+                            P.vout[at_v] = av[t];
+                            if (mo != 0) P.vout[at_v + mo] = av[t];
+                            if (MODE == MODE_JTC) {
+                                P.vlow[at_v] = lv[t];
+                                if (mo != 0) P.vlow[at_v + mo] = lv[t];
+                            }
                         }
                 } else {
                     // local index inside the tile: (z * 16 + y) * 16 + x
                     const int loc = (((ozi + dz) * TILE_Y) + oyi + dy) * TILE_X + oxi;
                     *reinterpret_cast<float4*>(P.gpart + (int64_t)item.slot * TILE_VOX + loc) =
                         make_float4(av[0], av[1], av[2], av[3]);
+                    if (MODE == MODE_JTC)
+                        *reinterpret_cast<float4*>(P.gpart_low + (int64_t)item.slot * TILE_VOX + loc) =
+                            make_float4(lv[0], lv[1], lv[2], lv[3]);
                 }
             }
         }
@@ -1048,7 +1106,8 @@ inline void launch_apply(fft_geom g, const ApplyParams& P, cudaStream_t st) {
     if (apply_ncol<MODE>() == 8) {
         apply_kernel<MODE, DT, G, S, PHI><<<g->sms, 32 * col8_warps<S>(), apply_smem8(g, col8_warps<S>()), st>>>(P);
     } else if (apply_sharp_wide<MODE, DT, S, PHI>()) {
-        apply_kernel<MODE, DT, G, S, PHI><<<g->sharp_ctas, 32 * g->sharp_warps, apply_smem(g, g->sharp_warps), st>>>(P);
+        const int w = std::min(g->sharp_warps, sharp_bound_warps<MODE>());
+        apply_kernel<MODE, DT, G, S, PHI><<<g->sharp_ctas, 32 * w, apply_smem(g, w), st>>>(P);
     } else if (apply_plain_wide<MODE, DT, S, PHI>() && g->plain_warps > APPLY_WARPS) {
         apply_kernel<MODE, DT, G, S, PHI><<<g->plain_ctas, 32 * g->plain_warps, apply_smem(g, g->plain_warps), st>>>(P);
     } else {
@@ -1108,7 +1167,7 @@ inline fft_status launch_mode_impl(fft_geom g, const ApplyParams& P, cudaStream_
     return FFT_OK;
 }
 
-// The batch modes (stable detour only).
+// The modes that exist for the stable detour only: batches, compensated sums.
 template <int MODE>
 inline fft_status launch_batch_impl(fft_geom g, const ApplyParams& P, cudaStream_t st) {
     FFT_CUDA(cudaMemsetAsync(g->counter, 0, 2 * sizeof(int32_t), st));
@@ -1139,6 +1198,8 @@ template <int MODE>
 fft_status set_attr_mode(size_t smem);
 template <> fft_status launch_mode<MODE_JT>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status launch_mode<MODE_J>(fft_geom g, const ApplyParams& P, cudaStream_t st);
+template <> fft_status launch_mode<MODE_JTC>(fft_geom g, const ApplyParams& P, cudaStream_t st);
+template <> fft_status launch_mode<MODE_JC>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status launch_mode<MODE_COUNT>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status launch_mode<MODE_FROB>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status launch_mode<MODE_COV>(fft_geom g, const ApplyParams& P, cudaStream_t st);
@@ -1148,6 +1209,8 @@ template <> fft_status launch_batch<MODE_J4>(fft_geom g, const ApplyParams& P, c
 template <> fft_status launch_batch<MODE_J8>(fft_geom g, const ApplyParams& P, cudaStream_t st);
 template <> fft_status set_attr_mode<MODE_JT>(size_t smem);
 template <> fft_status set_attr_mode<MODE_J>(size_t smem);
+template <> fft_status set_attr_mode<MODE_JTC>(size_t smem);
+template <> fft_status set_attr_mode<MODE_JC>(size_t smem);
 template <> fft_status set_attr_mode<MODE_COUNT>(size_t smem);
 template <> fft_status set_attr_mode<MODE_FROB>(size_t smem);
 template <> fft_status set_attr_mode<MODE_COV>(size_t smem);

@@ -2,8 +2,8 @@
 // Gamma_pr = I, alpha J(dc) = 1/2 lambda |dc|^2): the normal equations
 // (J^T J + lambda I) m = J^T d are solved iteratively with J and J^T applied on the fly.
 //
-// Vectors are FP32; every inner product is accumulated in FP64 by a fixed grid of blocks
-// followed by a fixed-order final sum, and alpha, beta, gamma live in FP64 device memory,
+// Vectors are FP32 (the products of small operators two floats each, see solver_J); every
+// inner product is accumulated in FP64 by a fixed grid of blocks followed by a fixed-order final sum, and alpha, beta, gamma live in FP64 device memory,
 // so the loop needs no host round trip and is bit-reproducible. The loop is captured once
 // into a CUDA graph (per iteration count) on a private stream and replayed on the caller's
 // stream; it touches only the handle's own buffers, so the graph is independent of the
@@ -40,14 +40,20 @@ __device__ double block_reduce(double v, double* sh) {
     return s;
 }
 
+// A vector's element, with its low part where it has one.
+__device__ __forceinline__ double with_low(const float* v, const float* low, int64_t i) {
+    return low ? (double)v[i] + (double)low[i] : (double)v[i];
+}
+
 // part[blk] = sum_i a_i^2 over the block's grid-stride share of a; part[DOT_BLOCKS + blk] for b.
-__global__ void dot2_partial_kernel(const float* __restrict__ a, int64_t na, const float* __restrict__ b,
-                                    int64_t nb, double* __restrict__ part) {
+// (a_low, nullable: a's low parts)
+__global__ void dot2_partial_kernel(const float* __restrict__ a, const float* __restrict__ a_low, int64_t na,
+                                    const float* __restrict__ b, int64_t nb, double* __restrict__ part) {
     __shared__ double sh[DOT_THREADS / 32];
     const int64_t stride = (int64_t)DOT_BLOCKS * DOT_THREADS;
     double sa = 0.0, sb = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * DOT_THREADS + threadIdx.x; i < na; i += stride) {
-        double x = a[i];
+        const double x = with_low(a, a_low, i);
         sa += x * x;
     }
     for (int64_t i = (int64_t)blockIdx.x * DOT_THREADS + threadIdx.x; i < nb; i += stride) {
@@ -117,23 +123,28 @@ __global__ void set_lambda_kernel(double* scal, double lam) { scal[S_LAMBDA] = l
 __global__ void cg_hist0_kernel(const double* __restrict__ scal, double* __restrict__ hist) { hist[0] = scal[S_GAMMA]; }
 
 // r = d - q
-__global__ void residual_kernel(const float* __restrict__ d, const float* __restrict__ q, int64_t M,
-                                float* __restrict__ r) {
+__global__ void residual_kernel(const float* __restrict__ d, const float* __restrict__ q,
+                                const float* __restrict__ q_low, int64_t M, float* __restrict__ r) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < M) r[i] = d[i] - q[i];
+    if (i < M) r[i] = q_low ? (float)((double)d[i] - with_low(q, q_low, i)) : d[i] - q[i];
 }
 
 // s -= lambda m, partial sums of s^2.
-__global__ void cg_s_kernel(float* __restrict__ s, const float* __restrict__ m, int64_t V,
+__global__ void cg_s_kernel(float* __restrict__ s, float* __restrict__ s_low, const float* __restrict__ m, int64_t V,
                             const double* __restrict__ scal, double* __restrict__ part) {
     __shared__ double sh[DOT_THREADS / 32];
     const double lam = scal[S_LAMBDA];
     const int64_t stride = (int64_t)DOT_BLOCKS * DOT_THREADS;
     double acc = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * DOT_THREADS + threadIdx.x; i < V; i += stride) {
-        float v = (float)((double)s[i] - lam * (double)m[i]);
+        double x = with_low(s, s_low, i) - lam * (double)m[i];
+        const float v = (float)x;
         s[i] = v;
-        acc += (double)v * (double)v;
+        if (s_low)
+            s_low[i] = (float)(x - (double)v);
+        else
+            x = (double)v;
+        acc += x * x;
     }
     acc = block_reduce(acc, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = acc;
@@ -141,23 +152,23 @@ __global__ void cg_s_kernel(float* __restrict__ s, const float* __restrict__ m, 
 
 // m += alpha p; r -= alpha q.
 __global__ void cg_update_mr_kernel(float* __restrict__ m, const float* __restrict__ p, int64_t V,
-                                    float* __restrict__ r, const float* __restrict__ q, int64_t M,
-                                    const double* __restrict__ scal) {
+                                    float* __restrict__ r, const float* __restrict__ q,
+                                    const float* __restrict__ q_low, int64_t M, const double* __restrict__ scal) {
     const double al = scal[S_ALPHA];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V; i += stride)
         m[i] = (float)((double)m[i] + al * (double)p[i]);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < M; i += stride)
-        r[i] = (float)((double)r[i] - al * (double)q[i]);
+        r[i] = (float)((double)r[i] - al * with_low(q, q_low, i));
 }
 
 // p = s + beta p.
-__global__ void cg_update_p_kernel(float* __restrict__ p, const float* __restrict__ s, int64_t V,
-                                   const double* __restrict__ scal) {
+__global__ void cg_update_p_kernel(float* __restrict__ p, const float* __restrict__ s, const float* __restrict__ s_low,
+                                   int64_t V, const double* __restrict__ scal) {
     const double be = scal[S_BETA];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V; i += stride)
-        p[i] = (float)((double)s[i] + be * (double)p[i]);
+        p[i] = (float)(with_low(s, s_low, i) + be * (double)p[i]);
 }
 
 template <typename T>
@@ -180,6 +191,12 @@ fft_status ensure_workspace(fft_geom g, int32_t n_iter) {
     if ((rc = cg_alloc(&g->cg_s, g->V)) != FFT_OK) return rc;
     if ((rc = cg_alloc(&g->cg_p, g->V)) != FFT_OK) return rc;
     if ((rc = cg_alloc(&g->cg_m, g->V)) != FFT_OK) return rc;
+    if (has_compensated(g)) {
+        if ((rc = cg_alloc(&g->cg_ql, g->M)) != FFT_OK) return rc;
+        if ((rc = cg_alloc(&g->cg_sl, g->V)) != FFT_OK) return rc;
+        if ((rc = cg_alloc(&g->cg_jpart, 4 * (size_t)g->E)) != FFT_OK) return rc;
+        if ((rc = cg_alloc(&g->cg_gpart, (size_t)g->n_slots * TILE_VOX)) != FFT_OK) return rc;
+    }
     if ((rc = cg_alloc(&g->cg_scal, 8)) != FFT_OK) return rc;
     if ((rc = cg_alloc(&g->cg_dots, 2 * DOT_BLOCKS)) != FFT_OK) return rc;
     if ((rc = cg_alloc(&g->cg_status, 1)) != FFT_OK) return rc;
@@ -208,6 +225,24 @@ fft_status ensure_workspace(fft_geom g, int32_t n_iter) {
     return FFT_OK;
 }
 
+// q = J x and s = J^T r, each as two floats where the sums are compensated (has_compensated). CGLS amplifies
+// the rounding of its products and vectors 20 to 30 times in 20 iterations, by a factor that depends on the
+// data: with FP32 sums single solves of four 32-element slices came out up to 12e-6 from the 64-bit solve where
+// the operator's own entries account for 1.2e-6. With compensated sums, and q and s kept to 48 bits, only the
+// rounding of the state (m, p, r: FP32, as a saved state holds them) is left. Over 24 data sets, geometric
+// mean and worst: 2.4e-6 and 6.8e-6 without, 1.6e-6 and 3.3e-6 with them (entries alone: 1.2e-6 and 1.4e-6).
+// It costs 6 to 24 % of a solve (20 iterations: 32-element ring 1.74 -> 1.88 ms, four slices of 32
+// elements with three bands 5.32 -> 6.10 ms, of 56 elements 16.2 -> 19.5 ms). The line at 2^19 evaluated entries is
+// the largest size at which the distance was measured against a 64-bit solve; beyond it the products are
+// bound by evaluations and would pay the whole price (ring256: J 1.93 -> 2.34 ms).
+fft_status solver_J(fft_geom g, const float* x, cudaStream_t st) {
+    return g->cg_ql ? launch_J_comp(g, x, g->cg_q, g->cg_ql, g->cg_jpart, st) : launch_J(g, x, g->cg_q, st);
+}
+fft_status solver_JT(fft_geom g, cudaStream_t st) {
+    return g->cg_sl ? launch_JT_comp(g, g->cg_r, g->cg_s, g->cg_sl, g->cg_gpart, st)
+                    : launch_JT(g, g->cg_r, g->cg_s, st);
+}
+
 // The iteration loop from the handle's state (m, p, r, gamma, lambda); hist[it + 1] receives
 // |s|^2 after iteration it.
 fft_status enqueue_iterations(fft_geom g, int32_t n_iter, cudaStream_t st) {
@@ -215,17 +250,17 @@ fft_status enqueue_iterations(fft_geom g, int32_t n_iter, cudaStream_t st) {
     fft_status rc;
     for (int32_t it = 0; it < n_iter; ++it) {
         // q = J p; delta = |q|^2 + lambda |p|^2; alpha = gamma / delta
-        if ((rc = launch_J(g, g->cg_p, g->cg_q, st)) != FFT_OK) return rc;
-        dot2_partial_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_q, M, g->cg_p, V, g->cg_dots);
+        if ((rc = solver_J(g, g->cg_p, st)) != FFT_OK) return rc;
+        dot2_partial_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_q, g->cg_ql, M, g->cg_p, V, g->cg_dots);
         cg_alpha_kernel<<<1, DOT_THREADS, 0, st>>>(g->cg_scal, g->cg_dots, g->cg_status);
         // m += alpha p; r -= alpha q
-        cg_update_mr_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_m, g->cg_p, V, g->cg_r, g->cg_q, M,
-                                                                g->cg_scal);
+        cg_update_mr_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_m, g->cg_p, V, g->cg_r, g->cg_q, g->cg_ql,
+                                                                M, g->cg_scal);
         // s = J^T r - lambda m; beta = |s|^2 / gamma; p = s + beta p
-        if ((rc = launch_JT(g, g->cg_r, g->cg_s, st)) != FFT_OK) return rc;
-        cg_s_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_s, g->cg_m, V, g->cg_scal, g->cg_dots);
+        if ((rc = solver_JT(g, st)) != FFT_OK) return rc;
+        cg_s_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_s, g->cg_sl, g->cg_m, V, g->cg_scal, g->cg_dots);
         cg_beta_kernel<<<1, DOT_THREADS, 0, st>>>(g->cg_scal, g->cg_dots, g->cg_hist, it + 1, g->cg_status, 0);
-        cg_update_p_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_p, g->cg_s, V, g->cg_scal);
+        cg_update_p_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_p, g->cg_s, g->cg_sl, V, g->cg_scal);
     }
     FFT_CUDA(cudaGetLastError());
     return FFT_OK;
@@ -238,11 +273,11 @@ fft_status enqueue_solve(fft_geom g, int32_t n_iter, cudaStream_t st) {
     fft_status rc;
     FFT_CUDA(cudaMemsetAsync(g->cg_status, 0, sizeof(int32_t), st));
     // r = d - J m
-    if ((rc = launch_J(g, g->cg_m, g->cg_q, st)) != FFT_OK) return rc;
-    residual_kernel<<<rb, 256, 0, st>>>(g->cg_d, g->cg_q, M, g->cg_r);
+    if ((rc = solver_J(g, g->cg_m, st)) != FFT_OK) return rc;
+    residual_kernel<<<rb, 256, 0, st>>>(g->cg_d, g->cg_q, g->cg_ql, M, g->cg_r);
     // s = J^T r - lambda m; gamma = |s|^2; p = s
-    if ((rc = launch_JT(g, g->cg_r, g->cg_s, st)) != FFT_OK) return rc;
-    cg_s_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_s, g->cg_m, V, g->cg_scal, g->cg_dots);
+    if ((rc = solver_JT(g, st)) != FFT_OK) return rc;
+    cg_s_kernel<<<DOT_BLOCKS, DOT_THREADS, 0, st>>>(g->cg_s, g->cg_sl, g->cg_m, V, g->cg_scal, g->cg_dots);
     cg_beta_kernel<<<1, DOT_THREADS, 0, st>>>(g->cg_scal, g->cg_dots, g->cg_hist, 0, g->cg_status, 1);
     FFT_CUDA(cudaMemcpyAsync(g->cg_p, g->cg_s, sizeof(float) * V, cudaMemcpyDeviceToDevice, st));
     return enqueue_iterations(g, n_iter, st);

@@ -55,6 +55,7 @@ constexpr int NX_LANE = 4;             // voxels per lane per sub-brick (along x
 constexpr int SUBS_PER_WARP = 2;
 constexpr int MAX_BANDS = 8;
 constexpr int DEFAULT_ITEMS_PER_CTA = 0;   // before tuning: items sized by default_item_rows
+constexpr int64_t COMP_MAX_ENTRIES = 1 << 19;   // evaluated entries, see solver_J
 constexpr float CULL_MARGIN = 2e-3f;   // in units of the band's maximum detour
 
 // Per-row record, lengths in units of the row's band maximum detour U_b = c0 * dt_max_b.
@@ -211,6 +212,10 @@ struct fft_geom_s {
     float* cg_r = nullptr;               // [M] residual d - J m
     float* cg_q = nullptr;               // [M] J p
     float* cg_s = nullptr;               // [V] J^T r - lambda m
+    float* cg_ql = nullptr;              // [M] low part of q (compensated products only)
+    float* cg_sl = nullptr;              // [V] low part of s
+    double* cg_jpart = nullptr;          // [E * 4] J partials of the compensated form
+    float* cg_gpart = nullptr;           // [n_slots * TILE_VOX] low parts of its J^T partials
     float* cg_p = nullptr;               // [V] search direction
     float* cg_d = nullptr;               // [M] copy of the data
     float* cg_m = nullptr;               // [V] iterate
@@ -237,6 +242,11 @@ namespace fftgb {
 // Launch helpers implemented in fft_apply.cu (used by CG and PSF).
 fft_status launch_J(fft_geom g, const float* m, float* d, cudaStream_t st);
 fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st);
+// With compensated sums, as two floats each (has_compensated: the operators that the solver takes them for).
+bool has_compensated(fft_geom g);
+fft_status launch_J_comp(fft_geom g, const float* m, float* d, float* d_low, double* jpart64, cudaStream_t st);
+fft_status launch_JT_comp(fft_geom g, const float* din, float* gout, float* g_low, float* gpart_low,
+                          cudaStream_t st);
 fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st);
 fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_per_cta);
 fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st);

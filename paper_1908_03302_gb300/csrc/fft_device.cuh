@@ -88,6 +88,20 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+// hi + lo += a b: the rounding error of the sum goes to lo. With |hi| at least |a b| it is exact (Dekker's
+// fast two-sum, the product's own rounding included by the second FMA), else off by an ulp of a b.
+__device__ __forceinline__ void fma2_comp(f2 a, f2 b, f2& hi, f2& lo) {
+    const f2 t = fma2(a, b, hi), z = add2(t, neg2(hi));
+    lo = add2(lo, fma2(a, b, neg2(z)));
+    hi = t;
+}
+// s = a + b rounded, and what that lacks (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float& s) {
+    const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+    s = t;
+    return e;
+}
 __device__ __forceinline__ f2 rsqrt2(f2 v) {
     const float2 a = up(v);
     return pk(rsqrt_approx(a.x), rsqrt_approx(a.y));

@@ -326,7 +326,8 @@ void free_geom(fft_geom g) {
     if (g->nested) g->jpart = g->jpart4 = g->gpart = g->gpart4 = nullptr;   // the parent's
     void* ptrs[] = {g->d_band, g->rec, g->rec64, g->row_band, g->tab, g->tile_off, g->tile_rows, g->ebase, g->ebase3,
                     g->row_off, g->row_ent, g->items, g->tile_slot0, g->tile_nslot, g->jpart,
-                    g->gpart, g->counter, g->cg_r, g->cg_q, g->cg_s, g->cg_p, g->cg_d, g->cg_m,
+                    g->gpart, g->counter, g->cg_r, g->cg_q, g->cg_s, g->cg_ql, g->cg_sl, g->cg_jpart,
+                    g->cg_gpart, g->cg_p, g->cg_d, g->cg_m,
                     g->cg_scal, g->cg_dots, g->cg_status, g->cg_hist, g->vol, g->jpart4, g->gpart4,
                     g->psf_crec, g->stk_rows, g->stk_x, g->stk_d, g->stk_jpart, g->stk_gpart, g->zw};
     for (void* p : ptrs)
@@ -418,12 +419,12 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
         g->scratch_bytes -= (int64_t)(sizeof(Item) * g->n_items + 2 * sizeof(int32_t) * g->n_tiles);
         if (!g->nested) g->scratch_bytes -= (int64_t)(sizeof(float) * (size_t)g->n_slots * TILE_VOX);
     }
-    void* old[] = {g->items, g->tile_slot0, g->tile_nslot, g->gpart};
+    void* old[] = {g->items, g->tile_slot0, g->tile_nslot, g->gpart, g->cg_gpart};   // (cg_gpart: at the next solve)
     for (void* q : old)
         if (q) cudaFree(q);
     g->items = nullptr;
     g->tile_slot0 = g->tile_nslot = nullptr;
-    g->gpart = nullptr;
+    g->gpart = g->cg_gpart = nullptr;
     g->n_items = (int32_t)items.size();
     g->n_slots = slots;
     g->items_per_cta = items_per_cta;
