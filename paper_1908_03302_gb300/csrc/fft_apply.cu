@@ -247,9 +247,14 @@ static int plain_max_warps(fft_geom g) {
 }
 
 // Raise the dynamic shared-memory limit of every kernel instantiation once per geometry
-// (outside any stream capture), so launches need no attribute calls.
+// (outside any stream capture), so launches need no attribute calls. The limit belongs to the
+// kernel, not to the handle: always the device's largest, so that a handle with small tables does not
+// lower it under a live one with large tables. (Occupancy and launches go by the size that they use.)
 fft_status set_apply_attributes(fft_geom g) {
-    const size_t smem = apply_smem(g, std::max(sharp_max_warps(g), plain_max_warps(g)));
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    const size_t smem = (size_t)optin;
     fft_status rc;
     if ((rc = set_attr_mode<MODE_JT>(smem)) != FFT_OK) return rc;
     if ((rc = set_attr_mode<MODE_J>(smem)) != FFT_OK) return rc;
@@ -260,16 +265,12 @@ fft_status set_apply_attributes(fft_geom g) {
     // batch modes: stable detour only (other geometries apply the columns one by one)
     if ((rc = set_attr_mode<MODE_JT4>(smem)) != FFT_OK) return rc;
     if ((rc = set_attr_mode<MODE_J4>(smem)) != FFT_OK) return rc;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, dev);
     g->sms = std::max(g->sms, 1);
-    const size_t smem8 = apply_smem8(g, col8_warps<false>());
-    g->col8 = g->dt_mode == FFT_DT_STABLE && smem8 <= (size_t)optin;
+    g->col8 = g->dt_mode == FFT_DT_STABLE && apply_smem8(g, col8_warps<false>()) <= smem;
     if (g->col8) {
-        if ((rc = set_attr_mode<MODE_JT8>(smem8)) != FFT_OK) return rc;
-        if ((rc = set_attr_mode<MODE_J8>(smem8)) != FFT_OK) return rc;
+        if ((rc = set_attr_mode<MODE_JT8>(smem)) != FFT_OK) return rc;
+        if ((rc = set_attr_mode<MODE_J8>(smem)) != FFT_OK) return rc;
     }
     return set_attr_mode<MODE_FROB>(smem);
 }
