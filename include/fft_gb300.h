@@ -210,12 +210,15 @@ fft_status fft_JT_apply(fft_geom g, const float* d_dev, float* g_dev, void* stre
  *   m_dev  device float32, n columns of length V (column c at m_dev + c * V);
  *   d_dev  device float32, n columns of length M (column c at d_dev + c * M);
  *   g_dev  device float32, n columns of length V.
- * From four columns on they are processed in groups of up to eight (four where the scratch for
- * eight is not there); fewer, and every column of geometries with a non-stable detour mode, go
- * through the single-vector kernels. Each column matches the
- * single-vector call to rounding (same entries, same summation order). The first call
- * allocates the handle's batch scratch (E * 32 + slots * 4 * 2048 floats; twice that
- * from five columns on, where it takes at most half of the free memory).
+ * From four columns on they are processed in groups of up to eight (as two passes of four where
+ * the scratch for eight is not there: the same bits); fewer, a last column alone in its group of eight,
+ * and every column of geometries with a non-stable detour mode go through the single-vector
+ * kernels. (Elevation stacks treat a column's slices as such columns, whatever n is.) Each column
+ * matches the single-vector call to rounding. The first call allocates the handle's batch
+ * scratch (E * 32 + slots * 4 * 2048 floats); the first of five columns and more outside a
+ * stream capture adds twice that beside it, if it takes at most half of the free memory (asked
+ * once). It never moves: a captured J, J^T, coverage, 2-D or batch call stays valid until
+ * fft_geom_autotune or fft_geom_destroy.
  */
 fft_status fft_J_apply_batch(fft_geom g, const float* m_dev, int32_t n, float* d_dev, void* stream);
 fft_status fft_JT_apply_batch(fft_geom g, const float* d_dev, int32_t n, float* g_dev, void* stream);

@@ -330,50 +330,70 @@ void plain_launch_shape(fft_geom g) {
     g->plain_ctas = std::max(best_b, 1) * sms;
 }
 
-// Partials of a batch of n columns: for eight columns at once where n is more than four, the kernels
-// fit and memory allows it, else for four. Kept with the geometry, and grown unless the stream is capturing.
-static fft_status batch_scratch(fft_geom g, int n, cudaStream_t st) {
-    if (g->nested) return FFT_OK;   // the parent's (stack_scratch)
-    int cols = (n > 4 && g->col8) ? 8 : 4;
-    if (g->batch_cols >= cols) return FFT_OK;
-    if (cols == 8) {   // taken, or grown to, only with memory to spare
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        size_t mem_free = 0, mem_total = 0;
-        FFT_CUDA(cudaStreamIsCapturing(st, &cap));
-        FFT_CUDA(cudaMemGetInfo(&mem_free, &mem_total));
-        const double need = 8.0 * sizeof(float) * ((double)g->E * 8 + (double)g->n_slots * TILE_VOX);
-        if (cap != cudaStreamCaptureStatusNone || 2.0 * need > (double)mem_free) cols = 4;
-        if (g->batch_cols >= cols) return FFT_OK;
-        free_batch_scratch(g);
-    }
-    for (; cols >= 4; cols -= 4) {
-        cudaError_t e = cudaMalloc(&g->jpart4, sizeof(float) * (size_t)(g->E > 0 ? g->E : 1) * 8 * cols);
-        if (e == cudaSuccess && g->n_slots > 0)
-            e = cudaMalloc(&g->gpart4, sizeof(float) * (size_t)g->n_slots * cols * TILE_VOX);
-        if (e == cudaSuccess) {
-            g->batch_cols = cols;
-            g->scratch_bytes += batch_scratch_bytes(g);
-            return FFT_OK;
-        }
-        cudaGetLastError();
-        cudaFree(g->jpart4);
-        g->jpart4 = nullptr;
-    }
-    set_error("batch apply: cudaMalloc of the partial buffers failed");
-    return FFT_ERR_OOM;
+static int64_t batch_bytes(fft_geom g, int cols) {
+    return (int64_t)sizeof(float) * cols * (g->E * 8 + (int64_t)g->n_slots * TILE_VOX);
 }
 
-int64_t batch_scratch_bytes(fft_geom g) {
-    return (int64_t)sizeof(float) * g->batch_cols * (g->E * 8 + (int64_t)g->n_slots * TILE_VOX);
+static cudaError_t alloc_batch(fft_geom g, int cols, float** jp, float** gp) {
+    *jp = *gp = nullptr;
+    cudaError_t e = cudaMalloc(jp, sizeof(float) * (size_t)(g->E > 0 ? g->E : 1) * 8 * cols);
+    if (e == cudaSuccess && g->n_slots > 0) e = cudaMalloc(gp, sizeof(float) * (size_t)g->n_slots * cols * TILE_VOX);
+    if (e == cudaSuccess) return e;
+    cudaGetLastError();
+    cudaFree(*jp);
+    *jp = *gp = nullptr;
+    return e;
+}
+
+// Partials of a batch of n columns: for eight columns at once where n is more than four, the kernels
+// fit and memory allows it (asked once), else for four. A caller may have captured a call that uses the
+// four-column buffers, so they stay beside the eight-column ones, until new work items replace both.
+static fft_status batch_scratch(fft_geom g, int n, cudaStream_t st) {
+    if (g->nested) return FFT_OK;   // the parent's (stack_scratch)
+    const bool wide = n > 4 && g->col8 && !g->batch8_refused;
+    if (g->batch_cols == 8 || (g->batch_cols == 4 && !wide)) return FFT_OK;
+    if (wide) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        FFT_CUDA(cudaStreamIsCapturing(st, &cap));
+        if (cap == cudaStreamCaptureStatusNone) {
+            // (relaxed: growing must not break a capture that another stream is in the middle of)
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            FFT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+            size_t mem_free = 0, mem_total = 0;
+            float *jp = nullptr, *gp = nullptr;
+            const bool grown = cudaMemGetInfo(&mem_free, &mem_total) == cudaSuccess &&
+                               2.0 * (double)batch_bytes(g, 8) <= (double)mem_free &&
+                               alloc_batch(g, 8, &jp, &gp) == cudaSuccess;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            if (grown) {
+                g->jpart4_kept = g->jpart4;
+                g->gpart4_kept = g->gpart4;
+                g->jpart4 = jp;
+                g->gpart4 = gp;
+                g->batch_cols = 8;
+                g->scratch_bytes += batch_bytes(g, 8);
+                return FFT_OK;
+            }
+            g->batch8_refused = true;
+        }
+        if (g->batch_cols == 4) return FFT_OK;
+    }
+    if (alloc_batch(g, 4, &g->jpart4, &g->gpart4) != cudaSuccess) {
+        set_error("batch apply: cudaMalloc of the partial buffers failed");
+        return FFT_ERR_OOM;
+    }
+    g->batch_cols = 4;
+    g->scratch_bytes += batch_bytes(g, 4);
+    return FFT_OK;
 }
 
 void free_batch_scratch(fft_geom g) {
     if (g->nested || g->batch_cols == 0) return;
-    g->scratch_bytes -= batch_scratch_bytes(g);
-    cudaFree(g->jpart4);
-    cudaFree(g->gpart4);
-    g->jpart4 = g->gpart4 = nullptr;
+    g->scratch_bytes -= batch_bytes(g, g->batch_cols) + (g->jpart4_kept ? batch_bytes(g, 4) : 0);
+    for (float* p : {g->jpart4, g->gpart4, g->jpart4_kept, g->gpart4_kept}) cudaFree(p);
+    g->jpart4 = g->gpart4 = g->jpart4_kept = g->gpart4_kept = nullptr;
     g->batch_cols = 0;
+    g->batch8_refused = false;
 }
 
 // Columns of the next pass of rem columns: one alone, two to four in a four-column pass, five to eight
@@ -421,32 +441,49 @@ static fft_status jt_pass(fft_geom g, const float* d, int nc, float* gout, cudaS
     return launch_jt_reduce<NC>(g, g->gpart4, nc, gout, st);
 }
 
-// d[:, c] = J m[:, c] for n columns: on stable-detour geometries passes of up to eight or four columns
-// (from four columns on: fewer need no batch scratch; a stack's operator has it), single columns otherwise.
+// Columns of the next pass of n from column c on, and whether it goes through the single-column kernels:
+// fewer than four columns (they need no batch scratch; a stack's operator has it), those of other detour modes,
+// and a last column alone in its group of eight. Passes of four and eight give a column the same bits, so
+// the result does not depend on which of the two there was memory for.
+static int next_pass(fft_geom g, int n, int c, bool batch, bool& single) {
+    const int nc = batch ? pass_columns(g, n - c) : 1;
+    single = !batch || (nc == 1 && c % 8 == 0);
+    return nc;
+}
+
+// d[:, c] = J m[:, c] for n columns.
 fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st) {
     if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_J(g, m, n, d, st);
     const bool batch = g->dt_mode == FFT_DT_STABLE && (n >= 4 || g->nested);
     fft_status rc = batch ? batch_scratch(g, n, st) : FFT_OK;
     for (int c = 0; c < n && rc == FFT_OK;) {
-        const int nc = batch ? pass_columns(g, n - c) : 1;
+        bool single;
+        const int nc = next_pass(g, n, c, batch, single);
         const float* mc = m + (int64_t)c * g->V;
         float* dc = d + (int64_t)c * g->M;
-        rc = nc == 1 ? launch_J(g, mc, dc, st) : (nc > 4 ? j_pass<8, MODE_J8>(g, mc, nc, dc, st) : j_pass<4, MODE_J4>(g, mc, nc, dc, st));
+        if (single)
+            rc = launch_J(g, mc, dc, st);
+        else
+            rc = nc > 4 ? j_pass<8, MODE_J8>(g, mc, nc, dc, st) : j_pass<4, MODE_J4>(g, mc, nc, dc, st);
         c += nc;
     }
     return rc;
 }
 
-// g[:, c] = J^T d[:, c] for n columns (passes as above).
+// g[:, c] = J^T d[:, c] for n columns.
 fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st) {
     if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_JT(g, din, n, gout, st);
     const bool batch = g->dt_mode == FFT_DT_STABLE && (n >= 4 || g->nested);
     fft_status rc = batch ? batch_scratch(g, n, st) : FFT_OK;
     for (int c = 0; c < n && rc == FFT_OK;) {
-        const int nc = batch ? pass_columns(g, n - c) : 1;
+        bool single;
+        const int nc = next_pass(g, n, c, batch, single);
         const float* dc = din + (int64_t)c * g->M;
         float* gc = gout + (int64_t)c * g->V;
-        rc = nc == 1 ? launch_JT(g, dc, gc, st) : (nc > 4 ? jt_pass<8, MODE_JT8>(g, dc, nc, gc, st) : jt_pass<4, MODE_JT4>(g, dc, nc, gc, st));
+        if (single)
+            rc = launch_JT(g, dc, gc, st);
+        else
+            rc = nc > 4 ? jt_pass<8, MODE_JT8>(g, dc, nc, gc, st) : jt_pass<4, MODE_JT4>(g, dc, nc, gc, st);
         c += nc;
     }
     return rc;

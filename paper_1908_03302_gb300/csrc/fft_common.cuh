@@ -228,6 +228,8 @@ struct fft_geom_s {
     int batch_cols = 0;                  // columns that the batch partials hold: 0 (none yet), 4 or 8
     float* jpart4 = nullptr;             // [E * 8 * batch_cols] J partials of the batch applies
     float* gpart4 = nullptr;             // [n_slots * batch_cols * TILE_VOX] their J^T partials
+    float *jpart4_kept = nullptr, *gpart4_kept = nullptr;   // the four-column ones once there are eight
+    bool batch8_refused = false;         // no memory for the eight-column ones
     double* cg_hist = nullptr;           // [cg_hist_cap]
     int32_t cg_hist_cap = 0;
     void* cg_graph = nullptr;            // cudaGraphExec_t of the iteration loop
@@ -259,7 +261,6 @@ fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st)
 fft_status stack_JT(fft_geom g, const float* d, int n, float* gout, cudaStream_t st);
 fft_status stack_scratch(fft_geom g);
 int pass_columns(fft_geom g, int64_t rem);
-int64_t batch_scratch_bytes(fft_geom g);
 void free_batch_scratch(fft_geom g);
 fft_status stack_build_items(fft_geom g, int items_per_cta);
 fft_status check_device(int dev);

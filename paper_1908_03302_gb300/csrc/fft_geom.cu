@@ -329,6 +329,7 @@ void free_geom(fft_geom g) {
                     g->gpart, g->counter, g->cg_r, g->cg_q, g->cg_s, g->cg_ql, g->cg_sl, g->cg_jpart,
                     g->cg_gpart, g->cg_p, g->cg_d, g->cg_m,
                     g->cg_scal, g->cg_dots, g->cg_status, g->cg_hist, g->vol, g->jpart4, g->gpart4,
+                    g->jpart4_kept, g->gpart4_kept,
                     g->psf_crec, g->stk_rows, g->stk_x, g->stk_d, g->stk_jpart, g->stk_gpart, g->zw};
     for (void* p : ptrs)
         if (p) cudaFree(p);
