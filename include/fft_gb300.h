@@ -184,7 +184,9 @@ typedef struct {
  * For geometries with a band whose Phi does not vanish at its cut-off, J and J^T run in one
  * CTA of up to 20 warps per SM whatever the candidate; the CTA count then only sets the item
  * granularity. Synchronous; allocates test vectors for the duration of the call; invalidates
- * a captured CG loop (the next fft_cg_solve captures again). info may be NULL.
+ * a captured CG loop (the next fft_cg_solve captures again) and every other captured call on the
+ * handle. On FFT_ERR_OOM the previous decomposition stays; if even that can't be had again, calls on
+ * the handle return FFT_ERR_STATE until a later tuning succeeds. info may be NULL.
  */
 fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_t* info);
 
@@ -447,6 +449,13 @@ fft_status fft_psf_noalloc(fft_geom g, int64_t spike_vox, const int32_t* rows_de
  * Returns FFT_ERR_TIMEOUT if the bounded wait for the tensor cores gave up.
  */
 fft_status fft_tc_selftest(int32_t n, int32_t k, double* max_abs_err);
+
+/*
+ * fft_fail_alloc - diagnostic for the out-of-memory paths: on the calling thread the next `after` device
+ * allocations of handles' buffers succeed and the `count` after them report out of memory (no
+ * allocation is made). count = 0 ends it.
+ */
+void fft_fail_alloc(int32_t after, int32_t count);
 
 /* Message of the last failing call on this thread ("" if none). */
 const char* fft_last_error(void);

@@ -9,6 +9,7 @@ namespace fftgb {
 
 namespace {
 thread_local std::string g_last_error;
+thread_local int32_t g_fail_after = 0, g_fail_count = 0;   // fft_fail_alloc
 }
 
 void set_error(const std::string& msg) { g_last_error = msg; }
@@ -17,6 +18,16 @@ fft_status cuda_fail(cudaError_t e, const char* what) {
     g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
     if (e == cudaErrorMemoryAllocation) return FFT_ERR_OOM;
     return FFT_ERR_CUDA;
+}
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+    if (g_fail_count > 0 && g_fail_after-- <= 0) {
+        g_fail_after = 0;
+        --g_fail_count;
+        *p = nullptr;
+        return cudaErrorMemoryAllocation;
+    }
+    return cudaMalloc(p, bytes);
 }
 
 // Calls on a handle must run with the handle's device current.
@@ -33,5 +44,10 @@ fft_status check_device(int dev) {
 }
 
 }  // namespace fftgb
+
+extern "C" void fft_fail_alloc(int32_t after, int32_t count) {
+    fftgb::g_fail_after = after;
+    fftgb::g_fail_count = count;
+}
 
 extern "C" const char* fft_last_error(void) { return fftgb::g_last_error.c_str(); }

@@ -176,6 +176,12 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
     }
 }
 
+fft_status check_usable(fft_geom g) {
+    if (!g->unusable) return FFT_OK;
+    set_error("the operator has no work items: fft_geom_autotune ran out of memory (tune again or make a new one)");
+    return FFT_ERR_STATE;
+}
+
 static ApplyParams make_params(fft_geom g) {
     ApplyParams P;
     P.rec = g->rec;
@@ -336,8 +342,9 @@ static int64_t batch_bytes(fft_geom g, int cols) {
 
 static cudaError_t alloc_batch(fft_geom g, int cols, float** jp, float** gp) {
     *jp = *gp = nullptr;
-    cudaError_t e = cudaMalloc(jp, sizeof(float) * (size_t)(g->E > 0 ? g->E : 1) * 8 * cols);
-    if (e == cudaSuccess && g->n_slots > 0) e = cudaMalloc(gp, sizeof(float) * (size_t)g->n_slots * cols * TILE_VOX);
+    cudaError_t e = device_malloc((void**)jp, sizeof(float) * (size_t)(g->E > 0 ? g->E : 1) * 8 * cols);
+    if (e == cudaSuccess && g->n_slots > 0)
+        e = device_malloc((void**)gp, sizeof(float) * (size_t)g->n_slots * cols * TILE_VOX);
     if (e == cudaSuccess) return e;
     cudaGetLastError();
     cudaFree(*jp);

@@ -1142,6 +1142,7 @@ inline void launch_split(fft_geom g, const ApplyParams& P, cudaStream_t st) {
 
 template <int MODE>
 inline fft_status launch_mode_impl(fft_geom g, const ApplyParams& P, cudaStream_t st) {
+    if (g->unusable) return check_usable(g);
     FFT_CUDA(cudaMemsetAsync(g->counter, 0, 2 * sizeof(int32_t), st));
     if (g->n_items == 0) return FFT_OK;
     // MODE_COUNT evaluates no Phi: the table variant serves every representation
@@ -1170,6 +1171,7 @@ inline fft_status launch_mode_impl(fft_geom g, const ApplyParams& P, cudaStream_
 // The modes that exist for the stable detour only: batches, compensated sums.
 template <int MODE>
 inline fft_status launch_batch_impl(fft_geom g, const ApplyParams& P, cudaStream_t st) {
+    if (g->unusable) return check_usable(g);
     FFT_CUDA(cudaMemsetAsync(g->counter, 0, 2 * sizeof(int32_t), st));
     if (g->n_items == 0) return FFT_OK;
 #define FFT_LAUNCH_G(PV)                                                          \

@@ -174,7 +174,7 @@ __global__ void cg_update_p_kernel(float* __restrict__ p, const float* __restric
 template <typename T>
 fft_status cg_alloc(T** p, size_t n) {
     if (*p) return FFT_OK;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), (n ? n : 1) * sizeof(T));
+    cudaError_t e = device_malloc(reinterpret_cast<void**>(p), (n ? n : 1) * sizeof(T));
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("fft_cg_solve: cudaMalloc failed");

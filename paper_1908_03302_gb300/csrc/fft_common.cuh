@@ -16,6 +16,9 @@ namespace fftgb {
 void set_error(const std::string& msg);
 fft_status cuda_fail(cudaError_t e, const char* what);
 
+// cudaMalloc, except that fft_fail_alloc can make it report out of memory on the calling thread.
+cudaError_t device_malloc(void** p, size_t bytes);
+
 #define FFT_CUDA(call)                                         \
     do {                                                       \
         cudaError_t _e = (call);                               \
@@ -173,6 +176,7 @@ struct fft_geom_s {
     float* stk_gpart = nullptr;          // their J^T partials
     int64_t stk_gpart_cap = 0;           // (floats)
     bool nested = false;
+    bool unusable = false;               // new work items or their buffers could not be allocated
     uint8_t* zw = nullptr;               // nested: [nz] slices that hold the layer (support count, Frobenius norm)
     int64_t E_used = 0;                  // entries of the tiles that the products evaluate
     int32_t tiles[3];
@@ -264,6 +268,7 @@ int pass_columns(fft_geom g, int64_t rem);
 void free_batch_scratch(fft_geom g);
 fft_status stack_build_items(fft_geom g, int items_per_cta);
 fft_status check_device(int dev);
+fft_status check_usable(fft_geom g);
 fft_status count_support(fft_geom g, int64_t* support, int64_t* evaluated);
 fft_status compute_frob2(fft_geom g, double* out);
 fft_status set_apply_attributes(fft_geom g);

@@ -310,7 +310,7 @@ template <typename T>
 fft_status dmalloc(fft_geom g, T** p, size_t count) {
     *p = nullptr;
     if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), count * sizeof(T));
+    cudaError_t e = device_malloc(reinterpret_cast<void**>(p), count * sizeof(T));
     if (e != cudaSuccess) {
         cudaGetLastError();
         set_error("fft_geom_create: cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed");
@@ -366,7 +366,8 @@ static bool tile_used(fft_geom g, int64_t T) {
 // persistent CTA sees about items_per_cta items (at least 64 rows, a multiple of 32), or by
 // default_item_rows when items_per_cta is 0; tiles split over several items write J^T partial
 // slots. Heaviest items first. Replaces the geometry's previous items, slots and partial buffers
-// (the J partials do not depend on them).
+// (the J partials do not depend on them); those go first, so that tuning needs no more memory than the
+// larger of the two takes. If the new ones can't be had the operator is unusable until a later call succeeds.
 fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_per_cta) {
     // plain rows [toff, toff + nplain) and sharp-band rows [toff + nplain, toff1) of a split
     // geometry go to different items and launches; the tile's slots number its plain items first
@@ -414,6 +415,17 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
     std::stable_sort(items_sharp.begin(), items_sharp.end(), heavier);
     g->n_items_plain = (int32_t)items.size();
     items.insert(items.end(), items_sharp.begin(), items_sharp.end());
+    // a captured CG loop holds the old item list: capture again on the next solve
+    if (g->cg_graph) {
+        cudaGraphExecDestroy((cudaGraphExec_t)g->cg_graph);
+        g->cg_graph = nullptr;
+        g->cg_graph_iters = -1;
+    }
+    if (g->cg_graph_cont) {
+        cudaGraphExecDestroy((cudaGraphExec_t)g->cg_graph_cont);
+        g->cg_graph_cont = nullptr;
+        g->cg_graph_cont_iters = -1;
+    }
     if (g->nested) g->jpart4 = g->gpart = g->gpart4 = nullptr;   // the parent's (stack_scratch sets them again)
     free_batch_scratch(g);   // rebuilt with the new slot count on first use
     if (g->items) {          // the buffers below are replaced: take them out of the scratch count
@@ -429,29 +441,32 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
     g->n_items = (int32_t)items.size();
     g->n_slots = slots;
     g->items_per_cta = items_per_cta;
-    fft_status rc;
-    if ((rc = dmalloc(g, &g->items, items.size())) != FFT_OK) return rc;
-    if ((rc = dmalloc(g, &g->tile_slot0, g->n_tiles)) != FFT_OK) return rc;
-    if ((rc = dmalloc(g, &g->tile_nslot, g->n_tiles)) != FFT_OK) return rc;
-    if (!g->nested && (rc = dmalloc(g, &g->gpart, (size_t)slots * TILE_VOX)) != FFT_OK) return rc;
+    g->unusable = true;
+    const int64_t before = g->scratch_bytes;
+    fft_status rc = dmalloc(g, &g->items, items.size());
+    if (rc == FFT_OK) rc = dmalloc(g, &g->tile_slot0, g->n_tiles);
+    if (rc == FFT_OK) rc = dmalloc(g, &g->tile_nslot, g->n_tiles);
+    if (rc == FFT_OK && !g->nested) rc = dmalloc(g, &g->gpart, (size_t)slots * TILE_VOX);
     cudaError_t e = cudaSuccess;
-    if (!items.empty()) e = cudaMemcpy(g->items, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
+    if (rc == FFT_OK && !items.empty())
+        e = cudaMemcpy(g->items, items.data(), sizeof(Item) * items.size(), cudaMemcpyHostToDevice);
+    if (rc == FFT_OK && e == cudaSuccess)
         e = cudaMemcpy(g->tile_slot0, slot0.data(), sizeof(int32_t) * g->n_tiles, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
+    if (rc == FFT_OK && e == cudaSuccess)
         e = cudaMemcpy(g->tile_nslot, nslot.data(), sizeof(int32_t) * g->n_tiles, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return cuda_fail(e, "work items");
-    // a captured CG loop holds the old item list: capture again on the next solve
-    if (g->cg_graph) {
-        cudaGraphExecDestroy((cudaGraphExec_t)g->cg_graph);
-        g->cg_graph = nullptr;
-        g->cg_graph_iters = -1;
+    if (e != cudaSuccess) rc = cuda_fail(e, "work items");
+    if (rc != FFT_OK) {
+        void* got[] = {g->items, g->tile_slot0, g->tile_nslot, g->gpart};
+        for (void* q : got)
+            if (q) cudaFree(q);
+        g->items = nullptr;
+        g->tile_slot0 = g->tile_nslot = nullptr;
+        g->gpart = nullptr;
+        g->n_items = g->n_items_plain = g->n_slots = 0;
+        g->scratch_bytes = before;
+        return rc;
     }
-    if (g->cg_graph_cont) {
-        cudaGraphExecDestroy((cudaGraphExec_t)g->cg_graph_cont);
-        g->cg_graph_cont = nullptr;
-        g->cg_graph_cont_iters = -1;
-    }
+    g->unusable = false;
     return FFT_OK;
 }
 
@@ -478,6 +493,7 @@ fft_status stack_scratch(fft_geom g) {
 
 // Work items of the operators of a stack (the autotuner's candidates).
 fft_status stack_build_items(fft_geom g, int items_per_cta) {
+    g->unusable = true;   // the classes' operators lose their buffers here, until stack_scratch succeeds
     for (StackClass& c : g->stk) {
         std::vector<int64_t> toff(c.sub->n_tiles + 1);
         FFT_CUDA(cudaMemcpy(toff.data(), c.sub->tile_off, sizeof(int64_t) * toff.size(), cudaMemcpyDeviceToHost));
@@ -485,7 +501,9 @@ fft_status stack_build_items(fft_geom g, int items_per_cta) {
         const fft_status rc = build_items(c.sub, toff, items_per_cta);
         if (rc != FFT_OK) return rc;
     }
-    return stack_scratch(g);
+    const fft_status rc = stack_scratch(g);
+    g->unusable = rc != FFT_OK;
+    return rc;
 }
 
 namespace {

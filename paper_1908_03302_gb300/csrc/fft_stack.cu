@@ -202,6 +202,7 @@ double stack_entries(fft_geom g, int64_t n) {
 }
 
 fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st) {
+    if (g->unusable) return check_usable(g);
     const int64_t plane = (int64_t)g->grid.nx * g->grid.ny;
     return for_each_pass(g, n, [&](fft_geom sub, const StackJobs& J) -> fft_status {
         stack_models_kernel<<<dim3((unsigned)ceil_div(sub->V, 256), J.n), 256, 0, st>>>(J, m, g->V, plane, sub->V, g->stk_x);
@@ -215,6 +216,7 @@ fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st)
 }
 
 fft_status stack_JT(fft_geom g, const float* d, int n, float* gout, cudaStream_t st) {
+    if (g->unusable) return check_usable(g);
     const int64_t plane = (int64_t)g->grid.nx * g->grid.ny;
     return for_each_pass(g, n, [&](fft_geom sub, const StackJobs& J) -> fft_status {
         stack_gather_kernel<<<dim3((unsigned)ceil_div(sub->M, 256), J.n), 256, 0, st>>>(J, d, g->M, sub->M, g->stk_d);

@@ -62,10 +62,15 @@ extern "C" fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_
     const int n_cand = 6;
     double best = 1e300, best_j = 0.0, best_jt = 0.0, last = 0.0;
     int best_items = g->items_per_cta, best_ctas = g->apply_ctas / std::max(sms, 1), tried = 0, best_ii = 0;
+    // Items of the operator and, for an elevation stack, of its classes' operators.
+    auto set_items = [&](int n_ctas, int items_per_cta) {
+        g->apply_ctas = n_ctas;
+        const fft_status r = build_items(g, toff, items_per_cta);
+        return r == FFT_OK && !g->stk.empty() ? stack_build_items(g, items_per_cta) : r;
+    };
+    const int old_ctas = g->apply_ctas, old_items = g->items_per_cta;
     auto try_one = [&](int ctas, int ii) -> bool {
-        g->apply_ctas = ctas * sms;
-        if ((rc = build_items(g, toff, cand_items[ii])) != FFT_OK) return false;
-        if (!g->stk.empty() && (rc = stack_build_items(g, cand_items[ii])) != FFT_OK) return false;
+        if ((rc = set_items(ctas * sms, cand_items[ii])) != FFT_OK) return false;
         if (tried == 0 || last < 20.0) {
             if ((rc = launch_JT(g, d, out_v, st)) != FFT_OK) return false;
             if ((rc = launch_J(g, m, out_m, st)) != FFT_OK) return false;
@@ -106,10 +111,10 @@ extern "C" fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_
         }
     }
     if (e == cudaSuccess && rc == FFT_OK) {
-        g->apply_ctas = best_ctas * sms;
-        rc = build_items(g, toff, best_items);
-        if (rc == FFT_OK && !g->stk.empty()) rc = stack_build_items(g, best_items);
+        rc = set_items(best_ctas * sms, best_items);
     }
+    // an operator that lost its items to a failed allocation gets the ones back that it came with
+    if (g->unusable) set_items(old_ctas, old_items);
     if (e == cudaSuccess && rc == FFT_OK) e = cudaStreamSynchronize(st);
     cudaFree(m);
     cudaFree(d);
