@@ -166,7 +166,7 @@ fft_status fft_geom_info(fft_geom g, fft_geom_info_t* info);
 
 /* Result of fft_geom_autotune. */
 typedef struct {
-    int32_t items_per_cta; /* chosen work-item granularity (items per persistent CTA) */
+    int32_t items_per_cta; /* chosen work-item granularity (items per persistent CTA; nearest listed) */
     int32_t ctas_per_sm;   /* chosen persistent CTAs per SM of the J / J^T kernels */
     double ms_J, ms_JT;    /* their measured times with the chosen decomposition */
     int32_t n_tried;       /* candidates timed */
@@ -174,13 +174,16 @@ typedef struct {
 
 /*
  * fft_geom_autotune - pick the work decomposition of J and J^T for this geometry by timing
- * them on the device (without it a rule on the number of entries sizes the items): a tile's candidate rows are cut into work items sized for 4, 8, 16, 32,
+ * them on the device. Without it a rule on the number of entries sizes the items; that rule's sizes
+ * are timed first, then a tile's candidate rows cut into work items sized for 4, 8, 16, 32,
  * 64 or 128 items per persistent CTA (at least 64 rows each), with the most CTAs per SM that
  * fit or one fewer. The sizes are swept at the occupancy limit (stopping after two in a row
- * more than 2 % slower than the best), then the best size and its two neighbours with one CTA
- * per SM fewer: 2 to 9 candidates. Each runs J^T and J once timed (CUDA events on `stream`),
- * after one untimed pass unless the previous candidate's pair took over 20 ms, and the
- * fastest is kept. Results do not depend on the choice beyond rounding of the split J^T sums.
+ * more than 2 % slower than the best of them), then the best size and its two neighbours with one
+ * CTA per SM fewer: 3 to 9 candidates. Each runs J^T and J timed (CUDA events on `stream`): the
+ * least of three after an untimed pass, one of each where the pair takes over 20 ms. The fastest is
+ * kept, the rule's sizes unless another one is more than 2 % faster (items_per_cta is then the
+ * listed size nearest to them). Results do not depend on the choice beyond rounding of the split
+ * J^T sums.
  * For geometries with a band whose Phi does not vanish at its cut-off, J and J^T run in one
  * CTA of up to 20 warps per SM whatever the candidate; the CTA count then only sets the item
  * granularity. Synchronous; allocates test vectors for the duration of the call; invalidates

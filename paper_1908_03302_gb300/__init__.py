@@ -174,8 +174,8 @@ class Geometry:
         return out
 
     def autotune(self, stream=None) -> dict:
-        """Time J and J^T for twelve work decompositions (items per CTA x CTAs per SM) and keep
-        the fastest (fft_geom_autotune)."""
+        """Time J and J^T for up to nine work decompositions (the untuned one, and items per CTA x CTAs
+        per SM) and keep the fastest (fft_geom_autotune)."""
         out = _lib.fft_tune_info_t()
         check(_lib.load().fft_geom_autotune(self.handle, _stream_handle(stream), ctypes.byref(out)))
         return {"items_per_cta": out.items_per_cta, "ctas_per_sm": out.ctas_per_sm, "ms_J": out.ms_J,
