@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
         auto add = [&](const float4& x) {
             const float xv[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {   // Kahan's sum
+            for (int k = 0; k < 4; ++k) {   // Kahan's sum (an infinite one, of infinite data, has nothing to add)
                 const float y = xv[k] - low[k], t = acc[k] + y;
-                low[k] = (t - acc[k]) - y;
+                low[k] = isinf(t) ? 0.0f : (t - acc[k]) - y;
                 acc[k] = t;
             }
         };
