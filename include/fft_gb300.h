@@ -164,6 +164,19 @@ typedef struct {
 } fft_geom_info_t;
 fft_status fft_geom_info(fft_geom g, fft_geom_info_t* info);
 
+/* How a geometry's products are evaluated now (diagnostic; the results do not depend on it beyond
+ * rounding). */
+typedef struct {
+    int32_t mirror;        /* layers k and mirror - k share one evaluation; -1: no mirror plane */
+    int32_t stack_classes; /* classes of slices that share one; 0: not an elevation stack (a stack is
+                              also left out where its operators do not fit the memory at creation) */
+    int32_t stack_batch;   /* 1: batches go through the classes too */
+    int32_t batch_cols;    /* columns of the batch scratch: 0 (no batch yet), 4 or 8 */
+    int32_t segments;      /* sine series: quadratic segments per band; 0: tables, or the recurrence */
+    int32_t solver_comp;   /* 1: solves use compensated products */
+} fft_route_t;
+fft_status fft_geom_route(fft_geom g, fft_route_t* route);
+
 /* Result of fft_geom_autotune. */
 typedef struct {
     int32_t items_per_cta; /* chosen work-item granularity (items per persistent CTA; nearest listed) */

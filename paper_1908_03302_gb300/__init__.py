@@ -173,6 +173,12 @@ class Geometry:
         check(_lib.load().fft_geom_info(self.handle, ctypes.byref(out)))
         return out
 
+    def route(self) -> dict:
+        """How the products are evaluated now (fft_geom_route): mirror plane, stack classes, batch width ..."""
+        out = _lib.fft_route_t()
+        check(_lib.load().fft_geom_route(self.handle, ctypes.byref(out)))
+        return {n: getattr(out, n) for n, _ in out._fields_}
+
     def autotune(self, stream=None) -> dict:
         """Time J and J^T for up to nine work decompositions (the untuned one, and items per CTA x CTAs
         per SM) and keep the fastest (fft_geom_autotune)."""

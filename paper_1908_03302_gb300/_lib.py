@@ -64,6 +64,11 @@ class fft_geom_info_t(ctypes.Structure):
                 ("psf_tc_mma_flops", ctypes.c_double), ("psf_tc_entries", ctypes.c_double)]
 
 
+class fft_route_t(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int32) for n in ("mirror", "stack_classes", "stack_batch", "batch_cols", "segments",
+                                              "solver_comp")]
+
+
 # (name, restype, argtypes) for every function declared in include/fft_gb300.h
 _VP, _I32, _I64, _D = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_double
 SIGNATURES = {
@@ -74,6 +79,7 @@ SIGNATURES = {
                                        _I32, ctypes.POINTER(_VP)]),
     "fft_geom_destroy": (None, [_VP]),
     "fft_geom_info": (ctypes.c_int, [_VP, ctypes.POINTER(fft_geom_info_t)]),
+    "fft_geom_route": (ctypes.c_int, [_VP, ctypes.POINTER(fft_route_t)]),
     "fft_geom_autotune": (ctypes.c_int, [_VP, _VP, ctypes.POINTER(fft_tune_info_t)]),
     "fft_J_apply": (ctypes.c_int, [_VP, _VP, _VP, _VP]),
     "fft_JT_apply": (ctypes.c_int, [_VP, _VP, _VP, _VP]),

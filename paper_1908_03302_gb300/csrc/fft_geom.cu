@@ -1006,6 +1006,17 @@ extern "C" void fft_geom_destroy(fft_geom g) {
     if (cur != dev) cudaSetDevice(cur);
 }
 
+extern "C" fft_status fft_geom_route(fft_geom g, fft_route_t* route) {
+    FFT_ARG(g && route, "fft_geom_route: null argument");
+    route->mirror = g->mirror;
+    route->stack_classes = (int32_t)g->stk.size();
+    route->stack_batch = g->stk_batch ? 1 : 0;
+    route->batch_cols = g->batch_cols;
+    route->segments = g->seg_n;
+    route->solver_comp = has_compensated(g) ? 1 : 0;
+    return FFT_OK;
+}
+
 extern "C" fft_status fft_geom_info(fft_geom g, fft_geom_info_t* info) {
     FFT_ARG(g && info, "fft_geom_info: null argument");
     info->n_rows = g->M;
