@@ -810,7 +810,9 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                         c2v[1] = c2;
                         c3v[1] = c3;
                         c12v[1] = PL ? c12_planar : __fmul_rn(c1, c1);
-                        if (DT == FFT_DT_STABLE && ((cw >> (24 + h)) & 1u)) {
+                        // (the recurrence, inlined at each use, is one use fewer per layer without it: five series cut
+                        // after six periods, 96 elements, J 9.4 ms with and 6.1 ms without, 7.1 ms by the general form)
+                        if (DT == FFT_DT_STABLE && PHI != PHI_TRIG && ((cw >> (24 + h)) & 1u)) {
                             f2 v[2][2], w[2][2];
                             eval_deep<2, SH, PL>(psv, prv, c2v, c3v, c12v, hy, hz, dr, v, w, near);
                             accumulate(2 * h, v[0], w[0]);
