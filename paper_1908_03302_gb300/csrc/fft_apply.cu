@@ -450,11 +450,12 @@ static fft_status jt_pass(fft_geom g, const float* d, int nc, float* gout, cudaS
 
 // Columns of the next pass of n from column c on, and whether it goes through the single-column kernels:
 // fewer than four columns (they need no batch scratch; a stack's operator has it), those of other detour modes,
-// and a last column alone in its group of eight. Passes of four and eight give a column the same bits, so
-// the result does not depend on which of the two there was memory for.
+// and a last column alone in its group of eight (of four where the tables leave no room for the kernels of
+// eight). Passes of four and eight give a column the same bits, so the result does not depend on which of
+// the two there was memory for.
 static int next_pass(fft_geom g, int n, int c, bool batch, bool& single) {
     const int nc = batch ? pass_columns(g, n - c) : 1;
-    single = !batch || (nc == 1 && c % 8 == 0);
+    single = !batch || (nc == 1 && c % (g->col8 ? 8 : 4) == 0);
     return nc;
 }
 
