@@ -192,11 +192,11 @@ typedef struct {
  * 64 or 128 items per persistent CTA (at least 64 rows each), with the most CTAs per SM that
  * fit or one fewer. The sizes are swept at the occupancy limit (stopping after two in a row
  * more than 2 % slower than the best of them), then the best size and its two neighbours with one
- * CTA per SM fewer: 3 to 9 candidates. Each runs J^T and J timed (CUDA events on `stream`): the
- * least of three after an untimed pass, one of each where the pair takes over 20 ms. The fastest is
- * kept, the rule's sizes unless another one is more than 2 % faster (items_per_cta is then the
- * listed size nearest to them). Results do not depend on the choice beyond rounding of the split
- * J^T sums.
+ * CTA per SM fewer: 2 to 9 candidates, sizes that come to the same items once. Each runs J^T and
+ * J timed (CUDA events on `stream`): the least of three after an untimed pass, one of each where
+ * the pair takes over 20 ms. The fastest is kept, the rule's sizes unless another one is more than
+ * 2 % faster (items_per_cta is then the listed size nearest to them). Results do not depend on
+ * the choice beyond rounding of the split J^T sums.
  * For geometries with a band whose Phi does not vanish at its cut-off, J and J^T run in one
  * CTA of up to 20 warps per SM whatever the candidate; the CTA count then only sets the item
  * granularity. Synchronous; allocates test vectors for the duration of the call; invalidates

@@ -255,6 +255,7 @@ fft_status launch_JT_comp(fft_geom g, const float* din, float* gout, float* g_lo
                           cudaStream_t st);
 fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st);
 fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_per_cta);
+int64_t item_rows(int64_t E, int items_per_cta, int ctas);
 fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st);
 bool find_stack(const double* tx, const int32_t* rows, int64_t M, const int32_t* band, const fft_grid& gr,
                 std::vector<StackPlan>& plan);

@@ -356,6 +356,13 @@ int64_t default_item_rows(int64_t E) {
     return n < 32 ? n : ceil_div(n, 32) * 32;
 }
 
+// Rows per work item for about items_per_cta items per persistent CTA.
+int64_t item_rows(int64_t E, int items_per_cta, int ctas) {
+    const int64_t target = (int64_t)items_per_cta * ctas;
+    const int64_t ch = std::max<int64_t>(64, ceil_div(std::max<int64_t>(E, 1), std::max<int64_t>(target, 1)));
+    return ceil_div(ch, 32) * 32;
+}
+
 // Does tile T hold layers the products evaluate?
 static bool tile_used(fft_geom g, int64_t T) {
     const int64_t tz = T / ((int64_t)g->tiles[0] * g->tiles[1]);
@@ -374,9 +381,7 @@ fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_p
     const bool split = !g->tile_nplain.empty();
     int64_t chp, chs;   // rows per plain and per sharp item
     if (items_per_cta > 0) {
-        const int64_t target = (int64_t)items_per_cta * g->apply_ctas;
-        chp = std::max<int64_t>(64, ceil_div(std::max<int64_t>(g->E, 1), std::max<int64_t>(target, 1)));
-        chp = chs = ceil_div(chp, 32) * 32;
+        chp = chs = item_rows(g->E, items_per_cta, g->apply_ctas);
     } else {
         int64_t Ep = 0, Es = 0;   // entries of the two launches
         for (int64_t T = 0; T < g->n_tiles; ++T) {

@@ -72,6 +72,16 @@ extern "C" fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_
         const fft_status r = build_items(g, toff, items_per_cta);
         return r == FFT_OK && !g->stk.empty() ? stack_build_items(g, items_per_cta) : r;
     };
+    // The listed sizes of small operators come to the same rows an item: one of them is timed.
+    const bool wide = g->plain_warps > APPLY_WARPS && g->phi_eval != PHI_TRIG && g->dt_mode == FFT_DT_STABLE;
+    std::vector<std::vector<int64_t>> seen;
+    auto timed_before = [&](int ctas, int ii) {
+        std::vector<int64_t> key = {wide ? 0 : ctas, item_rows(g->E, cand_items[ii], ctas * sms)};
+        for (const StackClass& k : g->stk) key.push_back(item_rows(k.sub->E, cand_items[ii], ctas * sms));
+        if (std::find(seen.begin(), seen.end(), key) != seen.end()) return true;
+        seen.push_back(key);
+        return false;
+    };
     const int old_ctas = g->apply_ctas, old_items = g->items_per_cta;
     auto try_one = [&](int ctas, int ii) -> bool {
         if ((rc = set_items(ctas * sms, cand_items[ii])) != FFT_OK) return false;
@@ -110,7 +120,7 @@ extern "C" fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_
     if (e == cudaSuccess && try_one(occ, 0)) {
         int worse = 0, centre = 1;
         double swept = 1e300;   // the best of the listed sizes
-        for (int ii = 1; ii < n_cand; ++ii) {
+        for (int ii = 1; ii < n_cand && !timed_before(occ, ii); ++ii) {   // (then the larger ones are alike too)
             if (!try_one(occ, ii)) break;
             worse = (last > 1.02 * swept) ? worse + 1 : 0;
             if (worse == 2) break;
@@ -121,7 +131,7 @@ extern "C" fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_
         }
         if (e == cudaSuccess && rc == FFT_OK && occ > 1) {
             for (int ii = std::max(1, centre - 1); ii <= std::min(n_cand - 1, centre + 1) && tried < max_tried; ++ii)
-                if (!try_one(occ - 1, ii)) break;
+                if (!timed_before(occ - 1, ii) && !try_one(occ - 1, ii)) break;
         }
     }
     if (e == cudaSuccess && rc == FFT_OK) rc = set_items(best_ctas * sms, best_items);
