@@ -171,6 +171,7 @@ typedef struct {
     int32_t stack_classes; /* classes of slices that share one; 0: not an elevation stack (a stack is
                               also left out where its operators do not fit the memory at creation) */
     int32_t stack_batch;   /* 1: batches go through the classes too */
+    int32_t stack_psf;     /* FP32 PSFs do in mode 0 (bit 0), in mode 2 (bit 1) */
     int32_t batch_cols;    /* columns of the batch scratch: 0 (no batch yet), 4 or 8 */
     int32_t segments;      /* sine series: quadratic segments per band; 0: tables, or the recurrence */
     int32_t solver_comp;   /* 1: solves use compensated products */

@@ -65,7 +65,7 @@ class fft_geom_info_t(ctypes.Structure):
 
 
 class fft_route_t(ctypes.Structure):
-    _fields_ = [(n, ctypes.c_int32) for n in ("mirror", "stack_classes", "stack_batch", "batch_cols", "segments",
+    _fields_ = [(n, ctypes.c_int32) for n in ("mirror", "stack_classes", "stack_batch", "stack_psf", "batch_cols", "segments",
                                               "solver_comp")]
 
 

@@ -479,8 +479,8 @@ fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStrea
 }
 
 // g[:, c] = J^T d[:, c] for n columns.
-fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st) {
-    if (!g->stk.empty() && (n < 4 || g->stk_batch)) return stack_JT(g, din, n, gout, st);
+fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st, bool sparse) {
+    if (!g->stk.empty() && (n < 4 || g->stk_batch) && (!sparse || g->stk_psf4)) return stack_JT(g, din, n, gout, st);
     const bool batch = g->dt_mode == FFT_DT_STABLE && (n >= 4 || g->nested);
     fft_status rc = batch ? batch_scratch(g, n, st) : FFT_OK;
     for (int c = 0; c < n && rc == FFT_OK;) {
@@ -512,8 +512,8 @@ fft_status launch_J(fft_geom g, const float* m, float* d, cudaStream_t st) {
     return FFT_OK;
 }
 
-fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st) {
-    if (!g->stk.empty()) return stack_JT(g, din, 1, gout, st);
+fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st, bool sparse) {
+    if (!g->stk.empty() && (!sparse || g->stk_psf1)) return stack_JT(g, din, 1, gout, st);
     ApplyParams P = make_params(g);
     P.vin = din;
     P.vout = gout;

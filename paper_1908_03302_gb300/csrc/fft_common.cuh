@@ -169,6 +169,7 @@ struct fft_geom_s {
     // parent's partial buffers; theirs (`nested`) are never allocated or freed on their own.
     std::vector<fftgb::StackClass> stk;
     bool stk_batch = false;
+    bool stk_psf1 = false, stk_psf4 = false;   // PSFs: J^T of one, of four sparse columns through them (sparse_pays)
     int32_t* stk_rows = nullptr;         // [M] the slices' rows, class by class
     float* stk_x = nullptr;              // [columns of a pass x extended voxels]
     float* stk_d = nullptr;              // [columns of a pass x rows of a slice]
@@ -247,7 +248,8 @@ struct fft_geom_s {
 namespace fftgb {
 // Launch helpers implemented in fft_apply.cu (used by CG and PSF).
 fft_status launch_J(fft_geom g, const float* m, float* d, cudaStream_t st);
-fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st);
+// (sparse: most rows of din are zero, as in the PSFs)
+fft_status launch_JT(fft_geom g, const float* din, float* gout, cudaStream_t st, bool sparse = false);
 // With compensated sums, as two floats each (has_compensated: the operators that the solver takes them for).
 bool has_compensated(fft_geom g);
 fft_status launch_J_comp(fft_geom g, const float* m, float* d, float* d_low, double* jpart64, cudaStream_t st);
@@ -256,7 +258,7 @@ fft_status launch_JT_comp(fft_geom g, const float* din, float* gout, float* g_lo
 fft_status launch_J_batch(fft_geom g, const float* m, int n, float* d, cudaStream_t st);
 fft_status build_items(fft_geom g, const std::vector<int64_t>& toff, int items_per_cta);
 int64_t item_rows(int64_t E, int items_per_cta, int ctas);
-fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st);
+fft_status launch_JT_batch(fft_geom g, const float* din, int n, float* gout, cudaStream_t st, bool sparse = false);
 bool find_stack(const double* tx, const int32_t* rows, int64_t M, const int32_t* band, const fft_grid& gr,
                 std::vector<StackPlan>& plan);
 double stack_cost(const std::vector<StackPlan>& plan, int64_t M, const fft_grid& gr);

@@ -528,6 +528,22 @@ void drop_stack(fft_geom g) {
     g->stk_gpart_cap = 0;
 }
 
+// Do J^T of sparse columns, the PSFs, go through the classes? Few rows have a weight, so that the general path
+// does little, while a class's pass costs what its slices' extended volumes take to write, reduce and add,
+// and five launches. Measured by the entries per voxel of those volumes (fill), six PSFs, general path against
+// classes, one column at a time and four: 64 elements in 11 slices (fill 0.11) 1.89 against 2.27 and 1.71
+// against 2.92 ms, 100 in 5 (0.23) 2.28 / 1.67 and 2.14 / 2.28, 128 in 7 (0.26) 3.27 / 2.71 and 3.15 / 3.06,
+// 128 in 2 (0.6) 2.49 / 1.71 and 2.29 / 1.74, 200 in 11 (0.7) 41.3 / 15.6 and 32.3 / 18.1; three classes of
+// 96 in 9 (1.3e6 entries) 1.89 / 2.21 and 1.71 / 1.72.
+void sparse_pays(fft_geom g) {
+    double vox = 0.0;
+    for (const StackClass& c : g->stk) vox += (double)c.off.size() * (double)c.sub->V;
+    const double fill = (double)g->E_used / vox;
+    const bool enough = g->E_used >= STACK_MIN_ENTRIES / 2 * (int64_t)g->stk.size();
+    g->stk_psf1 = enough && fill >= 0.2;
+    g->stk_psf4 = enough && fill >= 0.3;
+}
+
 // Operators of an elevation stack's classes where they pay: from STACK_MIN_ENTRIES entries (below, a
 // product is bound by launches and the classes add more of them: a PSF of ten 57-element slices, about
 // 6e5 entries of which few have a weight, 0.35 -> 0.41 ms with them), with at most 0.8 of the entries of a
@@ -612,6 +628,7 @@ void build_stack(fft_geom g, const double* tx, const int32_t* rows, const int32_
     }
     // several columns at once: against passes of the same width over all rows
     g->stk_batch = stack_entries(g, 8) <= pass_cost(8, g->col8) * (double)g->E_used;
+    sparse_pays(g);
 }
 
 }  // namespace
@@ -1016,6 +1033,7 @@ extern "C" fft_status fft_geom_route(fft_geom g, fft_route_t* route) {
     route->mirror = g->mirror;
     route->stack_classes = (int32_t)g->stk.size();
     route->stack_batch = g->stk_batch ? 1 : 0;
+    route->stack_psf = (g->stk_psf1 ? 1 : 0) + (g->stk_psf4 ? 2 : 0);
     route->batch_cols = g->batch_cols;
     route->segments = g->seg_n;
     route->solver_comp = has_compensated(g) ? 1 : 0;

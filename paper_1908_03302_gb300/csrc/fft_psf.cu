@@ -287,7 +287,7 @@ fft_status psf_fp32_batched(fft_geom g, const int64_t* spike_vox, int32_t n_spik
             e = cudaGetLastError();
         }
         if (e != cudaSuccess) break;
-        if ((rc = launch_JT_batch(g, D4, 4, Y4, st)) != FFT_OK) break;
+        if ((rc = launch_JT_batch(g, D4, 4, Y4, st, true)) != FFT_OK) break;
         for (int j = 0; j < nc && e == cudaSuccess; ++j) {
             const int k = (int)((c0 + j) / n_subsets), s = (int)((c0 + j) % n_subsets);
             e = cudaMemcpyAsync(out_dev + ((int64_t)s * n_spike + k) * g->V, Y4 + (int64_t)j * g->V,
@@ -370,7 +370,7 @@ extern "C" fft_status fft_psf_batch(fft_geom g, const int64_t* spike_vox, int32_
                 e = cudaGetLastError();
                 if (e != cudaSuccess) break;
             }
-            rc = launch_JT(g, D, out_dev + ((int64_t)s * n_spike + k) * g->V, st);
+            rc = launch_JT(g, D, out_dev + ((int64_t)s * n_spike + k) * g->V, st, true);
         }
     }
     cudaError_t e2 = cudaStreamSynchronize(st);

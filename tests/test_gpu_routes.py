@@ -53,6 +53,30 @@ def test_stacks(fg, layers, nz, order, odd, stack, series):
     assert gen.route()["stack_classes"] == 0 and gen.route()["mirror"] == -1
 
 
+@pytest.mark.parametrize("n_tx,n,step,grid,classes,psf", [
+    (64, 11, 3e-3, (120, 113, 40, 1e-3), 1, 0), (100, 5, 8e-3, (120, 113, 60, 1e-3), 1, 1),
+    (128, 2, 3e-3, (180, 173, 40, 1e-3), 1, 3), (96, 9, 2e-3, (100, 93, 30, 1.5e-3), 3, 0)])
+def test_sparse_columns_of_stacks(fg, n_tx, n, step, grid, classes, psf):
+    """PSFs take the classes where a stack is dense enough in entries, in either mode the values of the general path
+    (2e-6: each is within 1e-6 of the exact PSF)."""
+    ring, pairs = wl.ring(n_tx, 85e-3), wl.unordered_pairs(range(n_tx))
+    tx = np.concatenate([ring + [0.0, 0.0, (k - (n - 1) / 2) * step] for k in range(n)])
+    rows = np.concatenate([pairs + n_tx * k for k in range(n)]).astype(np.int32)
+    far = np.array([[0.5, 0.5, 0.5], [0.51, 0.5, 0.53]])
+    tab = fg.Table(1.0e6, 0.4e6)
+    geo = fg.Geometry(tx, rows, wl.Grid.centred(*grid), 1500.0, [tab])
+    gen = fg.Geometry(np.concatenate([tx, far]), np.concatenate([rows, [[len(tx), len(tx) + 1]]]).astype(np.int32),
+                      wl.Grid.centred(*grid), 1500.0, [tab])
+    assert (geo.route()["stack_classes"], geo.route()["stack_psf"]) == (classes, psf)
+    nx, ny, nz, _ = grid
+    middle = (nz // 2 * ny + ny // 2) * nx + nx // 2
+    spikes = np.array([middle, middle + 7], dtype=np.int64)
+    subs = [np.arange(geo.M, dtype=np.int32), np.arange(0, geo.M, 2, dtype=np.int32)]
+    for mode in (0, 2):
+        a, b = (g.psf_batch(spikes, subs, mode=mode).double() for g in (geo, gen))
+        assert float((a - b).norm() / b.norm()) <= 2e-6
+
+
 def test_batch_width_grows_once(fg):
     geo, _ = gpu_geometry(wl.slices32())
     rng = np.random.default_rng(4)
@@ -77,5 +101,5 @@ def test_batch_width_grows_once(fg):
 
 def test_large_solves_keep_plain_products(fg):
     geo, _ = gpu_geometry(wl.ring256())
-    assert geo.route() == {"mirror": wl.ring256().grid.nz - 1, "stack_classes": 0, "stack_batch": 0, "batch_cols": 0,
+    assert geo.route() == {"mirror": wl.ring256().grid.nz - 1, "stack_classes": 0, "stack_batch": 0, "stack_psf": 0, "batch_cols": 0,
                            "segments": 0, "solver_comp": 0}
