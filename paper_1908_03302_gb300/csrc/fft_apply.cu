@@ -87,9 +87,9 @@ __global__ void __launch_bounds__(256) j_reduce_n_kernel(const int64_t* __restri
 // g for voxels of tiles with several items (the sum of their slots) or with none (0); tiles with
 // one item were written by the apply kernel. A CTA takes 32 runs of 4 x voxels of a tile, a lane
 // each; warp w adds slots w, w + 8, .. in that order (compensated, so that the sum does not lose
-// to the number of slots), the eight partial sums are added in FP64: a fixed order, and eight times
+// to the number of slots), the eight partial sums are added as two floats: a fixed order, and eight times
 // as many loads in flight as with one thread per run, which a tile cut into many small items
-// needs (32-element ring: about 45 slots per tile).
+// needs (32-element ring: about 45 slots per tile). (In FP64 those eight took half of the kernel.)
 // NCOL = 4, 8: the batch forms, slot q of column r at gpart[((s0 + q) * NCOL + r) * TILE_VOX],
 // g[r * V + v], columns r < ncol. LOW (the compensated form, one column): the partials have low
 // parts (gpart_low), and what g lacks after rounding goes to g_low.
@@ -156,17 +156,17 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
         if (LOW) sh_low[w][lane] = make_float4(low[0], low[1], low[2], low[3]);
         __syncthreads();
         if (w < 4) {   // warp w: component w of the 32 runs
-            double s = 0.0;
+            float s = 0.0f, l = 0.0f;   // the sum and what it lacks
 #pragma unroll
             for (int k = 0; k < RED_WARPS; ++k) {
-                s += (double)reinterpret_cast<const float*>(&sh[k][lane])[w];
-                if (LOW) s += (double)reinterpret_cast<const float*>(&sh_low[k][lane])[w];
+                l += two_sum(s, reinterpret_cast<const float*>(&sh[k][lane])[w], s);
+                if (LOW) l += reinterpret_cast<const float*>(&sh_low[k][lane])[w];
             }
+            if (!isinf(s)) l = two_sum(s, l, s);
             if (inside && ix + w < nx) {
-                g[(int64_t)r * V + v + w] = (float)s;
-                if (mo != 0) g[(int64_t)r * V + v + mo + w] = (float)s;
+                g[(int64_t)r * V + v + w] = s;
+                if (mo != 0) g[(int64_t)r * V + v + mo + w] = s;
                 if (LOW) {
-                    const float l = (float)(s - (double)(float)s);
                     g_low[v + w] = l;
                     if (mo != 0) g_low[v + mo + w] = l;
                 }
