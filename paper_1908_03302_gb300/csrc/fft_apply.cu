@@ -129,31 +129,36 @@ __global__ void __launch_bounds__(32 * RED_WARPS) jt_reduce_kernel(const int32_t
                 acc[k] = t;
             }
         };
+        const float* lbase = LOW && ns > 0 ? gpart_low + (int64_t)s0 * TILE_VOX + loc : nullptr;
+        float lows[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        auto add_low = [&](const float4& x) {
+            lows[0] += x.x;
+            lows[1] += x.y;
+            lows[2] += x.z;
+            lows[3] += x.w;
+        };
         int q = w;
         for (; q + 3 * RED_WARPS < ns; q += 4 * RED_WARPS) {   // four slots in flight
-            float4 x[4];
+            float4 x[4], y[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                x[k] = __ldcs(reinterpret_cast<const float4*>(base + (int64_t)(q + k * RED_WARPS) * NCOL * TILE_VOX));
+            for (int k = 0; k < 4; ++k) {
+                const int64_t slot = q + k * RED_WARPS;
+                x[k] = __ldcs(reinterpret_cast<const float4*>(base + slot * NCOL * TILE_VOX));
+                if (LOW) y[k] = __ldcs(reinterpret_cast<const float4*>(lbase + slot * TILE_VOX));
+            }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) add(x[k]);
-        }
-        for (; q < ns; q += RED_WARPS)
-            add(__ldcs(reinterpret_cast<const float4*>(base + (int64_t)q * NCOL * TILE_VOX)));
-        if (LOW && ns > 0) {   // low[k]: so far what acc lacks, with the opposite sign
-            const float* lbase = gpart_low + (int64_t)s0 * TILE_VOX + loc;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) low[k] = -low[k];
-            for (q = w; q < ns; q += RED_WARPS) {
-                const float4 x = __ldcs(reinterpret_cast<const float4*>(lbase + (int64_t)q * TILE_VOX));
-                low[0] += x.x;
-                low[1] += x.y;
-                low[2] += x.z;
-                low[3] += x.w;
+            for (int k = 0; k < 4; ++k) {
+                add(x[k]);
+                if (LOW) add_low(y[k]);
             }
         }
+        for (; q < ns; q += RED_WARPS) {
+            add(__ldcs(reinterpret_cast<const float4*>(base + (int64_t)q * NCOL * TILE_VOX)));
+            if (LOW) add_low(__ldcs(reinterpret_cast<const float4*>(lbase + (int64_t)q * TILE_VOX)));
+        }
         sh[w][lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        if (LOW) sh_low[w][lane] = make_float4(low[0], low[1], low[2], low[3]);
+        if (LOW)   // (low is what acc has too much)
+            sh_low[w][lane] = make_float4(lows[0] - low[0], lows[1] - low[1], lows[2] - low[2], lows[3] - low[3]);
         __syncthreads();
         if (w < 4) {   // warp w: component w of the 32 runs
             float s = 0.0f, l = 0.0f;   // the sum and what it lacks
@@ -430,8 +435,8 @@ static fft_status launch_jt_reduce(fft_geom g, const float* gpart, int ncol, flo
                                    const float* gpart_low = nullptr, float* g_low = nullptr) {
     if (g->n_tiles == 0) return FFT_OK;
     jt_reduce_kernel<NCOL, LOW><<<(unsigned)(g->n_tiles * (TILE_VOX / 128)), 32 * RED_WARPS, 0, st>>>(
-        g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->z_lo, g->z_end, g->mirror, g->tiles[0],
-        g->tiles[1], ncol, gout, gpart_low, g_low);
+        g->tile_slot0, g->tile_nslot, gpart, g->grid.nx, g->grid.ny, g->grid.nz, g->z_lo, g->z_end, g->mirror,
+        g->tiles[0], g->tiles[1], ncol, gout, gpart_low, g_low);
     FFT_CUDA(cudaGetLastError());
     return FFT_OK;
 }
