@@ -13,8 +13,9 @@ paper's lab dataset is not available).
 One step = one damped least-squares solve (fft_cg_solve) on resident data: (n_iter + 1)
 applications each of J and J^T, every entry rebuilt on the fly. The Phi tables and the culled
 geometry are built once before timing (their build time is reported as ``setup_ms``). The
-metric is in-support pair-voxel evaluations per second (J and J^T together); the roofline is
-that of the J^T kernel against the FP32 issue rate of the chip.
+metric is in-support pair-voxel evaluations per second (J and J^T together), counted as served: one
+evaluation may serve a mirrored layer or several slices. The roofline is that of the J^T kernel
+against the FP32 issue rate of the chip at one evaluation per pair.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|reference]
 Under torchrun each rank runs its own replica (the path has no exchange step on one
@@ -50,11 +51,7 @@ FP32_LANES_PER_SM_CLK = 128
 # DRAM bytes (read + write) of one J^T (the apply kernel and its slot reduction, as timed) per
 # workload, from ncu captures of the current kernels (dram__bytes_read.sum +
 # dram__bytes_write.sum); a workload without a capture of the current build reports null.
-APPLY_TRAFFIC_BYTES = {
-    # plain-band apply 3910192640 + 149975552, sharp-band apply 5340387840 + 374120960,
-    # jt_reduce 342418176 + 6821632
-    "slices3d": 10123916800,
-}
+APPLY_TRAFFIC_BYTES = {}
 
 
 def peaks():
@@ -558,7 +555,8 @@ def main():
     stream = torch.cuda.current_stream()
     n_iter = w.cg_iters
     evals_per_step = 2 * (n_iter + 1) * support
-    launches_per_step = 8 + 10 * n_iter
+    # a solve: 4 vector kernels and 6 per iteration beside (n_iter + 1) J and J^T
+    launches_per_step = 4 + 6 * n_iter + 2 * (n_iter + 1) * geo.route()["launches"]
 
     def step(mbuf):
         mbuf.zero_()
@@ -732,6 +730,8 @@ def main():
                      "frac": achieved / peak_evals,
                      "traffic": APPLY_TRAFFIC_BYTES.get(w.name) if (args.dt_mode == 0 and n_terms == 0) else None,
                      "kernel": "apply_kernel (J^T) + jt_reduce",
+                     "served": "in-support pairs per second; one evaluation serves a layer and its mirror image, or up "
+                               "to eight slices of a stack, so that frac can pass 1",
                      "peak_basis": f"{sm_count} SMs x {FP32_LANES_PER_SM_CLK} FP32 lanes x {sm_max:.0f} MHz "
                                    f"({pk_kind}) / {ops} ops per eval"},
         "err_vs_fp64_oracle": err,

@@ -155,7 +155,8 @@ typedef struct {
                                 of one J or J^T (counted on the device at creation) */
     int64_t scratch_bytes;   /* device bytes owned by the handle */
     int32_t dt_mode;
-    int64_t evaluated_evals; /* (row, voxel) evaluations one apply performs after culling */
+    int64_t evaluated_evals; /* (row, voxel) pairs one apply covers after culling (an evaluation may
+                                serve several: a mirrored layer, the slices of a stack) */
     int32_t phi_terms;       /* 0: sampled tables; else the largest sine-series length */
     double psf_tc_mma_flops; /* tensor-core MMA flops of the last fft_psf_batch call in mode 1:
                                 2 x 128 x 96 x N per chunk of generated J tile, N the MMA width */
@@ -175,6 +176,7 @@ typedef struct {
     int32_t batch_cols;    /* columns of the batch scratch: 0 (no batch yet), 4 or 8 */
     int32_t segments;      /* sine series: quadratic segments per band; 0: tables, or the recurrence */
     int32_t solver_comp;   /* 1: solves use compensated products */
+    int32_t launches;      /* kernels that one J or one J^T of one column launches */
 } fft_route_t;
 fft_status fft_geom_route(fft_geom g, fft_route_t* route);
 
@@ -223,8 +225,8 @@ fft_status fft_JT_apply(fft_geom g, const float* d_dev, float* g_dev, void* stre
 
 /*
  * fft_J_apply_batch / fft_JT_apply_batch - J or J^T applied to n vectors at once (the
- * operator of Eq. forward_compact and its adjoint, for block methods such as the low-rank
- * eigensolver): every evaluated entry J[p, v] is used for up to eight columns, so a group of
+ * operator of Eq. forward_compact and its adjoint, for block methods; the low-rank eigensolver
+ * below takes four columns at a time): every evaluated entry J[p, v] is used for up to eight columns, so a group of
  * eight costs about one and a half applications, a group of four one and a quarter.
  *   m_dev  device float32, n columns of length V (column c at m_dev + c * V);
  *   d_dev  device float32, n columns of length M (column c at d_dev + c * M);
@@ -322,8 +324,9 @@ fft_status fft_frob2(fft_geom g, double* out);
  * Vectors are FP32, but up to 2^19 evaluated entries the products J p and J^T r come with
  * compensated sums as two floats each (CGLS amplifies their rounding); inner products, alpha,
  * beta and gamma are FP64 on the device (no host round trip). The iteration loop is captured
- * once per handle into a CUDA graph and replayed. A vanishing gradient (|J^T r - lambda m|^2 = 0) means m already minimises the
- * misfit: the remaining iterations keep it, and that is not a breakdown.
+ * once per handle into a CUDA graph and replayed. A vanishing gradient (|J^T r - lambda m|^2 = 0)
+ * means m already minimises the misfit: the remaining iterations keep it, and that is not a
+ * breakdown.
  * Asynchronous on `stream` when hist_host is NULL: the call returns once the solve is
  * enqueued, and fft_cg_status gives its outcome. With hist_host the call synchronises and
  * returns that outcome itself. The first solve on a handle also computes |J|_F^2

@@ -65,8 +65,8 @@ class fft_geom_info_t(ctypes.Structure):
 
 
 class fft_route_t(ctypes.Structure):
-    _fields_ = [(n, ctypes.c_int32) for n in ("mirror", "stack_classes", "stack_batch", "stack_psf", "batch_cols", "segments",
-                                              "solver_comp")]
+    _fields_ = [(n, ctypes.c_int32) for n in ("mirror", "stack_classes", "stack_batch", "stack_psf", "batch_cols",
+                                              "segments", "solver_comp", "launches")]
 
 
 # (name, restype, argtypes) for every function declared in include/fft_gb300.h

@@ -661,7 +661,9 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     if (fabsf(fmaf(cx, ex, fmaf(cy, ey, cz * ez))) + pext <= hl) inb |= 1u << s;
                     if (fmaf(cx, cx, fmaf(cy, cy, cz * cz)) <= rim2) dpb |= 1u << s;
                 }
-                const uint32_t od = okb & dpb & ~full, both = ((od & 3u) == 3u ? 1u : 0u) | ((od & 12u) == 12u ? 2u : 0u);
+                const uint32_t od = okb & dpb & ~full;
+                const uint32_t both = ((od & 3u) == 3u ? 1u : 0u) | ((od & 12u) == 12u ? 2u : 0u);
+                const uint32_t fl = (okb << 12) | (inb << 16) | (dpb << 20) | (both << 24) | (full << 28);
                 stg[lane * SR + 0] = base;
                 stg[lane * SR + 1] = make_float4(r.c.x, r.c.y, r.c.z, base3);
                 // planar pair (both transducers at one z): stepping along x changes only c3
@@ -672,8 +674,7 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                     PHI == PHI_TRIG ? __uint_as_float(tab_addr + (uint32_t)(b * P.n_tab) * 8u)
                                     : fmaf((float)(b * (PHI == PHI_SEG ? P.seg_n + SEG_PAD : P.n_tab)), MAGIC2_ULP, MAGIC2);
                 stg[lane * SR + 2] = make_float4(W, row_m, DT == FFT_DT_FP64 ? __int_as_float(p) : lam,
-                                                 __int_as_float(b | (bc.sharp << 8) | (planar << 9) |
-                                                                (int)((okb << 12) | (inb << 16) | (dpb << 20) | (both << 24) | (full << 28))));
+                                                 __int_as_float(b | (bc.sharp << 8) | (planar << 9) | (int)fl));
                 if (MODE == MODE_JTC) stg[lane * SR + 3].x = Wlow;
                 if (JTN) {
 #pragma unroll
@@ -842,7 +843,8 @@ __global__ void __launch_bounds__(apply_block_bound<MODE, DT, SHARP, PHI>(),
                                 w[1] = pk(ww[2], ww[3]);
                             } else if (DT == FFT_DT_STABLE && form_of(cw, s) == FORM_DEEP) {
                                 f2 v1[1][2], w1[1][2];
-                                const float a[1] = {psv[q]}, b[1] = {prv[q]}, c[1] = {c2v[q]}, d[1] = {c3v[q]}, f[1] = {c12v[q]};
+                                const float a[1] = {psv[q]}, b[1] = {prv[q]}, c[1] = {c2v[q]}, d[1] = {c3v[q]},
+                                            f[1] = {c12v[q]};
                                 eval_deep<1, SH, PL>(a, b, c, d, f, hy, hz, dr, v1, w1, near);
                                 v[0] = v1[0][0];
                                 v[1] = v1[0][1];
@@ -1137,7 +1139,8 @@ inline void launch_split(fft_geom g, const ApplyParams& P, cudaStream_t st) {
         Q.items = P.items + np;
         Q.n_items = ns;
         Q.counter = P.counter + 1;
-        if (Q.dsum) Q.dsum = P.dsum + (size_t)np * apply_regions<MODE>();   // per-unit partials follow the plain launch's
+        // (per-unit partials follow the plain launch's)
+        if (Q.dsum) Q.dsum = P.dsum + (size_t)np * apply_regions<MODE>();
         launch_apply<MODE, DT, G, true, PHI>(g, Q, st);
     }
 }

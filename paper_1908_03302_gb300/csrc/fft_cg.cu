@@ -3,11 +3,11 @@
 // (J^T J + lambda I) m = J^T d are solved iteratively with J and J^T applied on the fly.
 //
 // Vectors are FP32 (the products of small operators two floats each, see solver_J); every
-// inner product is accumulated in FP64 by a fixed grid of blocks followed by a fixed-order final sum, and alpha, beta, gamma live in FP64 device memory,
-// so the loop needs no host round trip and is bit-reproducible. The loop is captured once
-// into a CUDA graph (per iteration count) on a private stream and replayed on the caller's
-// stream; it touches only the handle's own buffers, so the graph is independent of the
-// caller's pointers.
+// inner product is accumulated in FP64 by a fixed grid of blocks followed by a fixed-order
+// final sum, and alpha, beta, gamma live in FP64 device memory, so the loop needs no host
+// round trip and is bit-reproducible. The loop is captured once into a CUDA graph (per
+// iteration count) on a private stream and replayed on the caller's stream; it touches only
+// the handle's own buffers, so the graph is independent of the caller's pointers.
 //
 // The state between iterations is (m, p, r, gamma, lambda) plus the breakdown flag:
 // fft_cg_continue runs more iterations from it, and fft_cg_save / fft_cg_load copy it to and
@@ -231,8 +231,8 @@ fft_status ensure_workspace(fft_geom g, int32_t n_iter) {
 // the operator's own entries account for 1.2e-6. With compensated sums, and q and s kept to 48 bits, only the
 // rounding of the state (m, p, r: FP32, as a saved state holds them) is left. Over 24 data sets, geometric
 // mean and worst: 2.4e-6 and 6.8e-6 without, 1.6e-6 and 3.3e-6 with them (entries alone: 1.2e-6 and 1.4e-6).
-// It costs 6 to 24 % of a solve (20 iterations: 32-element ring 1.74 -> 1.88 ms, four slices of 32
-// elements with three bands 5.32 -> 6.10 ms, of 56 elements 16.2 -> 19.5 ms). The line at 2^19 evaluated entries is
+// It costs 6 to 24 % of a solve (20 iterations: 32-element ring 1.74 -> 1.84 ms, four slices of 32
+// elements with three bands 5.32 -> 6.05 ms, of 56 elements 16.2 -> 19.4 ms). The line at 2^19 evaluated entries is
 // the largest size at which the distance was measured against a 64-bit solve; beyond it the products are
 // bound by evaluations and would pay the whole price (ring256: J 1.93 -> 2.34 ms).
 fft_status solver_J(fft_geom g, const float* x, cudaStream_t st) {

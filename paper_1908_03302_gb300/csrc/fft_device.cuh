@@ -162,7 +162,8 @@ __device__ __forceinline__ bool box_inside(float dx, float dy, float dz, float e
         const float x = dx + ((c & 1) ? hx : -hx), y = dy + ((c & 2) ? hy : -hy), z = dz + ((c & 4) ? hz : -hz);
         const float sx = fmaf(hl, ex, x), sy = fmaf(hl, ey, y), sz = fmaf(hl, ez, z);
         const float rx = fmaf(-hl, ex, x), ry = fmaf(-hl, ey, y), rz = fmaf(-hl, ez, z);
-        const float ss = fmaxf(fmaf(sx, sx, fmaf(sy, sy, sz * sz)), 1e-12f), rr = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-12f);
+        const float ss = fmaxf(fmaf(sx, sx, fmaf(sy, sy, sz * sz)), 1e-12f);
+        const float rr = fmaxf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)), 1e-12f);
         m = fmaxf(m, fmaf(ss, rsqrt_approx(ss), rr * rsqrt_approx(rr)));
     }
     return m - 2.0f * hl < 1.0f - 1e-3f;
@@ -391,8 +392,8 @@ __device__ __forceinline__ void phi_trig_n(const float* v, uint32_t tb, int nq, 
 // holds Phi = c0 + u (c1 + u c2), u = 2^-22 (v n - k), through the series' values at the segment's
 // ends and middle (seg_n is chosen so that they stay within 5e-8 of max |Phi|). c0 and c1 are one
 // 64-bit load, c2 a 32-bit one: about 5 + 3.2 shared-memory wavefronts, against 56 FP32 operations
-// of the 20-term recurrence (ring256 J^T 15.81 -> 4.54 ms, error against 64 bits 5.9e-7 -> 3.8e-7). t = v n 2^-22 + magic, magic = 2 + (first segment of the band)
-// 2^-22, rounded down has the bits 0x40000000 + segment, whose shifts by 3 and 2 are the byte
+// of the 20-term recurrence (ring256 J^T 15.81 -> 4.54 ms, error against 64 bits 5.9e-7 -> 3.8e-7).
+// t = v n 2^-22 + magic, magic = 2 + (first segment of the band) 2^-22, rounded down has the bits 0x40000000 + segment, whose shifts by 3 and 2 are the byte
 // offsets; t - magic = k 2^-22 exactly. The entries past the segments are zeros: the cut-off.
 __device__ __forceinline__ float phi_seg(float v, float magic, float scale, uint32_t base01, uint32_t base2) {
     const float t = __fmaf_rd(v, scale, magic);

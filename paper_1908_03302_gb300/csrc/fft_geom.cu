@@ -1028,6 +1028,20 @@ extern "C" void fft_geom_destroy(fft_geom g) {
     if (cur != dev) cudaSetDevice(cur);
 }
 
+// Kernels of one J or J^T of one column: an item kernel per kind of rows and a reduction, per pass of a class of
+// a stack two more.
+static int product_launches(fft_geom g) {
+    int n = 0;
+    for (const StackClass& c : g->stk)
+        for (int64_t left = (int64_t)c.off.size(); left > 0;) {
+            n += product_launches(c.sub) + 2;
+            left -= pass_columns(c.sub, left);
+        }
+    if (!g->stk.empty()) return n;
+    const bool split = g->sharp && g->dt_mode != FFT_DT_FP64;
+    return 1 + (split ? (g->n_items_plain > 0 ? 1 : 0) + (g->n_items > g->n_items_plain ? 1 : 0) : 1);
+}
+
 extern "C" fft_status fft_geom_route(fft_geom g, fft_route_t* route) {
     FFT_ARG(g && route, "fft_geom_route: null argument");
     route->mirror = g->mirror;
@@ -1037,6 +1051,7 @@ extern "C" fft_status fft_geom_route(fft_geom g, fft_route_t* route) {
     route->batch_cols = g->batch_cols;
     route->segments = g->seg_n;
     route->solver_comp = has_compensated(g) ? 1 : 0;
+    route->launches = product_launches(g);
     return FFT_OK;
 }
 

@@ -151,7 +151,8 @@ bool find_stack(const double* tx, const int32_t* rows, int64_t M, const int32_t*
         for (size_t i = 0; i < a.size(); ++i) {
             if (band && band[a[i]] != band[b[i]]) return false;
             for (int e = 0; e < 2; ++e) {
-                const double *u = tx + 3 * (int64_t)rows[2 * (int64_t)a[i] + e], *v = tx + 3 * (int64_t)rows[2 * (int64_t)b[i] + e];
+                const double* u = tx + 3 * (int64_t)rows[2 * (int64_t)a[i] + e];
+                const double* v = tx + 3 * (int64_t)rows[2 * (int64_t)b[i] + e];
                 if (u[0] != v[0] || u[1] != v[1]) return false;
             }
         }
@@ -189,7 +190,8 @@ double stack_cost(const std::vector<StackPlan>& plan, int64_t M, const fft_grid&
     for (const StackPlan& c : plan) {
         const double k = 2.0 * (c.z - gr.origin[2]) / gr.h;
         const bool mirrors = fabs(k - nearbyint(k)) <= 1e-9;
-        cost += pass_cost((int64_t)c.rows.size(), true) * (double)c.rows[0].size() / (double)M * (mirrors ? 0.5 : 1.0) * (7.0 / 6.0);
+        const double share = (double)c.rows[0].size() / (double)M;
+        cost += pass_cost((int64_t)c.rows.size(), true) * share * (mirrors ? 0.5 : 1.0) * (7.0 / 6.0);
     }
     return cost;
 }
@@ -197,7 +199,8 @@ double stack_cost(const std::vector<StackPlan>& plan, int64_t M, const fft_grid&
 // One J or J^T of n columns in entries evaluated (the measure that decides between the two ways).
 double stack_entries(fft_geom g, int64_t n) {
     double c = 0.0;
-    for (const StackClass& k : g->stk) c += pass_cost(n * (int64_t)k.off.size(), k.sub->batch_cols == 8) * (double)k.sub->E_used;
+    for (const StackClass& k : g->stk)
+        c += pass_cost(n * (int64_t)k.off.size(), k.sub->batch_cols == 8) * (double)k.sub->E_used;
     return c;
 }
 
@@ -205,7 +208,8 @@ fft_status stack_J(fft_geom g, const float* m, int n, float* d, cudaStream_t st)
     if (g->unusable) return check_usable(g);
     const int64_t plane = (int64_t)g->grid.nx * g->grid.ny;
     return for_each_pass(g, n, [&](fft_geom sub, const StackJobs& J) -> fft_status {
-        stack_models_kernel<<<dim3((unsigned)ceil_div(sub->V, 256), J.n), 256, 0, st>>>(J, m, g->V, plane, sub->V, g->stk_x);
+        stack_models_kernel<<<dim3((unsigned)ceil_div(sub->V, 256), J.n), 256, 0, st>>>(J, m, g->V, plane, sub->V,
+                                                                                         g->stk_x);
         FFT_CUDA(cudaGetLastError());
         const fft_status rc = launch_J_batch(sub, g->stk_x, J.n, g->stk_d, st);
         if (rc != FFT_OK) return rc;

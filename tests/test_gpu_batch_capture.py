@@ -35,7 +35,8 @@ def test_replay_after_a_wider_call(name):
     wide = {n: (geo.J_batch(cut[n][0]).clone(), geo.JT_batch(cut[n][1]).clone()) for n in cols}
     assert geo.info().scratch_bytes > small   # the wider one came beside it
     torch.cuda.synchronize()
-    taken = [torch.full((1 << 22,), float("nan"), device="cuda") for _ in range(16)]   # what was freed would be used again
+    # (what was freed would be used again)
+    taken = [torch.full((1 << 22,), float("nan"), device="cuda") for _ in range(16)]
     for n in cols:
         for _ in range(2):
             out[n][0].zero_(), out[n][1].zero_()

@@ -81,7 +81,7 @@ def test_batch_width_grows_once(fg):
     geo, _ = gpu_geometry(wl.slices32())
     rng = np.random.default_rng(4)
     X, D = to_dev(rng.normal(size=(9, geo.V))), to_dev(1e-8 * rng.normal(size=(9, geo.M)))
-    assert geo.route()["batch_cols"] == 0 and geo.route()["solver_comp"] == 1
+    assert geo.route()["batch_cols"] == 0 and geo.route()["solver_comp"] == 1 and geo.route()["launches"] == 3
     geo.J_batch(X[:4].contiguous())
     assert geo.route()["batch_cols"] == 4
     want = [(geo.J_batch(X[:n].contiguous()).clone(), geo.JT_batch(D[:n].contiguous()).clone()) for n in (5, 8, 9)]
@@ -102,4 +102,4 @@ def test_batch_width_grows_once(fg):
 def test_large_solves_keep_plain_products(fg):
     geo, _ = gpu_geometry(wl.ring256())
     assert geo.route() == {"mirror": wl.ring256().grid.nz - 1, "stack_classes": 0, "stack_batch": 0, "stack_psf": 0, "batch_cols": 0,
-                           "segments": 0, "solver_comp": 0}
+                           "segments": 0, "solver_comp": 0, "launches": 2}

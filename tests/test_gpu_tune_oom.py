@@ -22,7 +22,8 @@ def operator(fg, stack):
 
 
 @pytest.mark.parametrize("stack", [False, True])
-@pytest.mark.parametrize("after", [0, 1, 3, 4, 6, 8, 9])   # (parent: four allocations a candidate; a class's operator: three; their J^T partials)
+# (four allocations a candidate; with a stack three for a class's operator, and the J^T partials' if they grow)
+@pytest.mark.parametrize("after", [0, 1, 3, 4, 6, 8, 9])
 def test_one_allocation_fails(stack, after):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
