@@ -212,7 +212,9 @@ fft_status fft_geom_autotune(fft_geom g, void* stream, fft_tune_info_t* info);
 /*
  * fft_J_apply - d = J m (Eq. forward_compact; m in m/s, d in s).
  *   m_dev  device float32[V]; d_dev device float32[M] (written entirely). No aliasing.
- * Each row's value is a fixed-order sum (deterministic, bit-reproducible run to run).
+ * Each row's value is a fixed-order sum (deterministic, bit-reproducible run to run on a handle;
+ * two handles of one geometry agree if both had the memory for the evaluation that elevation
+ * stacks share, see fft_geom_route).
  */
 fft_status fft_J_apply(fft_geom g, const float* m_dev, float* d_dev, void* stream);
 
