@@ -153,7 +153,7 @@ extern "C" fft_status fft_psf_noalloc(fft_geom g, int64_t spike_vox, const int32
                 D, err);
         FFT_CUDA(cudaGetLastError());
     }
-    if ((rc = launch_JT(g, D, out_dev, st)) != FFT_OK) return rc;
+    if ((rc = launch_JT(g, D, out_dev, st, true)) != FFT_OK) return rc;
     unsigned int bad = 0;
     FFT_CUDA(cudaMemcpyAsync(&bad, err, sizeof(bad), cudaMemcpyDeviceToHost, st));
     FFT_CUDA(cudaStreamSynchronize(st));

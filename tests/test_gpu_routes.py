@@ -75,6 +75,8 @@ def test_sparse_columns_of_stacks(fg, n_tx, n, step, grid, classes, psf):
     for mode in (0, 2):
         a, b = (g.psf_batch(spikes, subs, mode=mode).double() for g in (geo, gen))
         assert float((a - b).norm() / b.norm()) <= 2e-6
+    one = geo.psf_noalloc(middle, torch.arange(geo.M, device="cuda", dtype=torch.int32)).double()
+    assert float((one - b[0, 0]).norm() / b[0, 0].norm()) <= 2e-6
 
 
 def test_batch_width_grows_once(fg):
